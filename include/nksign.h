@@ -252,8 +252,9 @@ int nk_set_adapt_start(nk_ctx* ctx, int k_first);
 /*
  * Launch shape of the outer recurrence (batching of the RHS and the
  * autotuner; a property of the implementation, not of the method).
- *  stencil_threads  lattice sites per CTA of the fused stencil kernel, one
- *                   thread per site and vector: 64, 128 or 256;
+ *  stencil_threads  threads per CTA of the fused FP64 stencil kernel, 16 per
+ *                   site (one per hop and half-spinor column): 64, 128 or 256,
+ *                   that is 4, 8 or 16 sites;
  *  stencil_order    0: consecutive CTAs take all vectors (RHS and, for mu != 0,
  *                   both sides) of one block of sites, so the links of those
  *                   sites are read from HBM once and then from L2;
@@ -261,12 +262,13 @@ int nk_set_adapt_start(nk_ctx* ctx, int k_first);
  *  step2_blocks     CTAs per RHS of the step-2 and norm kernels (grid-stride),
  *                   1..4096; also the number of partial sums of their
  *                   deterministic reductions;
- *  stencil_split    threads per site of the fused stencil: 1, or 3 (one per
- *                   colour: each projects the neighbour spinors and forms one
- *                   colour row, with a third of the accumulators);
+ *  stencil_split    1, or 3 (three times the threads, one colour row of each
+ *                   hop's product per thread);
  *  early_threads, early_order, early_split
- *                   the stencil shape of the two-float steps before j0 in
- *                   NK_MIXED mode (unused in NK_FP64 mode).
+ *                   the stencil shape of the two-float steps of the optional
+ *                   two-float recurrence (nk_set_df_recurrence): sites per CTA,
+ *                   one thread (early_split = 3: one per colour) per site and
+ *                   vector.  The multi-RHS stencils of NK_MIXED have one shape.
  * A shape belongs to (n_rhs, sidedness of the current mu (mu != 0), the
  * NK_MIXED bit of flags).  Different shapes sum in different orders, so
  * results differ at rounding level; one shape is bitwise reproducible.

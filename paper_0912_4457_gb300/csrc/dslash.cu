@@ -17,116 +17,10 @@
 // Layouts (device-internal, set up by the engine):
 //   links:   [nu 4][e 9][site V] complex, e = 3*row + col (coalesced over sites)
 //   spinors: [component 12][site V] complex per vector, component = 3*spin + colour
-#include <type_traits>
-
 #include "nk_common.cuh"
-#include "nk_hop.cuh"
 #include "nk_kernels.h"
 
 namespace nk {
-
-template <typename R>
-struct Spinor {
-    typename C2<R>::T c[4][3];
-};
-
-template <typename R>
-__device__ __forceinline__ void load_spinor(const typename C2<R>::T* __restrict__ in, int V, int site,
-                                            typename C2<R>::T p[4][3]) {
-#pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) p[s][a] = in[(size_t)(3 * s + a) * V + site];
-}
-
-template <typename R>
-__device__ __forceinline__ void load_link(const typename C2<R>::T* __restrict__ U, int V, int nu, int site,
-                                          typename C2<R>::T u[3][3]) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) u[a][b] = U[(size_t)(nu * 9 + 3 * a + b) * V + site];
-}
-
-template <int NU, typename R>
-__device__ __forceinline__ void dir(typename C2<R>::T acc[4][3], const typename C2<R>::T* __restrict__ U,
-                                    const typename C2<R>::T* __restrict__ in, const Geom& g, int site,
-                                    int coord, int L, int stride, R wplus, R wminus) {
-    // backward neighbour y - nu: (1 + gamma) U_{y-nu,+nu} psi_{y-nu}
-    typedef typename C2<R>::T T;
-    const int sb = coord == 0 ? site + (L - 1) * stride : site - stride;
-    const R fb = (NU == 3 && g.antiperiodic && coord == 0) ? R(-1) : R(1);
-    const int sf = coord == L - 1 ? site - (L - 1) * stride : site + stride;
-    const R ff = (NU == 3 && g.antiperiodic && coord == L - 1) ? R(-1) : R(1);
-    T u[3][3], p[4][3];
-    load_link<R>(U, g.V, NU, sb, u);
-    load_spinor<R>(in, g.V, sb, p);
-    hop_regs<NU, false, R>(acc, p, u, R(1), wplus * fb);
-    // forward neighbour y + nu: (1 - gamma) U^dagger_{y,+nu} psi_{y+nu}
-    load_link<R>(U, g.V, NU, site, u);
-    load_spinor<R>(in, g.V, sf, p);
-    hop_regs<NU, true, R>(acc, p, u, R(-1), wminus * ff);
-}
-
-// ---- colour split: one thread per (site, colour a) -----------------------------
-// The same hop restricted to row a of M psi: the thread projects the whole
-// neighbour spinor (all three colours) but forms and accumulates only the a-th
-// row, so it holds a quarter of the accumulators; three threads share a site.
-template <int NU, bool DAG, typename R>
-__device__ __forceinline__ void hop_regs_a(typename C2<R>::T acc[4], const typename C2<R>::T psi[4][3],
-                                           const typename C2<R>::T urow[3], R s, R w) {
-    typedef typename C2<R>::T T;
-    T h0[3], h1[3];
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        T c0, c1;
-        if (NU == 0) { c0 = mul_mi(psi[3][b]); c1 = mul_mi(psi[2][b]); }
-        else if (NU == 1) { c0 = neg(psi[3][b]); c1 = psi[2][b]; }
-        else if (NU == 2) { c0 = mul_mi(psi[2][b]); c1 = mul_i(psi[3][b]); }
-        else { c0 = psi[2][b]; c1 = psi[3][b]; }
-        h0[b].x = psi[0][b].x + s * c0.x; h0[b].y = psi[0][b].y + s * c0.y;
-        h1[b].x = psi[1][b].x + s * c1.x; h1[b].y = psi[1][b].y + s * c1.y;
-    }
-    const R ws = w * s;
-    T x0, x1;
-    x0.x = 0; x0.y = 0; x1.x = 0; x1.y = 0;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        const T e = urow[b];
-        R ey = DAG ? -e.y : e.y;
-        x0.x += e.x * h0[b].x - ey * h0[b].y; x0.y += e.x * h0[b].y + ey * h0[b].x;
-        x1.x += e.x * h1[b].x - ey * h1[b].y; x1.y += e.x * h1[b].y + ey * h1[b].x;
-    }
-    acc[0].x += w * x0.x; acc[0].y += w * x0.y;
-    acc[1].x += w * x1.x; acc[1].y += w * x1.y;
-    T b0, b1;
-    if (NU == 0) { b0 = mul_i(x1); b1 = mul_i(x0); }
-    else if (NU == 1) { b0 = x1; b1 = neg(x0); }
-    else if (NU == 2) { b0 = mul_i(x0); b1 = mul_mi(x1); }
-    else { b0 = x0; b1 = x1; }
-    acc[2].x += ws * b0.x; acc[2].y += ws * b0.y;
-    acc[3].x += ws * b1.x; acc[3].y += ws * b1.y;
-}
-
-template <int NU, typename R>
-__device__ __forceinline__ void dir_a(typename C2<R>::T acc[4], const typename C2<R>::T* __restrict__ U,
-                                      const typename C2<R>::T* __restrict__ in, const Geom& g, int site, int a,
-                                      int coord, int L, int stride, R wplus, R wminus) {
-    typedef typename C2<R>::T T;
-    const int sb = coord == 0 ? site + (L - 1) * stride : site - stride;
-    const R fb = (NU == 3 && g.antiperiodic && coord == 0) ? R(-1) : R(1);
-    const int sf = coord == L - 1 ? site - (L - 1) * stride : site + stride;
-    const R ff = (NU == 3 && g.antiperiodic && coord == L - 1) ? R(-1) : R(1);
-    T urow[3], p[4][3];
-#pragma unroll
-    for (int b = 0; b < 3; ++b) urow[b] = U[(size_t)(NU * 9 + 3 * a + b) * g.V + sb];   // row a of U
-    load_spinor<R>(in, g.V, sb, p);
-    hop_regs_a<NU, false, R>(acc, p, urow, R(1), wplus * fb);
-#pragma unroll
-    for (int b = 0; b < 3; ++b) urow[b] = U[(size_t)(NU * 9 + 3 * b + a) * g.V + site]; // column a: row a of U^dagger
-    load_spinor<R>(in, g.V, sf, p);
-    hop_regs_a<NU, true, R>(acc, p, urow, R(-1), wminus * ff);
-}
 
 // ---- the two-float stencil: one copy of the hop body --------------------------
 // Two-float arithmetic turns every flop into 7-11 FP32 instructions; the
@@ -306,22 +200,6 @@ __device__ __forceinline__ void stencil_hops_df_a(dfc acc[4], const dfc* __restr
     for (int sp = 0; sp < 4; ++sp) acc[sp] = dfc_value(A[sp]);
 }
 
-// precision-generic conversions (float via the integer pipe, see nk_common.cuh)
-__device__ __forceinline__ double to_double(float a) { return f2d_int(a); }
-__device__ __forceinline__ double to_double(double a) { return a; }
-__device__ __forceinline__ double to_double(df a) { return df_to_double(a); }
-template <typename R> __device__ __forceinline__ R from_double(double d);
-template <> __device__ __forceinline__ float from_double<float>(double d) { return d2f_int(d); }
-template <> __device__ __forceinline__ double from_double<double>(double d) { return d; }
-template <> __device__ __forceinline__ df from_double<df>(double d) { return df_from_double(d); }
-// two-float complex values for the mixed-schedule epilogue
-__device__ __forceinline__ dfc to_dfc(float2 v) {
-    dfc r;
-    r.x = df(v.x, 0.0f);
-    r.y = df(v.y, 0.0f);
-    return r;
-}
-__device__ __forceinline__ dfc to_dfc(dfc v) { return v; }
 __device__ __forceinline__ dfc dfc_of2(double2 v) {
     dfc r;
     r.x = df_from_double(v.x);
@@ -335,162 +213,77 @@ static df df_host(double d) {
     r.lo = (float)(d - (double)r.hi);
     return r;
 }
-// s - c p and s + c p with explicit FMA (4 FP64 instructions each)
-__device__ __forceinline__ double2 caxpy_neg(double2 s, double2 c, double2 p) {
-    return make_double2(fma(-c.x, p.x, fma(c.y, p.y, s.x)), fma(-c.x, p.y, fma(-c.y, p.x, s.y)));
-}
+// s + c p with explicit FMA (4 FP64 instructions)
 __device__ __forceinline__ double2 caxpy_pos(double2 s, double2 c, double2 p) {
     return make_double2(fma(c.x, p.x, fma(-c.y, p.y, s.x)), fma(c.x, p.y, fma(c.y, p.x, s.y)));
 }
 
 // out = gamma5 (psi - kappa * hops)(site) for one vector: A psi (dag = 0) or
-// A^dagger psi = gamma5 D_w(-mu) psi (dag = 1), in precision R.
-template <typename R>
-__device__ __forceinline__ void stencil_site(const typename C2<R>::T* __restrict__ U,
-                                             const typename C2<R>::T* __restrict__ in, const Geom& g,
-                                             int site, int dag, R kappa, R emu, R emu_inv,
-                                             typename C2<R>::T out[4][3]) {
-    typedef typename C2<R>::T T;
+// A^dagger psi = gamma5 D_w(-mu) psi (dag = 1), in two-float arithmetic.
+__device__ __forceinline__ void stencil_site(const dfc* __restrict__ U, const dfc* __restrict__ in, const Geom& g,
+                                             int site, int dag, df kappa, df emu, df emu_inv, dfc out[4][3]) {
     // temporal weights: A uses (e^{mu}, e^{-mu}); A^dagger exchanges them
-    const R wp_t = dag ? emu_inv : emu;
-    const R wm_t = dag ? emu : emu_inv;
-    int x = site % g.Lx;
+    const df wp_t = dag ? emu_inv : emu;
+    const df wm_t = dag ? emu : emu_inv;
     int r = site / g.Lx;
-    int y = r % g.Ly; r /= g.Ly;
-    int z = r % g.Lz;
-    int t = r / g.Lz;
-    T acc[4][3];
-#pragma unroll
-    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int a = 0; a < 3; ++a) { acc[sp][a].x = 0; acc[sp][a].y = 0; }
-    if constexpr (std::is_same<R, df>::value) {
-        const int coord[4] = {x, y, z, t};
-        stencil_hops_df(acc, U, in, g, site, coord, wp_t, wm_t);
-    } else {
-        dir<0, R>(acc, U, in, g, site, x, g.Lx, 1, R(1), R(1));
-        dir<1, R>(acc, U, in, g, site, y, g.Ly, g.Lx, R(1), R(1));
-        dir<2, R>(acc, U, in, g, site, z, g.Lz, g.Lx * g.Ly, R(1), R(1));
-        dir<3, R>(acc, U, in, g, site, t, g.Lt, g.Lx * g.Ly * g.Lz, wp_t, wm_t);
-    }
-    T p[4][3];
-    load_spinor<R>(in, g.V, site, p);
+    const int x = site % g.Lx, y = r % g.Ly;
+    r /= g.Ly;
+    const int coord[4] = {x, y, r % g.Lz, r / g.Lz};
+    dfc acc[4][3];
+    stencil_hops_df(acc, U, in, g, site, coord, wp_t, wm_t);
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp) {
-        const R sg = sp < 2 ? R(1) : R(-1);  // gamma5 = diag(1, 1, -1, -1)
+        const df sg = sp < 2 ? df(1) : df(-1);  // gamma5 = diag(1, 1, -1, -1)
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            out[sp][a].x = sg * (p[sp][a].x - kappa * acc[sp][a].x);
-            out[sp][a].y = sg * (p[sp][a].y - kappa * acc[sp][a].y);
+            const dfc p = in[(size_t)(3 * sp + a) * g.V + site];
+            out[sp][a].x = sg * (p.x - kappa * acc[sp][a].x);
+            out[sp][a].y = sg * (p.y - kappa * acc[sp][a].y);
         }
     }
 }
 
 // The colour-a components of gamma5 (psi - kappa * hops)(site): out[sp] for colour a.
-template <typename R>
-__device__ __forceinline__ void stencil_site_a(const typename C2<R>::T* __restrict__ U,
-                                               const typename C2<R>::T* __restrict__ in, const Geom& g,
-                                               int site, int a, int dag, R kappa, R emu, R emu_inv,
-                                               typename C2<R>::T out[4]) {
-    typedef typename C2<R>::T T;
-    const R wp_t = dag ? emu_inv : emu;
-    const R wm_t = dag ? emu : emu_inv;
-    int x = site % g.Lx;
+__device__ __forceinline__ void stencil_site_a(const dfc* __restrict__ U, const dfc* __restrict__ in, const Geom& g,
+                                               int site, int a, int dag, df kappa, df emu, df emu_inv, dfc out[4]) {
+    const df wp_t = dag ? emu_inv : emu;
+    const df wm_t = dag ? emu : emu_inv;
     int r = site / g.Lx;
-    int y = r % g.Ly; r /= g.Ly;
-    int z = r % g.Lz;
-    int t = r / g.Lz;
-    T acc[4];
-#pragma unroll
-    for (int sp = 0; sp < 4; ++sp) { acc[sp].x = 0; acc[sp].y = 0; }
-    if constexpr (std::is_same<R, df>::value) {
-        const int coord[4] = {x, y, z, t};
-        stencil_hops_df_a(acc, U, in, g, site, a, coord, wp_t, wm_t);
-    } else {
-        dir_a<0, R>(acc, U, in, g, site, a, x, g.Lx, 1, R(1), R(1));
-        dir_a<1, R>(acc, U, in, g, site, a, y, g.Ly, g.Lx, R(1), R(1));
-        dir_a<2, R>(acc, U, in, g, site, a, z, g.Lz, g.Lx * g.Ly, R(1), R(1));
-        dir_a<3, R>(acc, U, in, g, site, a, t, g.Lt, g.Lx * g.Ly * g.Lz, wp_t, wm_t);
-    }
+    const int x = site % g.Lx, y = r % g.Ly;
+    r /= g.Ly;
+    const int coord[4] = {x, y, r % g.Lz, r / g.Lz};
+    dfc acc[4];
+    stencil_hops_df_a(acc, U, in, g, site, a, coord, wp_t, wm_t);
 #pragma unroll
     for (int sp = 0; sp < 4; ++sp) {
-        const R sg = sp < 2 ? R(1) : R(-1);
-        const T p = in[(size_t)(3 * sp + a) * g.V + site];
+        const df sg = sp < 2 ? df(1) : df(-1);
+        const dfc p = in[(size_t)(3 * sp + a) * g.V + site];
         out[sp].x = sg * (p.x - kappa * acc[sp].x);
         out[sp].y = sg * (p.y - kappa * acc[sp].y);
     }
 }
 
-// One thread per (site, vector). Vectors [0, n0) come from set 0, [n0, n0+n1)
-// from set 1; set s applies A (dag = 0) or A^dagger (dag = 1).
-template <typename R>
-__global__ void __launch_bounds__(128) dslash_kernel(const typename C2<R>::T* __restrict__ U, Geom g,
-                                                      DslashSet s0, DslashSet s1, R kappa, R emu, R emu_inv) {
-    typedef typename C2<R>::T T;
-    const int nvec = s0.n + s1.n;
-    const int vec = blockIdx.x % nvec;
-    const int site = (blockIdx.x / nvec) * blockDim.x + threadIdx.x;
-    if (site >= g.V) return;
-    const DslashSet& S = vec < s0.n ? s0 : s1;
-    const int vi = vec < s0.n ? vec : vec - s0.n;
-    const T* __restrict__ in = reinterpret_cast<const T*>(S.in) + (size_t)vi * S.in_stride;
-    double2* __restrict__ out = S.out + (size_t)vi * S.out_stride;
-    T o[4][3];
-    stencil_site<R>(U, in, g, site, S.dag, kappa, emu, emu_inv, o);
-#pragma unroll
-    for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-            out[(size_t)(3 * sp + a) * g.V + site] = make_double2(to_double(o[sp][a].x), to_double(o[sp][a].y));
-}
-
-void launch_dslash(int precision, const void* U, const Geom& g, const DslashSet& s0,
-                   const DslashSet& s1, double kappa, double mu, cudaStream_t st) {
-    const int threads = 128;
-    const int nvec = s0.n + s1.n;
-    if (nvec == 0) return;
-    dim3 grid((unsigned)(((g.V + threads - 1) / threads) * nvec));
-    if (precision == 48)
-        dslash_kernel<df><<<grid, threads, 0, st>>>((const dfc*)U, g, s0, s1, df_host(kappa), df_host(exp(mu)),
-                                                   df_host(exp(-mu)));
-    else
-        dslash_kernel<double><<<grid, threads, 0, st>>>((const double2*)U, g, s0, s1, kappa, exp(mu), exp(-mu));
-}
-
-// ---- fused stencil + first half of an outer Lanczos step ------------------------
+// ---- two-float stencil fused with step 1 of the two-float recurrence -------------
 //
-// For outer step j (see lanczos.cu for the unnormalised basis q_j, p_j):
+// For outer step j >= o.ring_from of the optional two-float recurrence (see
+// lanczos.cu for the unnormalised basis q_j, p_j; the FP64 recurrence runs
+// through stencil64.cu, or a multi-RHS stencil and k_step1):
 //   right vectors (side 0, one per RHS):
 //     s = A q_j / n_j;  r = s - (c_{j-1}/n_{j-1}) q_{j-1}  (c = beta, two-sided gamma)
 //     r -> q_{j+1};  partial of H(j,j) = v_j^dag r  (two-sided w_j^dag r)
 //   left vectors (side 1, two-sided only):
 //     t = A^dag p_j / m_j;  l = t - (beta^*_{j-1}/m_{j-1}) p_{j-1};  l -> p_{j+1}
-// The stencil runs in precision R (FP32 reads the FP32 copies of q_j, p_j and
-// the FP32 links; the two-float stencil reads the two-float rings); the scale
-// 1/n_j of its output is part of the stencil application (A v_j = A q_j / n_j)
-// and is applied in the same precision.  The rest of the epilogue (the
-// update with q_{j-1}, p_{j-1} and the H(j,j) partial) runs in FP64 on the
-// FP64 vectors, or, from step o.ring_from on (the optional two-float
-// recurrence of the mixed schedule), in two-float arithmetic on the rings.  The blocks of side 0 reduce H(j,j) with the deterministic
-// two-stage scheme.  In double-pass mode side 0 also accumulates
-// y += c'_j q_j at its own site.
-// Minimum resident CTAs of kStencilMaxThreads threads per SM for the fused
-// stencil (a register cap): the FP32 and two-float instantiations are
-// latency bound (loads; long dependent FP32 chains) and gain from more
-// resident warps than their unconstrained register counts (about 160) allow.
-template <typename R> struct StencilMinBlocks { static constexpr int value = 1; };
-template <> struct StencilMinBlocks<df> { static constexpr int value = 2; };
-template <> struct StencilMinBlocks<float> { static constexpr int value = 3; };
-
+// all in two-float arithmetic on the rings.  The blocks of side 0 reduce
+// H(j,j) with the deterministic two-stage scheme.  In double-pass mode side 0
+// also accumulates y += c'_j q_j at its own site.  Two CTAs of
+// kStencilMaxThreads threads per SM (a register cap): the long dependent FP32
+// chains gain from more resident warps than about 160 registers allow.
+//
 // CS: threads per site (1, or 3 with one colour each; blockDim = (sites, CS)).
-template <typename R, bool TS, bool PASS2, int CS>
-__global__ void __launch_bounds__(CS * kStencilMaxThreads, CS == 1 ? StencilMinBlocks<R>::value : 1) k_dslash_step1(
-    const typename C2<R>::T* __restrict__ U, Geom g, Outer o, int j, R kappa, R emu, R emu_inv,
-    const typename C2<R>::T* __restrict__ qin, long qin_stride, const typename C2<R>::T* __restrict__ pin,
-    long pin_stride) {
-    typedef typename C2<R>::T T;
+template <bool TS, bool PASS2, int CS>
+__global__ void __launch_bounds__(CS * kStencilMaxThreads, CS == 1 ? 2 : 1) k_dslash_step1(
+    const dfc* __restrict__ U, Geom g, Outer o, int j, df kappa, df emu, df emu_inv) {
     __shared__ double2 sh[33];
-    __shared__ double2 coef[3];
     const int nvec = TS ? 2 * o.n_rhs : o.n_rhs;
     const int nsb = gridDim.x / nvec;
     const int vec = o.st_order == 0 ? blockIdx.x % nvec : blockIdx.x / nsb;
@@ -500,126 +293,58 @@ __global__ void __launch_bounds__(CS * kStencilMaxThreads, CS == 1 ? StencilMinB
     if (o.status[rhs] != kStatusOK) return;
     if (side == 1 && j == o.k - 1) return;   // the last step needs no left vector
     const size_t hb = (size_t)rhs * o.k;
-    // the scalars of this step (a complex FP64 division or inverse each), one
-    // per warp so that they run side by side instead of one after another
-    if ((block_tid() & 31) == 0) {
-        const int nw = block_threads() >> 5;   // 2 warps or more
-        for (int t = block_tid() >> 5; t < 3; t += nw) {
-            const double2 zero = make_double2(0.0, 0.0);
-            double2 v;
-            if (side == 0) {
-                if (t == 0) v = cinv(scale_n(o, rhs, j));
-                else if (t == 1) v = j > 0 ? cdiv(TS ? o.gamma[hb + j - 1] : o.beta[hb + j - 1], scale_n(o, rhs, j - 1)) : zero;
-                else v = TS ? cinv(cconj(scale_m(o, rhs, j))) : cinv(scale_n(o, rhs, j));
-            } else {
-                if (t == 0) v = cinv(scale_m(o, rhs, j));
-                else if (t == 1) v = j > 0 ? cdiv(cconj(o.beta[hb + j - 1]), scale_m(o, rhs, j - 1)) : zero;
-                else v = zero;
-            }
-            coef[t] = v;
-        }
-    }
-    __syncthreads();
+    const double2* __restrict__ sc = o.sc + (size_t)rhs * kScalars;
     const int site = sb * blockDim.x + threadIdx.x;
     double2 acc = make_double2(0.0, 0.0);
     if (site < g.V) {
-        const T* __restrict__ in = side == 0 ? qin + (size_t)rhs * qin_stride : pin + (size_t)rhs * pin_stride;
-        // the stencil output of this thread's components, handed to epi(sp, a, value)
-        auto for_each_out = [&](auto&& epi) {
-            if constexpr (CS == 1) {
-                T out[4][3];
-                stencil_site<R>(U, in, g, site, side, kappa, emu, emu_inv, out);
-#pragma unroll
-                for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) epi(sp, a, out[sp][a]);
+        const int jp = j > 0 ? j - 1 : j;
+        const dfc* __restrict__ in = side == 0 ? ring_q(o, rhs, j) : ring_p(o, rhs, j);
+        const dfc scr = dfc_of2(sc[side ? kScM : kScN]);      // 1/n_j (1/m_j)
+        const dfc c1d = dfc_of2(sc[side ? kScC1L : kScC1]);   // zero at j = 0 (the previous vector is then any valid one)
+        // one accumulator per spin component: four short dependency chains
+        // of two-float additions instead of one of twelve
+        df ax[4] = {df(0), df(0), df(0), df(0)}, ay[4] = {df(0), df(0), df(0), df(0)};
+        const dfc* __restrict__ prv = side == 0 ? ring_q(o, rhs, jp) : ring_p(o, rhs, jp);
+        dfc* __restrict__ nxt = side == 0 ? ring_q(o, rhs, j + 1) : ring_p(o, rhs, j + 1);
+        const dfc* __restrict__ dotv = TS ? ring_p(o, rhs, j) : ring_q(o, rhs, j);
+        double2* __restrict__ yacc = PASS2 ? o.y + (size_t)rhs * o.N : nullptr;
+        const double2 cpj = PASS2 ? o.cp[hb + j] : make_double2(0.0, 0.0);
+        const double2* __restrict__ qj = outer_q(o, rhs, j);
+        auto epi = [&](int sp, int a, const dfc& v) {
+            const size_t idx = (size_t)(3 * sp + a) * g.V + site;
+            const dfc pv = prv[idx];
+            dfc rr;
+            if (TS || side == 1) {
+                rr.x = (v.x * scr.x - v.y * scr.y) - (c1d.x * pv.x - c1d.y * pv.y);   // s - c1 q_{j-1}
+                rr.y = (v.x * scr.y + v.y * scr.x) - (c1d.x * pv.y + c1d.y * pv.x);
             } else {
-                const int a = threadIdx.y;
-                T out[4];
-                stencil_site_a<R>(U, in, g, site, a, side, kappa, emu, emu_inv, out);
-#pragma unroll
-                for (int sp = 0; sp < 4; ++sp) epi(sp, a, out[sp]);
+                rr.x = v.x * scr.x - c1d.x * pv.x;
+                rr.y = v.y * scr.x - c1d.x * pv.y;
+            }
+            nxt[idx] = rr;
+            if (side == 0) {
+                const dfc d = dotv[idx];
+                ax[sp] += d.x * rr.x + d.y * rr.y;        // conj(d) r
+                if (TS) ay[sp] += d.x * rr.y - d.y * rr.x;
+                if (PASS2) yacc[idx] = caxpy_pos(yacc[idx], cpj, qj[idx]);
             }
         };
-        const double2 c1 = coef[1];   // zero at j = 0 (the previous vector is then any valid one)
-        const int jp = j > 0 ? j - 1 : j;
-        bool ring_epilogue = false;
-        if constexpr (!std::is_same<R, double>::value) ring_epilogue = j >= o.ring_from;
-        if constexpr (!std::is_same<R, double>::value) if (ring_epilogue) {
-            // steps of the mixed schedule from ring_from on (the two-float
-            // recurrence): the epilogue in two-float arithmetic on the rings
-            const dfc scr = dfc_of2(coef[0]), c1d = dfc_of2(c1);
-            // one accumulator per spin component: four short dependency chains
-            // of two-float additions instead of one of twelve
-            df ax[4] = {df(0), df(0), df(0), df(0)}, ay[4] = {df(0), df(0), df(0), df(0)};
-            const dfc* __restrict__ prv = side == 0 ? ring_q(o, rhs, jp) : ring_p(o, rhs, jp);
-            dfc* __restrict__ nxt = side == 0 ? ring_q(o, rhs, j + 1) : ring_p(o, rhs, j + 1);
-            const dfc* __restrict__ dotv = TS ? ring_p(o, rhs, j) : ring_q(o, rhs, j);
-            double2* __restrict__ yacc = PASS2 ? o.y + (size_t)rhs * o.N : nullptr;
-            const double2 cpj = PASS2 ? o.cp[hb + j] : make_double2(0.0, 0.0);
-            const double2* __restrict__ qj = outer_q(o, rhs, j);
-            for_each_out([&](int sp, int a, const T& vout) {
-                const size_t idx = (size_t)(3 * sp + a) * g.V + site;
-                const dfc v = to_dfc(vout);
-                const dfc pv = prv[idx];
-                dfc rr;
-                if (TS || side == 1) {
-                    rr.x = (v.x * scr.x - v.y * scr.y) - (c1d.x * pv.x - c1d.y * pv.y);   // s - c1 q_{j-1}
-                    rr.y = (v.x * scr.y + v.y * scr.x) - (c1d.x * pv.y + c1d.y * pv.x);
-                } else {
-                    rr.x = v.x * scr.x - c1d.x * pv.x;
-                    rr.y = v.y * scr.x - c1d.x * pv.y;
-                }
-                nxt[idx] = rr;
-                if (side == 0) {
-                    const dfc d = dotv[idx];
-                    ax[sp] += d.x * rr.x + d.y * rr.y;        // conj(d) r
-                    if (TS) ay[sp] += d.x * rr.y - d.y * rr.x;
-                    if (PASS2) yacc[idx] = caxpy_pos(yacc[idx], cpj, qj[idx]);
-                }
-            });
-            acc = make_double2(df_to_double((ax[0] + ax[1]) + (ax[2] + ax[3])),
-                               df_to_double((ay[0] + ay[1]) + (ay[2] + ay[3])));
+        if constexpr (CS == 1) {
+            dfc out[4][3];
+            stencil_site(U, in, g, site, side, kappa, emu, emu_inv, out);
+#pragma unroll
+            for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) epi(sp, a, out[sp][a]);
+        } else {
+            const int a = threadIdx.y;
+            dfc out[4];
+            stencil_site_a(U, in, g, site, a, side, kappa, emu, emu_inv, out);
+#pragma unroll
+            for (int sp = 0; sp < 4; ++sp) epi(sp, a, out[sp]);
         }
-        if (!ring_epilogue) {
-            // the scale 1/n_j (1/m_j) in the stencil's precision
-            T scr;
-            scr.x = from_double<R>(coef[0].x);
-            scr.y = from_double<R>(coef[0].y);
-            if (side == 0) {
-                const double2* __restrict__ prv = outer_q(o, rhs, jp);
-                double2* __restrict__ nxt = outer_q(o, rhs, j + 1);   // at j = k-1 a scratch column
-                const double2* __restrict__ dotv = TS ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
-                double2* __restrict__ yacc = PASS2 ? o.y + (size_t)rhs * o.N : nullptr;
-                const double2 cpj = PASS2 ? o.cp[hb + j] : make_double2(0.0, 0.0);
-                const double2* __restrict__ qj = outer_q(o, rhs, j);
-                for_each_out([&](int sp, int a, const T& v) {
-                    const size_t idx = (size_t)(3 * sp + a) * g.V + site;
-                    double2 rr;
-                    if (TS) {
-                        rr = make_double2(to_double(v.x * scr.x - v.y * scr.y), to_double(v.x * scr.y + v.y * scr.x));
-                        rr = caxpy_neg(rr, c1, prv[idx]);               // r - c1 q_{j-1}
-                    } else {
-                        rr = make_double2(to_double(v.x * scr.x), to_double(v.y * scr.x));
-                        const double2 pv = prv[idx];
-                        rr = make_double2(fma(-c1.x, pv.x, rr.x), fma(-c1.x, pv.y, rr.y));
-                    }
-                    nxt[idx] = rr;
-                    const double2 d = dotv[idx];
-                    acc.x = fma(d.x, rr.x, fma(d.y, rr.y, acc.x));          // conj(d) r
-                    if (TS) acc.y = fma(d.x, rr.y, fma(-d.y, rr.x, acc.y));
-                    if (PASS2) yacc[idx] = caxpy_pos(yacc[idx], cpj, qj[idx]);
-                });
-            } else {
-                const double2* __restrict__ prv = outer_p(o, rhs, jp);
-                double2* __restrict__ nxt = outer_p(o, rhs, j + 1);
-                for_each_out([&](int sp, int a, const T& v) {
-                    const size_t idx = (size_t)(3 * sp + a) * g.V + site;
-                    double2 ll = make_double2(to_double(v.x * scr.x - v.y * scr.y), to_double(v.x * scr.y + v.y * scr.x));
-                    nxt[idx] = caxpy_neg(ll, c1, prv[idx]);             // l - c1 p_{j-1}
-                });
-            }
-        }
+        acc = make_double2(df_to_double((ax[0] + ax[1]) + (ax[2] + ax[3])),
+                           df_to_double((ay[0] + ay[1]) + (ay[2] + ay[3])));
     }
     if (side == 0) {
         double2 part = block_sum(acc, sh);
@@ -629,14 +354,13 @@ __global__ void __launch_bounds__(CS * kStencilMaxThreads, CS == 1 ? StencilMinB
             // with the step-2 scalars H(j,j)/n_j (warp 1) and H(j,j)^*/m_j (warp 0) side by side
             const int tid = block_tid();
             if (tid == 0 || tid == 32) {
-                const double2 al = TS ? cmul(coef[2], tot) : make_double2(tot.x * coef[2].x, 0.0);
+                const double2 al = TS ? cmul(sc[kScD], tot) : make_double2(tot.x * sc[kScD].x, 0.0);
                 if (tid == 0) {
                     o.alpha[hb + j] = al;
                     o.counters[rhs] = 0u;
-                    o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cdiv(cconj(al), scale_m(o, rhs, j))
-                                                              : make_double2(0.0, 0.0);
+                    o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cmul(cconj(al), sc[kScM]) : make_double2(0.0, 0.0);
                 } else {
-                    o.sc[(size_t)rhs * kScalars + kScC3] = cdiv(al, scale_n(o, rhs, j));
+                    o.sc[(size_t)rhs * kScalars + kScC3] = cmul(al, sc[kScN]);
                 }
             }
         }
@@ -645,41 +369,30 @@ __global__ void __launch_bounds__(CS * kStencilMaxThreads, CS == 1 ? StencilMinB
 
 int dslash_step1_blocks(const Geom& g, int threads) { return (g.V + threads - 1) / threads; }
 
-template <typename R, typename T, int CS>
-static void launch_step1_cs(dim3 grid, dim3 block, const T* U, const Geom& g, const Outer& o, int j, R kappa,
-                            R emu, R emu_inv, const T* qin, long qs, const T* pin, long ps, cudaStream_t st) {
+template <int CS>
+static void launch_step1_cs(dim3 grid, dim3 block, const dfc* U, const Geom& g, const Outer& o, int j, df kappa,
+                            df emu, df emu_inv, cudaStream_t st) {
     const bool pass2 = o.y != nullptr;
     if (o.two_sided) {
-        if (pass2)
-            k_dslash_step1<R, true, true, CS><<<grid, block, 0, st>>>(U, g, o, j, kappa, emu, emu_inv, qin, qs, pin, ps);
-        else
-            k_dslash_step1<R, true, false, CS><<<grid, block, 0, st>>>(U, g, o, j, kappa, emu, emu_inv, qin, qs, pin, ps);
+        if (pass2) k_dslash_step1<true, true, CS><<<grid, block, 0, st>>>(U, g, o, j, kappa, emu, emu_inv);
+        else k_dslash_step1<true, false, CS><<<grid, block, 0, st>>>(U, g, o, j, kappa, emu, emu_inv);
     } else {
-        if (pass2)
-            k_dslash_step1<R, false, true, CS><<<grid, block, 0, st>>>(U, g, o, j, kappa, emu, emu_inv, qin, qs, pin, ps);
-        else
-            k_dslash_step1<R, false, false, CS><<<grid, block, 0, st>>>(U, g, o, j, kappa, emu, emu_inv, qin, qs, pin, ps);
+        if (pass2) k_dslash_step1<false, true, CS><<<grid, block, 0, st>>>(U, g, o, j, kappa, emu, emu_inv);
+        else k_dslash_step1<false, false, CS><<<grid, block, 0, st>>>(U, g, o, j, kappa, emu, emu_inv);
     }
 }
 
-template <typename R, typename T>
-static void launch_step1_t(const T* U, const Geom& g, const Outer& o, int j, R kappa, R emu, R emu_inv, const T* qin,
-                           long qs, const T* pin, long ps, cudaStream_t st) {
+static void launch_step1_df(const dfc* U, const Geom& g, const Outer& o, int j, df kappa, df emu, df emu_inv,
+                            cudaStream_t st) {
     const int nvec = o.two_sided ? 2 * o.n_rhs : o.n_rhs;
-    // launch shape of this precision (the kernel reads the grid order from o)
+    // launch shape of the early steps (the kernel reads the grid order from o)
     Outer o2 = o;
-    int split = o.st_split;
-    if (std::is_same<R, df>::value) {
-        o2.st_threads = o.st_threads_df;
-        o2.st_order = o.st_order_df;
-        split = o.st_split_df;
-    }
+    o2.st_threads = o.st_threads_df;
+    o2.st_order = o.st_order_df;
     const int threads = o2.st_threads;
     dim3 grid((unsigned)(dslash_step1_blocks(g, threads) * nvec));
-    if (split == 3)
-        launch_step1_cs<R, T, 3>(grid, dim3(threads, 3), U, g, o2, j, kappa, emu, emu_inv, qin, qs, pin, ps, st);
-    else
-        launch_step1_cs<R, T, 1>(grid, dim3(threads, 1), U, g, o2, j, kappa, emu, emu_inv, qin, qs, pin, ps, st);
+    if (o.st_split_df == 3) launch_step1_cs<3>(grid, dim3(threads, 3), U, g, o2, j, kappa, emu, emu_inv, st);
+    else launch_step1_cs<1>(grid, dim3(threads, 1), U, g, o2, j, kappa, emu, emu_inv, st);
 }
 
 bool split_step(int precision, const Outer& o, int j) {
@@ -728,12 +441,9 @@ int launch_dslash_step1(int precision, const void* U, const Geom& g, const Outer
     if (precision == 32) {
         launch_stencil32_step1(U, g, o, j, kappa, mu, st);
     } else if (precision == 48) {   // the two-float stencil reads the two-float rings
-        launch_step1_t<df, dfc>((const dfc*)U, g, o, j, df_host(kappa), df_host(exp(mu)), df_host(exp(-mu)),
-                                ring_q(o, 0, j), 3 * o.N, o.two_sided ? ring_p(o, 0, j) : nullptr, 3 * o.N, st);
+        launch_step1_df((const dfc*)U, g, o, j, df_host(kappa), df_host(exp(mu)), df_host(exp(-mu)), st);
     } else {
-        const long qs = (long)o.qcols * o.N;
-        launch_step1_t<double, double2>((const double2*)U, g, o, j, kappa, exp(mu), exp(-mu), outer_q(o, 0, j), qs,
-                                        o.two_sided ? outer_p(o, 0, j) : nullptr, (long)o.pcols * o.N, st);
+        launch_stencil64_step1(U, g, o, j, kappa, mu, st);
     }
     return 1;
 }

@@ -212,6 +212,7 @@ Layout carve(char* base, const Geom& g, int n_rhs, int k, int ell, bool two_side
     o.st_split_df = lc.early_split;
     o.npart = std::max(nblk, nk::dslash_step1_blocks(g, std::min(lc.stencil_threads, lc.early_threads)));
     o.npart = std::max(o.npart, nk::stencil32_blocks(g, two_sided ? 2 * n_rhs : n_rhs));
+    o.npart = std::max(o.npart, nk::stencil64_blocks(g, lc.stencil_threads, two_sided ? 2 * n_rhs : n_rhs));
     o.q_ring = double_pass ? 1 : 0;
     o.qcols = double_pass ? 3 : k + 1;   // single pass: k basis vectors + one scratch column
     o.Q = (double2*)take(vec * (size_t)o.qcols * n_rhs);
@@ -1396,7 +1397,7 @@ int nk_eigs_smallest(nk_ctx* c, const double* b, int k, int m, double tol, doubl
             s0.out_stride = N;
             s0.n = n;
             s0.dag = left ? 1 : 0;
-            nk::launch_dslash(64, c->U64, g, s0, s1, kappa_of(c), c->mu, st);
+            nk::launch_stencil64(c->U64, g, s0, s1, false, kappa_of(c), c->mu, st);
             for (int g0 = 0; g0 < n; g0 += 12) {
                 const int ng = std::min(12, n - g0);
                 nk::VecCoefs ca, cb;
@@ -1518,7 +1519,7 @@ int nk_eigs_smallest(nk_ctx* c, const double* b, int k, int m, double tol, doubl
                 s0.out_stride = N;
                 s0.n = n;
                 s0.dag = side;
-                nk::launch_dslash(64, c->U64, g, s0, s1, kappa_of(c), c->mu, st);
+                nk::launch_stencil64(c->U64, g, s0, s1, false, kappa_of(c), c->mu, st);
                 for (int g0 = 0; g0 < n; g0 += 12) {
                     const int ng = std::min(12, n - g0);
                     if (side == 0) {   // theta' = <l, A r>
@@ -1899,19 +1900,19 @@ int nk_dslash_dev(nk_ctx* c, const double* in_dev, double* out_dev, int n_vec, i
         NK_CUDA(c, cudaGetLastError());
         return NK_OK;
     }
-    // scratch: SoA input (FP64 or two-float) and SoA output
-    size_t bytes = align_up(sizeof(double2) * N * n_vec) * 3;
-    int rc = ensure(c, c->staging, std::max(bytes, c->staging.bytes));
-    if (rc) return rc;
-    double2* in_soa = (double2*)c->staging.p;
-    double2* out_soa = (double2*)((char*)c->staging.p + align_up(sizeof(double2) * N * n_vec));
-    float2* in32 = (float2*)((char*)out_soa + align_up(sizeof(double2) * N * n_vec));
-    nk::launch_abi_to_soa((const double2*)in_dev, N, in_soa, N, c->V, n_vec, st);
     if (precision == 48) {
+        // scratch: SoA input, its two-float copy and SoA output
+        size_t bytes = align_up(sizeof(double2) * N * n_vec) * 3;
+        int rc = ensure(c, c->staging, std::max(bytes, c->staging.bytes));
+        if (rc) return rc;
+        double2* in_soa = (double2*)c->staging.p;
+        double2* out_soa = (double2*)((char*)c->staging.p + align_up(sizeof(double2) * N * n_vec));
+        nk::dfc* in_df = (nk::dfc*)((char*)out_soa + align_up(sizeof(double2) * N * n_vec));
+        nk::launch_abi_to_soa((const double2*)in_dev, N, in_soa, N, c->V, n_vec, st);
         // the multi-RHS two-float stencil of the solver's early steps
-        nk::launch_to_df(in_soa, N, (nk::dfc*)in32, N, N, n_vec, st);
+        nk::launch_to_df(in_soa, N, in_df, N, N, n_vec, st);
         nk::StencilDfSet sd;
-        sd.in_a = sd.in_d = (const nk::dfc*)in32;
+        sd.in_a = sd.in_d = in_df;
         sd.in_stride = N;
         sd.out_a = sd.out_d = out_soa;
         sd.out_stride = N;
@@ -1923,18 +1924,26 @@ int nk_dslash_dev(nk_ctx* c, const double* in_dev, double* out_dev, int n_vec, i
         NK_CUDA(c, cudaGetLastError());
         return NK_OK;
     }
+    // FP64: straight from and to the ABI layout; where out overlaps in, from a
+    // copy of in (a site's neighbours are read after its own result is written)
+    const size_t vbytes = sizeof(double2) * (size_t)N * n_vec;
+    const uintptr_t ia = (uintptr_t)in_dev, oa = (uintptr_t)out_dev;
+    if (ia < oa + vbytes && oa < ia + vbytes) {
+        int rc = ensure(c, c->staging, std::max(vbytes, c->staging.bytes));
+        if (rc) return rc;
+        NK_CUDA(c, cudaMemcpyAsync(c->staging.p, in_dev, vbytes, cudaMemcpyDeviceToDevice, st));
+        in_dev = (const double*)c->staging.p;
+    }
     nk::DslashSet s0, s1;
     std::memset(&s0, 0, sizeof(s0));
     std::memset(&s1, 0, sizeof(s1));
-    s0.in = in_soa;
+    s0.in = in_dev;
     s0.in_stride = N;
-    s0.out = out_soa;
+    s0.out = (double2*)out_dev;
     s0.out_stride = N;
     s0.n = n_vec;
     s0.dag = dagger ? 1 : 0;
-    nk::launch_dslash(precision, precision == 48 ? (const void*)c->Udf : (const void*)c->U64, geom_of(c), s0, s1,
-                      kappa_of(c), c->mu, st);
-    nk::launch_soa_to_abi(out_soa, N, (double2*)out_dev, N, nullptr, 0, c->V, n_vec, st);
+    nk::launch_stencil64(c->U64, geom_of(c), s0, s1, true, kappa_of(c), c->mu, st);
     NK_CUDA(c, cudaGetLastError());
     return NK_OK;
 }

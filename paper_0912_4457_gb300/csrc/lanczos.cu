@@ -123,46 +123,49 @@ __global__ void __launch_bounds__(kThreads) k_init(Outer o, int copy_mode) {
 
 // End of step 2: the deterministic reduction of the per-thread partial
 // (r^dag r, or r^dag l two-sided) and, in the last block, beta and gamma and
-// the scalars of step j + 1 (one complex division per warp, side by side on
-// the SM sub-partitions).
+// the scalars of step j + 1.  This tail is a chain of dependent FP64
+// operations on one lane, several microseconds long and all of a small
+// lattice's step, so it holds no division twice: 1/n_j and 1/m_j of the
+// current step are the scalars kScN and kScM, 1/beta serves gamma and 1/n_{j+1}.
 template <bool TS>
 __device__ __forceinline__ void step2_finish(const Outer& o, int rhs, int j, double2 acc, double2* sh) {
-    __shared__ double2 bg[2];
     double2 part = block_sum(acc, sh);
     if (finish_partial(part, o.partials + (size_t)rhs * o.npart, o.counters + rhs, blockIdx.x, o.nblk)) {
+        double2* sc = o.sc + (size_t)rhs * kScalars;
+        const double2 inv_n = sc[kScN], inv_m = sc[kScM];   // 1/n_j, 1/m_j
         double2 d = sum_partials(o.partials + (size_t)rhs * o.npart, o.nblk, sh);
         if (threadIdx.x == 0) {
             const size_t at = (size_t)rhs * o.k + j;
-            double2 b, g;
+            double2 b, g, ib = mk(0.0, 0.0);
+            bool ok = true;
             if (!TS) {
                 const double bb = sqrt(d.x);             // beta <- sqrt(r^dag r)
                 b = g = mk(bb, 0.0);
-                if (!(bb > 0.0) || !isfinite(bb)) mark_failed(o, rhs, kStatusBreakdown);
+                ok = bb > 0.0 && isfinite(bb);
+                if (!ok) mark_failed(o, rhs, kStatusBreakdown);
+                else ib = cinv(b);
             } else if ((d.x == 0.0 && d.y == 0.0) || !isfinite(d.x) || !isfinite(d.y)) {
                 // serious breakdown: delta = 0 (App. B); a non-finite delta is treated alike
                 mark_failed(o, rhs, kStatusBreakdown);
                 b = g = mk(0.0, 0.0);
+                ok = false;
             } else {
                 b = csqrt_principal(d);                  // beta <- sqrt(delta)
-                g = cdiv(cconj(d), b);                   // gamma <- delta^* / beta
+                ib = cinv(b);
+                g = cmul(cconj(d), ib);                  // gamma <- delta^* / beta
             }
             o.beta[at] = b;
             o.gamma[at] = g;
-            bg[0] = b;
-            bg[1] = g;
             o.counters[rhs] = 0u;
-        }
-        __syncthreads();
-        // step j + 1: n_{j+1} = beta_j, m_{j+1} = gamma_j^*
-        const int w = threadIdx.x >> 5;
-        if ((threadIdx.x & 31) == 0 && w < 5 && j + 1 < o.k && o.status[rhs] == kStatusOK) {
-            const double2 b = bg[0], g = bg[1];
-            double2* sc = o.sc + (size_t)rhs * kScalars;
-            if (w == 0) sc[kScN] = cinv(b);
-            else if (w == 1) sc[kScC1] = cdiv(TS ? g : b, scale_n(o, rhs, j));
-            else if (w == 2) sc[kScD] = TS ? cinv(g) : cinv(b);
-            else if (w == 3) sc[kScM] = cinv(cconj(g));
-            else sc[kScC1L] = cdiv(cconj(b), scale_m(o, rhs, j));
+            // step j + 1: n_{j+1} = beta_j, m_{j+1} = gamma_j^*
+            if (ok && j + 1 < o.k && o.status[rhs] == kStatusOK) {
+                const double2 ig = TS ? cinv(g) : ib;
+                sc[kScN] = ib;
+                sc[kScC1] = cmul(g, inv_n);              // gamma (Hermitian: beta) / n_j
+                sc[kScD] = ig;
+                sc[kScM] = cconj(ig);
+                sc[kScC1L] = cmul(cconj(b), inv_m);
+            }
         }
     }
 }
@@ -463,10 +466,10 @@ __global__ void __launch_bounds__(kStreamThreads) k_step1(Outer o, int j) {
             o.alpha[(size_t)rhs * o.k + j] = al;
             o.counters[rhs] = 0u;
         }
-        // the step-2 scalars H(j,j)/n_j and H(j,j)^*/m_j, one division per warp
-        if ((threadIdx.x & 31) == 0 && w == 1) o.sc[(size_t)rhs * kScalars + kScC3] = cdiv(al, scale_n(o, rhs, j));
+        // the step-2 scalars H(j,j)/n_j and H(j,j)^*/m_j from the inverses kScN and kScM
+        if ((threadIdx.x & 31) == 0 && w == 1) o.sc[(size_t)rhs * kScalars + kScC3] = cmul(al, sc[kScN]);
         if ((threadIdx.x & 31) == 0 && w == 2)
-            o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cdiv(cconj(al), scale_m(o, rhs, j)) : mk(0.0, 0.0);
+            o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cmul(cconj(al), sc[kScM]) : mk(0.0, 0.0);
     }
 }
 

@@ -1,6 +1,5 @@
-// The Wilson hop of Sec. 2 in the chiral basis, for FP32 and FP64 values in
-// registers: acc += w (1 + s gamma_nu) M psi with M = U or U^dagger.  Shared
-// by the stencil kernels of dslash.cu and stencil32.cu.
+// The Wilson hop of Sec. 2 in the chiral basis, for values in registers:
+// acc += w (1 + s gamma_nu) M psi with M = U or U^dagger (stencil32.cu).
 //
 // (1 + s gamma_nu) psi = [h ; s B_nu h] with the half spinor
 // h = psi_up + s C_nu psi_dn, C_k = -i sigma_k, B_k = i sigma_k, C_4 = B_4 = 1,
@@ -24,7 +23,7 @@ template <typename T> __device__ __forceinline__ T neg(T z) { T r; r.x = -z.x; r
 
 // One hop: acc += w * (1 + s gamma_nu) M psi_n with M = U (dag = false) or
 // U^dagger, from a neighbour spinor and link already loaded into registers
-// (FP32 and FP64; the two-float stencil has its own form below).
+// (the FP64 and the two-float stencils have their own forms).
 template <int NU, bool DAG, typename R>
 __device__ __forceinline__ void hop_regs(typename C2<R>::T acc[4][3], const typename C2<R>::T psi[4][3],
                                          const typename C2<R>::T u[3][3], R s, R w) {

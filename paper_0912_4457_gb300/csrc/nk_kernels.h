@@ -9,13 +9,14 @@ namespace nk {
 
 struct dfc;   // two-float complex (nk_common.cuh)
 
+struct Outer;
+
 struct Geom {
     int Lx, Ly, Lz, Lt, V;
     int antiperiodic;
 };
 
 // A set of vectors for one stencil launch: out_i = A in_i (dag = 0) or A^dagger in_i.
-// `in` is double2* for the FP64 stencil and float2* for the FP32 one.
 struct DslashSet {
     const void* in;
     long in_stride;   // elements (complex) between consecutive vectors
@@ -25,8 +26,14 @@ struct DslashSet {
     int dag;
 };
 
-void launch_dslash(int precision, const void* U, const Geom& g, const DslashSet& s0,
-                   const DslashSet& s1, double kappa, double mu, cudaStream_t st);
+// The FP64 stencil alone (stencil64.cu) on the vectors of two sets, in the ABI layout
+// ([site][12]) or the device one ([12][site]), and fused with the first half of outer
+// step j.
+void launch_stencil64(const void* U64, const Geom& g, const DslashSet& s0, const DslashSet& s1, bool abi, double kappa,
+                      double mu, cudaStream_t st);
+void launch_stencil64_step1(const void* U64, const Geom& g, const Outer& o, int j, double kappa, double mu,
+                            cudaStream_t st);
+int stencil64_blocks(const Geom& g, int threads, int nvec);   // CTAs, hence partial sums, per vector
 void launch_links_to_device_layout(const double2* in, double2* u64, float2* u32, dfc* udf, int V,
                                    cudaStream_t st);
 int plaquette_blocks(const Geom& g);

@@ -1,0 +1,339 @@
+// FP64 Wilson stencil A = gamma5 D_w(mu), A^dagger = gamma5 D_w(-mu) (Sec. 2):
+// alone, and fused with the first half of an outer Lanczos step.
+//
+// What bounds it.  A site and vector take 888 FP64 instructions per lane
+// (projection 96, link products 576, accumulation and output 216), and GB300
+// issues two FP64 lanes per clock and SM: one thread per site and vector
+// keeps a warp on the FP64 pipe for at least 888 x 16 clocks, and on the
+// small lattices most of the chip has no warp at all (4^4, one vector: 55 us
+// in two CTAs; 10^4, both sides of one source: 82 us against a floor of 29).
+// So a site is spread over 16 threads, one per hop h = 0..7 (nu = h / 2, odd
+// h forward) and half-spinor column c: each projects its column of the
+// neighbour spinor (6 additions), multiplies it by the link (36 fused
+// multiply-adds) and leaves the three colours in shared memory; after one
+// barrier 12 threads per site sum the eight hops of one spin-colour
+// component each.  No FP64 operation is done twice, the sums run over the
+// hops in the order 0..7, and a CTA of S sites (S = 4, 8 or 16) is short
+// enough to fill the chip from 4^4 on.  Measured, outer step (this kernel and
+// step 2) of one source: 4^4, mu = 0 51.5 -> 16.8 us; 6^4, mu = 0.1 58 -> 28;
+// 10^4, mu = 0.2 95 -> 65; 12 sources at 10^4, mu = 0: 235.  The stencil alone
+// on 12 vectors at 16^3 x 32, 2.44 -> 2.34 ms (its FP64 floor is 2.25), and
+// straight from and to the ABI layout, without the two conversion passes
+// (0.2 ms).  Profile at 10^4: FP64 pipe 82% busy while an SM has work.
+//
+// The gamma matrices act on the half spinors as multiplications by i^q (swaps
+// and sign flips on the integer pipe), so the lanes of a warp may work on
+// different hops without diverging.  SPLIT = 3 (a launch shape) gives each
+// colour row of the product its own thread: a third of the chain per thread
+// for 22% more FP64 work (the projection is repeated); it was never faster at
+// the default S = 8 (6^4 28 against 32 us) and level with it at S = 4, 4^4.
+#include "nk_common.cuh"
+#include "nk_kernels.h"
+
+namespace nk {
+
+namespace {
+
+constexpr int kS64Sites = 56;   // sites resident per SM: 56 / S CTAs (28 warps at 72 registers)
+
+__device__ __forceinline__ double flip(double x, unsigned mask) {   // mask: 0 or the sign bit
+    return __hiloint2double(__double2hiint(x) ^ (int)mask, __double2loint(x));
+}
+// z * i^q
+__device__ __forceinline__ double2 rot(double2 z, int q) {
+    const unsigned sx = ((q + 1) & 2) ? 0x80000000u : 0u;   // q = 1, 2
+    const unsigned sy = (q & 2) ? 0x80000000u : 0u;         // q = 2, 3
+    const double x = (q & 1) ? z.y : z.x, y = (q & 1) ? z.x : z.y;
+    return make_double2(flip(x, sx), flip(y, sy));
+}
+
+// Index of component c of a site: [12][V] (device layout) or [V][12] (ABI layout).
+template <bool ABI>
+__device__ __forceinline__ size_t comp_at(int c, int site, int V) {
+    return ABI ? (size_t)site * 12 + c : (size_t)c * V + site;
+}
+
+// Phase 1: thread (s, h, c[, a]) of the CTA's sites leaves row(s) a of
+// M (psi_up + s C psi_dn)_c of hop h in sx[((h * 2 + c) * 3 + a) * S + s].
+// The coordinate of `site` along nu decides the neighbour; sites past V use V - 1.
+template <int S, int SPLIT, bool ABI>
+__device__ __forceinline__ void s64_hops(const double2* __restrict__ U, const double2* __restrict__ in, const Geom& g,
+                                         int site0, double2* __restrict__ sx) {
+    constexpr int ROWS = 3 / SPLIT;
+    const int tid = threadIdx.x;
+    const int s = tid % S, hc = (tid / S) & 15, a0 = SPLIT == 1 ? 0 : tid / (16 * S);
+    const int h = hc >> 1, c = hc & 1, nu = h >> 1;
+    const bool fwd = (h & 1) != 0;
+    const int V = g.V;
+    const int site = min(site0 + s, V - 1);
+    const int L = nu == 0 ? g.Lx : nu == 1 ? g.Ly : nu == 2 ? g.Lz : g.Lt;
+    const int stride = nu == 0 ? 1 : nu == 1 ? g.Lx : nu == 2 ? g.Lx * g.Ly : g.Lx * g.Ly * g.Lz;
+    const int x = (int)(((unsigned)site / (unsigned)stride) % (unsigned)L);
+    const int sn = fwd ? (x == L - 1 ? site - (L - 1) * stride : site + stride)
+                       : (x == 0 ? site + (L - 1) * stride : site - stride);
+    // M = U(x - nu) backward, U(x)^dagger forward: row a, column b
+    const double2* __restrict__ Ul = U + (size_t)(nu * 9) * V + (fwd ? site : sn);
+    const int ra = fwd ? 1 : 3, rb = fwd ? 3 : 1;
+    const unsigned mc = fwd ? 0x80000000u : 0u;
+    double2 m[ROWS][3], up[3], dn[3];
+    // (C_nu psi_dn)_c = i^q psi_ic: nu = x: i^3 psi_3, i^3 psi_2; y: i^2 psi_3, psi_2;
+    // z: i^3 psi_2, i psi_3; t: psi_2, psi_3; forward hops take the opposite sign (q + 2)
+    const int ic = nu < 2 ? 3 - c : 2 + c;
+    const int q = (nu == 0 ? 3 : nu == 1 ? (c ? 0 : 2) : nu == 2 ? (c ? 1 : 3) : 0) + (fwd ? 2 : 0);
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        up[b] = in[comp_at<ABI>(3 * c + b, sn, V)];
+        dn[b] = in[comp_at<ABI>(3 * ic + b, sn, V)];
+    }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) m[r][b] = Ul[(size_t)((a0 + r) * ra + b * rb) * V];
+    double2 hh[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const double2 d = rot(dn[b], q);
+        hh[b] = make_double2(up[b].x + d.x, up[b].y + d.y);
+    }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        double2 v = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const double ex = m[r][b].x, ey = flip(m[r][b].y, mc), ny = flip(ey, 0x80000000u);
+            v.x = fma(ny, hh[b].y, b == 0 ? ex * hh[b].x : fma(ex, hh[b].x, v.x));
+            v.y = fma(ey, hh[b].x, b == 0 ? ex * hh[b].y : fma(ex, hh[b].y, v.y));
+        }
+        sx[((h * 2 + c) * 3 + a0 + r) * S + s] = v;
+    }
+}
+
+// Phase 2: the sum over the eight hops for spin sp, colour a of slot s.
+// (B_nu m)_0,1 of the lower spins: x: i m_1, i m_0; y: m_1, -m_0; z: i m_0,
+// -i m_1; t: m_0, m_1, times -1 for the forward hops; wp_t, wm_t are the
+// temporal weights of this site (with the boundary sign).
+template <int S>
+__device__ __forceinline__ double2 s64_sum(const double2* __restrict__ sx, int s, int sp, int a, double wp_t,
+                                           double wm_t) {
+    double2 acc = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+        const int nu = h >> 1;
+        const bool fwd = (h & 1) != 0;
+        // column and i^q of spins 2 and 3
+        const int col2 = nu < 2 ? 1 : 0, q2 = nu == 0 || nu == 2 ? 1 : 0;
+        const int q3 = nu == 0 ? 1 : nu == 1 ? 2 : nu == 2 ? 3 : 0;
+        const int col = sp < 2 ? sp : sp == 2 ? col2 : 1 - col2;
+        const int q = sp < 2 ? 0 : (sp == 2 ? q2 : q3) + (fwd ? 2 : 0);
+        const double2 b = rot(sx[((h * 2 + col) * 3 + a) * S + s], q);
+        if (nu == 3) {
+            const double w = fwd ? wm_t : wp_t;
+            acc.x = fma(w, b.x, acc.x);
+            acc.y = fma(w, b.y, acc.y);
+        } else if (h == 0) {
+            acc = b;
+        } else {
+            acc.x += b.x;
+            acc.y += b.y;
+        }
+    }
+    return acc;
+}
+
+// The temporal weights of a site: A uses (e^{mu}, e^{-mu}), A^dagger exchanges
+// them; a hop across the antiperiodic t boundary carries -1.
+__device__ __forceinline__ void t_weights(const Geom& g, int site, int dag, double emu, double emu_inv, double& wp,
+                                          double& wm) {
+    const int t = site / (g.Lx * g.Ly * g.Lz);
+    wp = dag ? emu_inv : emu;
+    wm = dag ? emu : emu_inv;
+    if (g.antiperiodic && t == 0) wp = flip(wp, 0x80000000u);
+    if (g.antiperiodic && t == g.Lt - 1) wm = flip(wm, 0x80000000u);
+}
+
+// ---- the stencil alone ------------------------------------------------------------
+// One CTA per block of S sites and vector, the vector index fastest (the links
+// of a block of sites come from HBM once and then from L2).
+template <int S, bool ABI>
+__global__ void __launch_bounds__(16 * S) k_stencil64(const double2* __restrict__ U, Geom g, DslashSet s0, DslashSet s1,
+                                                      double kappa, double emu, double emu_inv) {
+    __shared__ double2 sx[48 * S];
+    const int nvec = s0.n + s1.n;
+    const int vec = blockIdx.x % nvec, site0 = (blockIdx.x / nvec) * S;
+    const DslashSet& D = vec < s0.n ? s0 : s1;
+    const int vi = vec < s0.n ? vec : vec - s0.n;
+    const double2* __restrict__ in = reinterpret_cast<const double2*>(D.in) + (size_t)vi * D.in_stride;
+    s64_hops<S, 1, ABI>(U, in, g, site0, sx);
+    // component-fastest threads in the ABI layout, site-fastest in the device one (coalesced
+    // stores).  12 of 16 threads sum: which warps idle rotates with the block of sites, as
+    // the FP64 pipe of an SM sub-partition serves the warps of one residue mod 4
+    const int tid = (threadIdx.x + 32 * ((blockIdx.x / nvec) & 3)) % (16 * S);
+    const int s = ABI ? tid / 12 : tid % S, comp = ABI ? tid % 12 : tid / S;
+    const int site = site0 + s;
+    const bool live = tid < 12 * S && site < g.V;
+    double2 p = make_double2(0.0, 0.0);
+    if (live) p = in[comp_at<ABI>(comp, site, g.V)];
+    __syncthreads();
+    if (!live) return;
+    double wp, wm;
+    t_weights(g, site, D.dag, emu, emu_inv, wp, wm);
+    const int sp = comp / 3;
+    const double2 acc = s64_sum<S>(sx, s, sp, comp % 3, wp, wm);
+    const unsigned sg = sp < 2 ? 0u : 0x80000000u;   // gamma5 = diag(1, 1, -1, -1)
+    double2* __restrict__ out = D.out + (size_t)vi * D.out_stride;
+    out[comp_at<ABI>(comp, site, g.V)] = make_double2(flip(fma(-kappa, acc.x, p.x), sg), flip(fma(-kappa, acc.y, p.y), sg));
+}
+
+__device__ __forceinline__ double2 caxpy_neg(double2 s, double2 c, double2 p) {   // s - c p
+    return make_double2(fma(-c.x, p.x, fma(c.y, p.y, s.x)), fma(-c.x, p.y, fma(-c.y, p.x, s.y)));
+}
+__device__ __forceinline__ double2 caxpy_pos(double2 s, double2 c, double2 p) {   // s + c p
+    return make_double2(fma(c.x, p.x, fma(-c.y, p.y, s.x)), fma(c.x, p.y, fma(c.y, p.x, s.y)));
+}
+
+// ---- fused with the first half of outer step j --------------------------------------
+// (lanczos.cu describes the unnormalised basis q_j, p_j)
+//   side 0: r = (A q_j) / n_j - (c_{j-1}/n_{j-1}) q_{j-1} -> q_{j+1},
+//           H(j,j) = (p_j^dag r) / m_j^*  (Hermitian: Re(q_j^dag r) / n_j),
+//   side 1: l = (A^dag p_j) / m_j - (beta^*_{j-1}/m_{j-1}) p_{j-1} -> p_{j+1}.
+// The scalars of the step come from o.sc; the CTA that finishes last forms
+// H(j,j) and the step-2 scalars.  CTA b of a vector walks a contiguous range
+// of the site blocks; the grid is at most one wave (stencil64_blocks).
+// In double-pass mode side 0 also accumulates y += c'_j q_j at its own site.
+template <int S, int SPLIT, bool TS, bool PASS2>
+__global__ void __launch_bounds__(16 * S * SPLIT, SPLIT == 1 ? kS64Sites / S : 1) k_stencil64_step1(const double2* __restrict__ U, Geom g, Outer o, int j,
+                                                                    double kappa, double emu, double emu_inv, int nblk) {
+    __shared__ double2 sx[48 * S];
+    __shared__ double2 sh[33];
+    const int nvec = TS ? 2 * o.n_rhs : o.n_rhs;
+    const int vec = o.st_order == 0 ? blockIdx.x % nvec : blockIdx.x / nblk;
+    const int blk = o.st_order == 0 ? blockIdx.x / nvec : blockIdx.x % nblk;
+    const int side = vec / o.n_rhs;      // 0: A q_j, 1: A^dagger p_j
+    const int rhs = vec % o.n_rhs;
+    if (o.status[rhs] != kStatusOK) return;
+    if (side == 1 && j == o.k - 1) return;   // the last step needs no left vector
+    const double2* __restrict__ sc = o.sc + (size_t)rhs * kScalars;
+    const double2 scl = sc[side ? kScM : kScN];     // 1/n_j (1/m_j)
+    const double2 c1 = sc[side ? kScC1L : kScC1];   // zero at j = 0 (the previous vector is then any valid one)
+    const int V = g.V, nsb = (V + S - 1) / S;
+    const int b_lo = (int)((long)blk * nsb / nblk), b_hi = (int)((long)(blk + 1) * nsb / nblk);
+    const int jp = j > 0 ? j - 1 : j;
+    const double2* __restrict__ in = side ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
+    const double2* __restrict__ prv = side ? outer_p(o, rhs, jp) : outer_q(o, rhs, jp);
+    double2* __restrict__ nxt = side ? outer_p(o, rhs, j + 1) : outer_q(o, rhs, j + 1);   // a scratch column at j = k - 1
+    const double2* __restrict__ dotv = TS ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
+    double2* __restrict__ yacc = PASS2 ? o.y + (size_t)rhs * o.N : nullptr;
+    const double2 cpj = PASS2 ? o.cp[(size_t)rhs * o.k + j] : make_double2(0.0, 0.0);
+    const int tid = threadIdx.x;
+    const int t2 = (tid + 32 * (blk & 3)) % (16 * S * SPLIT);   // idle warps rotate, as in k_stencil64
+    const int s = t2 % S, comp = t2 / S, sp = comp / 3, a = comp % 3;
+    const unsigned sg = sp < 2 ? 0u : 0x80000000u;   // gamma5 = diag(1, 1, -1, -1)
+    double2 dot = make_double2(0.0, 0.0);
+    for (int b = b_lo; b < b_hi; ++b) {
+        s64_hops<S, SPLIT, false>(U, in, g, b * S, sx);
+        const int site = b * S + s;
+        const bool live = comp < 12 && site < V;
+        const size_t idx = (size_t)comp * V + site;
+        double2 p = make_double2(0.0, 0.0), pv = p, d = p;
+        if (live) {
+            p = in[idx];
+            pv = prv[idx];
+            if (side == 0) d = dotv[idx];
+        }
+        __syncthreads();
+        if (live) {
+            double wp, wm;
+            t_weights(g, site, side, emu, emu_inv, wp, wm);
+            const double2 acc = s64_sum<S>(sx, s, sp, a, wp, wm);
+            const double2 v = make_double2(flip(fma(-kappa, acc.x, p.x), sg), flip(fma(-kappa, acc.y, p.y), sg));
+            double2 rr;
+            if (TS) {
+                rr = make_double2(v.x * scl.x - v.y * scl.y, v.x * scl.y + v.y * scl.x);
+                rr = caxpy_neg(rr, c1, pv);
+            } else {
+                rr = make_double2(v.x * scl.x, v.y * scl.x);
+                rr = make_double2(fma(-c1.x, pv.x, rr.x), fma(-c1.x, pv.y, rr.y));
+            }
+            nxt[idx] = rr;
+            if (side == 0) {
+                dot.x = fma(d.x, rr.x, fma(d.y, rr.y, dot.x));      // conj(d) r
+                if (TS) dot.y = fma(d.x, rr.y, fma(-d.y, rr.x, dot.y));
+                if (PASS2) yacc[idx] = caxpy_pos(yacc[idx], cpj, TS ? p : d);
+            }
+        }
+        if (b + 1 < b_hi) __syncthreads();   // sx is rewritten
+    }
+    if (side != 0) return;
+    const double2 part = block_sum(dot, sh);
+    if (finish_partial(part, o.partials + (size_t)rhs * o.npart, o.counters + rhs, blk, nblk)) {
+        const double2 tot = sum_partials(o.partials + (size_t)rhs * o.npart, nblk, sh);
+        // Hermitian: H(j,j) = Re(q_j^dag r) / n_j, real (App. C); two-sided: (p_j^dag r) / m_j^*;
+        // the step-2 scalars H(j,j)/n_j (warp 1) and H(j,j)^*/m_j (warp 0) side by side
+        if (tid == 0 || tid == 32) {
+            const double2 al = TS ? cmul(sc[kScD], tot) : make_double2(tot.x * sc[kScD].x, 0.0);
+            if (tid == 0) {
+                o.alpha[(size_t)rhs * o.k + j] = al;
+                o.counters[rhs] = 0u;
+                o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cmul(cconj(al), sc[kScM]) : make_double2(0.0, 0.0);
+            } else {
+                o.sc[(size_t)rhs * kScalars + kScC3] = cmul(al, sc[kScN]);
+            }
+        }
+    }
+}
+
+template <int S, int SPLIT>
+void launch_s64_step1(const double2* U, const Geom& g, const Outer& o, int j, double kappa, double emu, double emu_inv,
+                      cudaStream_t st) {
+    const int nvec = o.two_sided ? 2 * o.n_rhs : o.n_rhs;
+    const int nblk = stencil64_blocks(g, 16 * S, nvec);
+    const unsigned grid = (unsigned)nblk * (unsigned)nvec;
+    constexpr int T = 16 * S * SPLIT;
+    const bool pass2 = o.y != nullptr;
+    if (o.two_sided) {
+        if (pass2) k_stencil64_step1<S, SPLIT, true, true><<<grid, T, 0, st>>>(U, g, o, j, kappa, emu, emu_inv, nblk);
+        else k_stencil64_step1<S, SPLIT, true, false><<<grid, T, 0, st>>>(U, g, o, j, kappa, emu, emu_inv, nblk);
+    } else {
+        if (pass2) k_stencil64_step1<S, SPLIT, false, true><<<grid, T, 0, st>>>(U, g, o, j, kappa, emu, emu_inv, nblk);
+        else k_stencil64_step1<S, SPLIT, false, false><<<grid, T, 0, st>>>(U, g, o, j, kappa, emu, emu_inv, nblk);
+    }
+}
+
+}  // namespace
+
+// CTAs (and partial sums) per vector of the fused kernel with `threads`
+// threads per CTA at split 1 (threads / 16 sites): one per block of sites, but
+// no more than one wave of the chip over all vectors
+int stencil64_blocks(const Geom& g, int threads, int nvec) {
+    const int S = threads / 16;
+    const int nsb = (g.V + S - 1) / S;
+    const int wave = 152 * (kS64Sites / S) / nvec;
+    return nsb < wave ? nsb : (wave > 0 ? wave : 1);
+}
+
+void launch_stencil64_step1(const void* U64, const Geom& g, const Outer& o, int j, double kappa, double mu,
+                            cudaStream_t st) {
+    const double2* U = (const double2*)U64;
+    const double ep = exp(mu), em = exp(-mu);
+#define NK_S64(S_)                                                                    \
+    do {                                                                              \
+        if (o.st_split == 3) launch_s64_step1<S_, 3>(U, g, o, j, kappa, ep, em, st);  \
+        else launch_s64_step1<S_, 1>(U, g, o, j, kappa, ep, em, st);                  \
+    } while (0)
+    if (o.st_threads == 64) NK_S64(4);
+    else if (o.st_threads == 128) NK_S64(8);
+    else NK_S64(16);
+#undef NK_S64
+}
+
+void launch_stencil64(const void* U64, const Geom& g, const DslashSet& s0, const DslashSet& s1, bool abi, double kappa,
+                      double mu, cudaStream_t st) {
+    const int nvec = s0.n + s1.n;
+    if (nvec == 0) return;
+    constexpr int S = 8;
+    const unsigned grid = (unsigned)((g.V + S - 1) / S) * (unsigned)nvec;
+    if (abi) k_stencil64<S, true><<<grid, 16 * S, 0, st>>>((const double2*)U64, g, s0, s1, kappa, exp(mu), exp(-mu));
+    else k_stencil64<S, false><<<grid, 16 * S, 0, st>>>((const double2*)U64, g, s0, s1, kappa, exp(mu), exp(-mu));
+}
+
+}  // namespace nk

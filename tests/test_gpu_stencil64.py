@@ -1,0 +1,85 @@
+"""The FP64 stencil (16 threads per site): the stencil alone and fused with the
+first half of an outer step, on lattices whose volume is no multiple of a
+CTA's sites, for every launch shape, and with overlapping input and output.
+
+Tolerances: one application sums about 100 products per component (1e-13);
+the first 12 steps of a recurrence agree to 1e-11, as in test_gpu_parity.
+"""
+import numpy as np
+import pytest
+
+import inputs
+from oracle import dirac, nested
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_0912_4457_gb300.nksign import NK_DOUBLE_PASS, NK_FP64, Context  # noqa: E402
+
+M_W = -2.0
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / np.linalg.norm(np.asarray(b)))
+
+
+def make_ctx(dims, mu, antiperiodic=True):
+    U = inputs.su3_links(dims, 41)[0]
+    ctx = Context(dims, antiperiodic)
+    ctx.load_links(U)
+    ctx.set_mu_mw(mu, M_W)
+    return ctx, U
+
+
+@pytest.mark.parametrize("dims,n", [((2, 2, 2, 2), 1), ((3, 3, 3, 3), 5), ((2, 3, 5, 7), 24), ((5, 2, 3, 3), 2)])
+@pytest.mark.parametrize("antiperiodic", [True, False])
+def test_alone_odd_volumes(dims, n, antiperiodic):
+    ctx, U = make_ctx(dims, 0.3, antiperiodic)
+    x = inputs.gaussian_sources(dims, 42, n_rhs=n)
+    xd = torch.from_numpy(x).cuda()
+    for dagger in (False, True):
+        out = torch.zeros_like(xd)
+        ctx.dslash_dev(xd, out, n, dagger=dagger, precision=64)
+        got = out.cpu().numpy()
+        f = dirac.apply_A_dagger if dagger else dirac.apply_A
+        for i in range(n):
+            assert rel(got[i], f(x[i], U, dims, 0.3, M_W, antiperiodic_t=antiperiodic)) < 1e-13
+    ctx.close()
+
+
+def test_alone_in_place_and_shifted():
+    """out may be in, or overlap it: the result is that of separate arrays."""
+    dims, n = (3, 4, 3, 5), 3
+    ctx, U = make_ctx(dims, 0.2)
+    x = torch.from_numpy(inputs.gaussian_sources(dims, 43, n_rhs=n + 1)).cuda()
+    ref = torch.zeros_like(x)
+    ctx.dslash_dev(x, ref, n, precision=64)
+    for shift in (0, 1):
+        buf = x.clone()
+        ctx.dslash_dev(buf[:n], buf[shift:shift + n], n, precision=64)
+        assert torch.equal(buf[shift:shift + n], ref[:n])
+    ctx.close()
+
+
+@pytest.mark.parametrize("mu", [0.0, 0.3])
+@pytest.mark.parametrize("threads,order,split", [(64, 0, 1), (128, 1, 1), (256, 0, 1), (64, 1, 3), (128, 0, 3), (256, 1, 3)])
+def test_fused_step_shapes(mu, threads, order, split):
+    dims, n, k = (3, 5, 3, 7), 2, 12
+    ctx, U = make_ctx(dims, mu)
+    b = inputs.gaussian_sources(dims, 44, n_rhs=n)
+    ctx.set_launch(n, NK_FP64, threads, order, 3, 128, 0, split, 1)
+    al, be, ga, _ = ctx.outer_lanczos_dev(torch.from_numpy(b).cuda(), n, k)
+    A, Ad, herm = nested.operator(U, dims, mu, M_W)
+    for i in range(n):
+        ref = nested.outer_basis(A, Ad, b[i], k, herm)
+        assert rel(al[i], ref.alpha) < 1e-11
+        assert rel(be[i, :k - 1], ref.beta[:k - 1]) < 1e-11
+        assert rel(ga[i, :k - 1], ref.gamma[:k - 1]) < 1e-11
+    # the second pass of a double-pass solve regenerates the same basis
+    y1, _, _ = ctx.sign_apply(b, k, 8, p=1.0)
+    y2, _, _ = ctx.sign_apply(b, k, 8, p=1.0, flags=NK_FP64 | NK_DOUBLE_PASS)
+    assert rel(y2, y1) < 1e-13
+    ctx.close()
