@@ -52,10 +52,9 @@ extern "C" {
 #define NK_ENOTCONV (-4)    /* adaptive k: tolerance not met at k_max */
 #define NK_ERHI (-5)        /* Roberts-Higham iteration did not converge */
 #define NK_ECUDA (-6)       /* CUDA runtime error */
-#define NK_ETIMEOUT (-7)    /* a bounded device-side wait ran out: the streaming kernels of the
-                               outer recurrence wait at most one second for the bulk copies of
-                               each tile into shared memory; that RHS is failed (the RHi
-                               clusters synchronise with hardware cluster barriers) */
+#define NK_ETIMEOUT (-7)    /* a bounded device-side wait ran out (kept for callers that test for it: no
+                               kernel waits on another one or on its own copies now; the clusters
+                               synchronise with hardware cluster barriers) */
 #define NK_ESTATE (-8)      /* call out of order (e.g. no links loaded) */
 
 /* Solve flags (bitwise or). */
@@ -272,7 +271,7 @@ int nk_set_adapt_start(nk_ctx* ctx, int k_first);
  * A shape belongs to (n_rhs, sidedness of the current mu (mu != 0), the
  * NK_MIXED bit of flags).  Different shapes sum in different orders, so
  * results differ at rounding level; one shape is bitwise reproducible.
- * Unset shapes use 128 / 0 / min(ceil(12 V / 2048), 608 / n_rhs) / 128 / 0 / 1 / 1.
+ * Unset shapes use 128 / 0 / min(ceil(6 V / 128), 760 / n_rhs in fours) / 128 / 0 / 1 / 1.
  */
 typedef struct nk_launch {
     int stencil_threads;

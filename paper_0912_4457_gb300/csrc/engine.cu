@@ -293,16 +293,11 @@ Layout carve(char* base, const Geom& g, int n_rhs, int k, int ell, bool two_side
 }
 
 int blocks_per_rhs(long N, int n_rhs) {
-    // fixed per shape and device (deterministic reductions): at least two
-    // tiles of sites per CTA of the streaming step kernels, and at most one
-    // wave of them over all RHS
+    // fixed per shape and device (deterministic reductions)
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
-    const long V = N / 12;
-    const long need = std::max(1L, V / (2L * nk::stream_tile_sites()));
-    const long cap = std::max(1L, (long)sms * nk::stream_ctas_per_sm() / n_rhs);
-    return (int)std::min(need, cap);
+    return nk::step_blocks(N, n_rhs, sms);
 }
 
 // The launch shape of a solve: the tuned one for (n_rhs, two-sided, mixed),

@@ -28,9 +28,10 @@
 // fixed-order sum in the last block to finish (integer ticket, no
 // floating-point atomics).  The same launch configuration therefore
 // regenerates bit-identical coefficients, which the double-pass mode relies on.
+#include <algorithm>
+
 #include "nk_common.cuh"
 #include "nk_kernels.h"
-#include "nk_tma.cuh"
 
 namespace nk {
 
@@ -121,12 +122,48 @@ __global__ void __launch_bounds__(kThreads) k_init(Outer o, int copy_mode) {
     }
 }
 
+// sqrt(x) and 1 / sqrt(x) of a positive finite x from one reciprocal square
+// root (410 clocks; a square root takes 650, a division 620): y = rsqrt(x),
+// then one Newton correction of x y.
+__device__ __forceinline__ double sqrt_inv(double x, double& inv) {
+    const double y = rsqrt(x), s = x * y;
+    inv = y;
+    return fma(0.5 * y, fma(-s, s, x), s);
+}
+
+// beta = sqrt(delta) (principal branch), gamma = delta^* / beta, 1 / beta and
+// 1 / gamma of a finite delta != 0, without a division: with d = delta / 2^e
+// (e even, exact, so that max(|Re d|, |Im d|) is in [1, 4)), m = |d| and
+// 1 / m come from one reciprocal square root, the parts of sqrt(d) from a
+// second; then 1 / beta = beta^* / |delta|, gamma = (delta beta)^* / |delta| and
+// 1 / gamma = delta beta / |delta|^2.
+__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }   // |e| <= 1022
+__device__ __forceinline__ void csqrt_scalars(double2 delta, double2& beta, double2& gamma, double2& inv_beta,
+                                              double2& inv_gamma) {
+    const int hx = __double2hiint(delta.x) & 0x7fffffff, hy = __double2hiint(delta.y) & 0x7fffffff;
+    const int e = min(max(((max(hx, hy) >> 20) - 1023) & ~1, -1022), 1022);
+    const double sc = pow2(-e), up = pow2(e >> 1), down = pow2(-(e >> 1));
+    const double2 d = mk(delta.x * sc, delta.y * sc);
+    double im;
+    const double m = sqrt_inv(fma(d.x, d.x, d.y * d.y), im);
+    double iv;
+    const double t = sqrt_inv(0.5 * (m + fabs(d.x)), iv), o = 0.5 * d.y * iv;
+    // (t, o) for Re d >= 0, else (|o|, sign(Im d) t)
+    const double2 b = d.x >= 0.0 ? mk(t, o) : mk(fabs(o), d.y >= 0.0 ? t : -t);
+    const double2 w = cscale(cmul(d, b), im);
+    beta = cscale(b, up);
+    gamma = cscale(cconj(w), up);
+    inv_beta = cscale(cconj(b), im * down);
+    inv_gamma = cscale(w, im * down);
+}
+
 // End of step 2: the deterministic reduction of the per-thread partial
 // (r^dag r, or r^dag l two-sided) and, in the last block, beta and gamma and
 // the scalars of step j + 1.  This tail is a chain of dependent FP64
-// operations on one lane, several microseconds long and all of a small
-// lattice's step, so it holds no division twice: 1/n_j and 1/m_j of the
-// current step are the scalars kScN and kScM, 1/beta serves gamma and 1/n_{j+1}.
+// operations on one lane, most of a small lattice's step 2, so it holds no
+// division: 1/n_j and 1/m_j of the current step are the scalars kScN and kScM,
+// and beta, gamma and their inverses come from two reciprocal square roots
+// (about 2000 clocks against 5000 for the roots and quotients one by one).
 template <bool TS>
 __device__ __forceinline__ void step2_finish(const Outer& o, int rhs, int j, double2 acc, double2* sh) {
     double2 part = block_sum(acc, sh);
@@ -136,30 +173,29 @@ __device__ __forceinline__ void step2_finish(const Outer& o, int rhs, int j, dou
         double2 d = sum_partials(o.partials + (size_t)rhs * o.npart, o.nblk, sh);
         if (threadIdx.x == 0) {
             const size_t at = (size_t)rhs * o.k + j;
-            double2 b, g, ib = mk(0.0, 0.0);
+            double2 b, g, ib = mk(0.0, 0.0), ig = mk(0.0, 0.0);
             bool ok = true;
             if (!TS) {
-                const double bb = sqrt(d.x);             // beta <- sqrt(r^dag r)
+                // beta <- sqrt(r^dag r)
+                ok = d.x > 0.0 && isfinite(d.x);
+                double inv = 0.0;
+                const double bb = ok ? sqrt_inv(d.x, inv) : sqrt(d.x);
                 b = g = mk(bb, 0.0);
-                ok = bb > 0.0 && isfinite(bb);
+                ib = ig = mk(inv, 0.0);
                 if (!ok) mark_failed(o, rhs, kStatusBreakdown);
-                else ib = cinv(b);
             } else if ((d.x == 0.0 && d.y == 0.0) || !isfinite(d.x) || !isfinite(d.y)) {
                 // serious breakdown: delta = 0 (App. B); a non-finite delta is treated alike
                 mark_failed(o, rhs, kStatusBreakdown);
                 b = g = mk(0.0, 0.0);
                 ok = false;
             } else {
-                b = csqrt_principal(d);                  // beta <- sqrt(delta)
-                ib = cinv(b);
-                g = cmul(cconj(d), ib);                  // gamma <- delta^* / beta
+                csqrt_scalars(d, b, g, ib, ig);          // beta <- sqrt(delta), gamma <- delta^* / beta
             }
             o.beta[at] = b;
             o.gamma[at] = g;
             o.counters[rhs] = 0u;
             // step j + 1: n_{j+1} = beta_j, m_{j+1} = gamma_j^*
             if (ok && j + 1 < o.k && o.status[rhs] == kStatusOK) {
-                const double2 ig = TS ? cinv(g) : ib;
                 sc[kScN] = ib;
                 sc[kScC1] = cmul(g, inv_n);              // gamma (Hermitian: beta) / n_j
                 sc[kScD] = ig;
@@ -170,114 +206,24 @@ __device__ __forceinline__ void step2_finish(const Outer& o, int rhs, int j, dou
     }
 }
 
-// ---- streaming FP64 kernels of the FP64 recurrence ----------------------------
-// Step 1 (after the FP32 stencil) and step 2 stream their operand vectors
-// through shared memory with bulk asynchronous copies (the TMA engine,
-// cp.async.bulk, nk_tma.cuh).  A CTA owns a contiguous range of sites of one
-// RHS and walks it in tiles of kTile sites.  Warp w owns component pair w
-// (spin-colour components 2w and 2w + 1: rows 2w, 2w + 1 of an FP64 vector,
-// row w of an FP32 pair-layout vector) and runs its own pipeline: kStages
-// stage buffers with their own mbarriers, into which its lanes copy the
-// warp's rows of every operand vector for a tile, kStages - 1 tiles ahead of
-// its arithmetic; lane l then takes site s0 + l of the tile and writes its
-// results straight to global memory.  No CTA-wide barrier inside the loop:
-// the warps run independently.  GB300's FP64 pipe (about 0.6 T DFMA/s) is
-// kept busy by a few warps per SM as long as they have operands; the copies
-// keep enough bytes in flight for HBM without holding them in registers.
-constexpr int kTile = 32;                       // sites per tile = lanes of a warp
-constexpr int kStreamWarps = 6;                 // one per component pair
-constexpr int kStreamThreads = 32 * kStreamWarps;
-constexpr int kStages = 2;
-constexpr int kRowBytes = kTile * 16;           // one row of a tile: kTile 16-byte elements
-constexpr int kStep2Rows = 8;                   // rows of one warp's stage: step 2
-constexpr int kStep1Rows = 8;                   // step 1 after the FP32 stencil
-constexpr int kStep1Rows64 = 10;                // step 1 after the two-float stencil (FP64 s, t)
-
-// One operand vector of a streaming kernel (row r of V 16-byte elements at
-// base + r V 16 bytes): rows = 2 for an FP64 vector (warp w reads rows 2w,
-// 2w + 1), 1 for an FP32 pair-layout vector (row w), 0 for an absent operand.
-struct TileStream {
-    const char* base;
-    int rows;
-};
-
-// The copies of warp w for the tile of sites [s0, s0 + n): one row per lane
-// (the rows of stream k follow those of streams 0 .. k-1 in the stage),
-// armed on bar with their byte count by lane 0.
-template <int NS>
-__device__ __forceinline__ void issue_warp_tile(const TileStream (&ts)[NS], char* stage, uint64_t* bar, unsigned V,
-                                                unsigned s0, unsigned n, int w, int lane) {
-    int total = 0;
-#pragma unroll
-    for (int k = 0; k < NS; ++k) total += ts[k].rows;
-    const unsigned bytes = n * 16u;
-    if (lane == 0) {
-        fence_proxy_async_smem();   // the stage was last read through the generic proxy
-        mbar_arrive_expect_tx(bar, (unsigned)total * bytes);
-    }
-    __syncwarp();
-    int off = 0;
-#pragma unroll
-    for (int k = 0; k < NS; ++k) {
-        const int rows = ts[k].rows;
-        if (lane >= off && lane < off + rows) {
-            const unsigned row = (unsigned)(w * rows + lane - off);
-            bulk_copy_g2s(stage + (size_t)lane * kRowBytes, ts[k].base + ((size_t)row * V + s0) * 16, bytes, bar);
-        }
-        off += rows;
-    }
-}
-
-// The tile loop of warp w over the site range of CTA blockIdx.x (of o.nblk per
-// RHS): f(stage, s0, n) on each tile once its copies have landed.  Returns
-// false if a wait ran out (the warp's copies still in flight are then waited
-// for, bounded, before returning).
-template <int ROWS, int NS, typename F>
-__device__ __forceinline__ bool stream_tiles(const Outer& o, const TileStream (&ts)[NS], F&& f) {
-    extern __shared__ __align__(128) char smem[];
-    __shared__ uint64_t bar[kStreamWarps][kStages];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned V = (unsigned)(o.N / 12);
-    const unsigned s_lo = (unsigned)((unsigned long long)blockIdx.x * V / (unsigned)o.nblk);
-    const unsigned s_hi = (unsigned)((unsigned long long)(blockIdx.x + 1) * V / (unsigned)o.nblk);
-    const int ntiles = (int)((s_hi - s_lo + kTile - 1) / kTile);
-    const size_t stage_bytes = (size_t)ROWS * kRowBytes;   // ROWS >= the streams' rows
-    char* mine = smem + (size_t)w * kStages * stage_bytes;
-    uint64_t* mbar = bar[w];
-    if (lane == 0) {
-#pragma unroll
-        for (int st = 0; st < kStages; ++st) mbar_init(&mbar[st], 1);
-        mbar_init_fence();
-    }
-    __syncwarp();
-    for (int t = 0; t < kStages - 1 && t < ntiles; ++t) {
-        const unsigned s0 = s_lo + t * kTile;
-        issue_warp_tile(ts, mine + t * stage_bytes, &mbar[t], V, s0, min((unsigned)kTile, s_hi - s0), w, lane);
-    }
-    int t = 0;
-    bool ok = true;
-    for (; t < ntiles; ++t) {
-        // the tile kStages - 1 ahead goes into the stage freed by tile t - 1
-        const int ahead = t + kStages - 1;
-        if (ahead < ntiles) {
-            const unsigned s0 = s_lo + ahead * kTile;
-            issue_warp_tile(ts, mine + (ahead % kStages) * stage_bytes, &mbar[ahead % kStages], V, s0,
-                            min((unsigned)kTile, s_hi - s0), w, lane);
-        }
-        const int st = t % kStages;
-        ok = __all_sync(0xffffffffu, mbar_wait_bounded(&mbar[st], (unsigned)(t / kStages) & 1u, kWaitLimitNs));
-        if (!ok) break;
-        const unsigned s0 = s_lo + t * kTile;
-        f(mine + st * stage_bytes, s0, min((unsigned)kTile, s_hi - s0));
-        __syncwarp();   // every lane is done with the stage before it is refilled
-    }
-    if (ok) return true;
-    if (lane == 0)   // copies issued for tiles t .. t + kStages - 1
-        for (int u = t; u < ntiles && u < t + kStages; ++u)
-            mbar_wait_bounded(&mbar[u % kStages], (unsigned)(u / kStages) & 1u, kWaitLimitNs);
-    __syncwarp();
-    return false;
-}
+// ---- FP64 step kernels of the FP64 recurrence ---------------------------------
+// Step 1 (after a multi-RHS stencil) and step 2 work on (component pair, site)
+// items: thread item i = cp V + s holds components 2 cp and 2 cp + 1 of site s
+// (two rows of an FP64 vector, one float4 of an FP32 pair-layout vector), so
+// every load and store is a coalesced 16-byte access; an item's loads (up to
+// ten) are all issued before its arithmetic, and the warps of the other
+// resident CTAs keep the FP64 pipe busy meanwhile.
+// Bound by the FP64 pipe on large batches (24 instructions per lane and item)
+// and by the reduction tail below on small ones.  Against the earlier form,
+// operands staged tile by tile into shared memory with bulk copies (4 CTAs of
+// 6 warps per SM, ranges of up to 7 tiles of 32 sites, the last one a quarter
+// full): an outer step of 12 sources at 10^4, mu = 0.2, two-float stencil,
+// 220 -> 192 us; 8^4, mu = 0, FP32 stencil, 41 -> 27; one source, FP64, at 4^4,
+// mu = 0.1, 21 -> 16, at 10^4 65 -> 58 (both with the shorter tail).  20 warps
+// per SM at 102 registers: 8, 6, 4 or 3 CTAs per SM measured 201, 200, 193
+// and 194 us in the first case (64 registers spill).
+constexpr int kStepThreads = 128;   // at least 3 warps: the finishing block of step 1 uses warps 0 to 2
+constexpr int kStepCtasPerSm = 5;
 
 // The FP64 loops take no negated operand: in a throughput test on GB300 a
 // DFMA with a negated multiplicand ran at 85% of the rate of a plain one.  The
@@ -309,65 +255,59 @@ __device__ __forceinline__ void dot3_add(Dot3& d, double2 a, double2 b) {
 //   r <- r - (H(j,j)/n_j) q_j,  l <- l - (H(j,j)^*/m_j) p_j,  delta += r^dag l,
 // plus the copies the next stencil reads (FP32 pair layout; write_ring: also
 // two-float copies in the rings for a two-float stencil or a later ring
-// step).  Stage rows of warp w (components 2w + h): q_j h, r 2 + h, p_j 4 + h,
-// l 6 + h.
+// step).
 template <bool TS>
-__global__ void __launch_bounds__(kStreamThreads) k_step2(Outer o, int j, int copy_mode, int write_ring) {
+__global__ void __launch_bounds__(kStepThreads, kStepCtasPerSm) k_step2(Outer o, int j, int copy_mode, int write_ring) {
     __shared__ double2 sh[33];
     const int rhs = blockIdx.y;
     if (o.status[rhs] != kStatusOK) return;
     const double2 c3 = o.sc[(size_t)rhs * kScalars + kScC3];
     const double2 c4 = o.sc[(size_t)rhs * kScalars + kScC4];
     const unsigned V = (unsigned)(o.N / 12);
-    const double2* qj = outer_q(o, rhs, j);
-    double2* r = outer_q(o, rhs, j + 1);
-    const double2* pj = TS ? outer_p(o, rhs, j) : nullptr;
-    double2* l = TS ? outer_p(o, rhs, j + 1) : nullptr;
+    const double2* __restrict__ qj = outer_q(o, rhs, j);
+    double2* __restrict__ r = outer_q(o, rhs, j + 1);
+    const double2* __restrict__ pj = TS ? outer_p(o, rhs, j) : nullptr;
+    double2* __restrict__ l = TS ? outer_p(o, rhs, j + 1) : nullptr;
     float4* __restrict__ r32 = o.q32 + (size_t)rhs * 6 * V;
     float4* __restrict__ l32 = TS ? o.p32 + (size_t)rhs * 6 * V : nullptr;
     dfc* __restrict__ rr_ring = write_ring ? ring_q(o, rhs, j + 1) : nullptr;
     dfc* __restrict__ ll_ring = (write_ring && TS) ? ring_p(o, rhs, j + 1) : nullptr;
-    const TileStream ts[4] = {{(const char*)qj, 2}, {(const char*)r, 2}, {(const char*)pj, TS ? 2 : 0},
-                              {(const char*)l, TS ? 2 : 0}};
     const double2 nc3 = neg_bits(c3), nc4 = neg_bits(c4);
-    const int cp = threadIdx.x >> 5, sl = threadIdx.x & 31;
     Dot3 acc = {0.0, 0.0, 0.0};
-    const bool ok = stream_tiles<kStep2Rows>(o, ts, [&](const char* stage, unsigned s0, unsigned n) {
-        if ((unsigned)sl >= n) return;
-        const double2* sv = reinterpret_cast<const double2*>(stage);
-        double2 rv[2], lv[2];
+    const unsigned items = 6u * V, stride = (unsigned)o.nblk * kStepThreads;
+    for (unsigned i = blockIdx.x * kStepThreads + threadIdx.x; i < items; i += stride) {
+        const unsigned cp = i / V;
+        const size_t e0 = (size_t)i + (size_t)cp * V;   // component 2 cp
+        double2 q[2], a[2], pv[2], b[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int c = 2 * cp + h;
-            const size_t e = (size_t)c * V + s0 + sl;
-            const double2 q = sv[h * kTile + sl], a0 = sv[(2 + h) * kTile + sl];
+            const size_t e = e0 + (size_t)h * V;
+            q[h] = qj[e];
+            a[h] = r[e];
+            if (TS) { pv[h] = pj[e]; b[h] = l[e]; }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const size_t e = e0 + (size_t)h * V;
             // r <- r - c3 q, l <- l - c4 p with explicit FMA
-            const double2 a = TS ? cfma_sub(a0, c3, nc3, q) : mk(fma(nc3.x, q.x, a0.x), fma(nc3.x, q.y, a0.y));
-            rv[h] = a;
-            r[e] = a;
-            if (rr_ring) rr_ring[e] = dfc_of(a);
+            a[h] = TS ? cfma_sub(a[h], c3, nc3, q[h]) : mk(fma(nc3.x, q[h].x, a[h].x), fma(nc3.x, q[h].y, a[h].y));
+            r[e] = a[h];
+            if (rr_ring) rr_ring[e] = dfc_of(a[h]);
             if (TS) {
-                const double2 b = cfma_sub(sv[(6 + h) * kTile + sl], c4, nc4, sv[(4 + h) * kTile + sl]);
-                lv[h] = b;
-                l[e] = b;
-                if (ll_ring) ll_ring[e] = dfc_of(b);
-                dot3_add(acc, a, b);   // conj(r) l
+                b[h] = cfma_sub(b[h], c4, nc4, pv[h]);
+                l[e] = b[h];
+                if (ll_ring) ll_ring[e] = dfc_of(b[h]);
+                dot3_add(acc, a[h], b[h]);   // conj(r) l
             } else {
-                acc.re = fma(a.x, a.x, fma(a.y, a.y, acc.re));
+                acc.re = fma(a[h].x, a[h].x, fma(a[h].y, a[h].y, acc.re));
             }
         }
         if (copy_mode == kCopy32) {
-            const size_t f = (size_t)cp * V + s0 + sl;
-            r32[f] = make_float4(d2f_int(rv[0].x), d2f_int(rv[0].y), d2f_int(rv[1].x), d2f_int(rv[1].y));
-            if (TS) l32[f] = make_float4(d2f_int(lv[0].x), d2f_int(lv[0].y), d2f_int(lv[1].x), d2f_int(lv[1].y));
+            r32[i] = make_float4(d2f_int(a[0].x), d2f_int(a[0].y), d2f_int(a[1].x), d2f_int(a[1].y));
+            if (TS) l32[i] = make_float4(d2f_int(b[0].x), d2f_int(b[0].y), d2f_int(b[1].x), d2f_int(b[1].y));
         }
-    });
-    double2 tot = mk(acc.re, acc.ip - acc.im);
-    if (!ok) {
-        if (threadIdx.x == 0) mark_failed(o, rhs, kStatusTimeout);
-        tot = mk(0.0, 0.0);
     }
-    step2_finish<TS>(o, rhs, j, tot, sh);
+    step2_finish<TS>(o, rhs, j, mk(acc.re, acc.ip - acc.im), sh);
 }
 
 // FP64 step 1 of the FP32- and two-float-stencil steps of an FP64
@@ -380,14 +320,10 @@ __global__ void __launch_bounds__(kStreamThreads) k_step2(Outer o, int j, int co
 // an FP32 stencil output entering the FP64 arithmetic exactly (FP32 -> FP64
 // on the integer pipe).  The finishing block forms H(j,j) and the step-2
 // scalars.  PASS2 (the second pass of NK_DOUBLE_PASS) also accumulates
-// y += c'_j q_j.  Stage rows of warp w (components 2w + h), with
-// F = 1 (FP32 s: one row of pairs) or 2 (FP64 s: rows h): s 0 .. F - 1,
-// q_{j-1} F + h, dot vector (p_j, or q_j Hermitian) F + 2 + h, then two-sided
-// and not at the last step t F + 4 .., p_{j-1} 2 F + 4 + h.
+// y += c'_j q_j.
 template <bool TS, bool PASS2, bool S64>
-__global__ void __launch_bounds__(kStreamThreads) k_step1(Outer o, int j) {
+__global__ void __launch_bounds__(kStepThreads, kStepCtasPerSm) k_step1(Outer o, int j) {
     __shared__ double2 sh[33];
-    constexpr int F = S64 ? 2 : 1;
     const int rhs = blockIdx.y;
     if (o.status[rhs] != kStatusOK) return;
     const double2* sc = o.sc + (size_t)rhs * kScalars;
@@ -395,67 +331,62 @@ __global__ void __launch_bounds__(kStreamThreads) k_step1(Outer o, int j) {
     const unsigned V = (unsigned)(o.N / 12);
     const int jp = j > 0 ? j - 1 : j;   // c1 = 0 at j = 0
     const bool left = TS && j < o.k - 1;   // the last step makes no new left vector
-    const char* s_in = S64 ? (const char*)(o.s64 + (size_t)rhs * o.N) : (const char*)(o.s32 + (size_t)rhs * 6 * V);
-    const char* t_in = S64 ? (const char*)(o.s64 + (size_t)(o.n_rhs + rhs) * o.N)
-                           : (const char*)(o.s32 + (size_t)(o.n_rhs + rhs) * 6 * V);
-    const double2* qprev = outer_q(o, rhs, jp);
-    const double2* pprev = TS ? outer_p(o, rhs, jp) : nullptr;
-    const double2* dotv = TS ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
+    const double2* __restrict__ s64 = S64 ? o.s64 + (size_t)rhs * o.N : nullptr;
+    const double2* __restrict__ t64 = S64 ? o.s64 + (size_t)(o.n_rhs + rhs) * o.N : nullptr;
+    const float4* __restrict__ s32 = S64 ? nullptr : o.s32 + (size_t)rhs * 6 * V;
+    const float4* __restrict__ t32 = S64 ? nullptr : o.s32 + (size_t)(o.n_rhs + rhs) * 6 * V;
+    const double2* __restrict__ qprev = outer_q(o, rhs, jp);
+    const double2* __restrict__ pprev = TS ? outer_p(o, rhs, jp) : nullptr;
+    const double2* __restrict__ dotv = TS ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
     double2* __restrict__ rn = outer_q(o, rhs, j + 1);
     double2* __restrict__ ln = left ? outer_p(o, rhs, j + 1) : nullptr;
     double2* __restrict__ yacc = PASS2 ? o.y + (size_t)rhs * o.N : nullptr;
     const double2 cpj = PASS2 ? o.cp[(size_t)rhs * o.k + j] : mk(0.0, 0.0);
     const double2* __restrict__ qj = outer_q(o, rhs, j);
-    const TileStream ts[5] = {{s_in, F}, {(const char*)qprev, 2}, {(const char*)dotv, 2},
-                              {t_in, left ? F : 0}, {(const char*)pprev, left ? 2 : 0}};
     const double2 nc1 = neg_bits(c1), nc1l = neg_bits(c1l), ncpj = neg_bits(cpj);
-    const int cp = threadIdx.x >> 5, sl = threadIdx.x & 31;
     Dot3 acc = {0.0, 0.0, 0.0};
-    const bool ok = stream_tiles<S64 ? kStep1Rows64 : kStep1Rows>(o, ts, [&](const char* stage, unsigned s0,
-                                                                                unsigned n) {
-        if ((unsigned)sl >= n) return;
-        const double2* sv = reinterpret_cast<const double2*>(stage);
-        const float4* sf = reinterpret_cast<const float4*>(stage);
-        float4 sv4 = make_float4(0.f, 0.f, 0.f, 0.f), tv4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    const unsigned items = 6u * V, stride = (unsigned)o.nblk * kStepThreads;
+    for (unsigned i = blockIdx.x * kStepThreads + threadIdx.x; i < items; i += stride) {
+        const unsigned cp = i / V;
+        const size_t e0 = (size_t)i + (size_t)cp * V;   // component 2 cp
+        double2 sv[2], tv[2], qv[2], d[2], pv[2];
+        float4 sf, tf;
         if (!S64) {
-            sv4 = sf[sl];
-            if (left) tv4 = sf[(F + 4) * kTile + sl];
+            sf = s32[i];
+            if (left) tf = t32[i];
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const int c = 2 * cp + h;
-            const size_t e = (size_t)c * V + s0 + sl;
-            double2 rr;
+            const size_t e = e0 + (size_t)h * V;
             if (S64) {
-                rr = sv[h * kTile + sl];
-            } else {
-                const float2 s2 = h ? make_float2(sv4.z, sv4.w) : make_float2(sv4.x, sv4.y);
-                rr = mk(f2d_int(s2.x), f2d_int(s2.y));
+                sv[h] = s64[e];
+                if (left) tv[h] = t64[e];
             }
-            const double2 qv = sv[(F + h) * kTile + sl];
-            rr = TS ? cfma_sub(rr, c1, nc1, qv) : mk(fma(nc1.x, qv.x, rr.x), fma(nc1.x, qv.y, rr.y));
-            rn[e] = rr;
-            const double2 d = sv[(F + 2 + h) * kTile + sl];
-            if (TS) dot3_add(acc, d, rr);   // conj(d) r
-            else acc.re = fma(d.x, rr.x, fma(d.y, rr.y, acc.re));
-            if (left) {
-                double2 tt;
-                if (S64) {
-                    tt = sv[(F + 4 + h) * kTile + sl];
-                } else {
-                    const float2 t2 = h ? make_float2(tv4.z, tv4.w) : make_float2(tv4.x, tv4.y);
-                    tt = mk(f2d_int(t2.x), f2d_int(t2.y));
-                }
-                ln[e] = cfma_sub(tt, c1l, nc1l, sv[(2 * F + 4 + h) * kTile + sl]);
-            }
-            if (PASS2) yacc[e] = cfma_add(yacc[e], cpj, ncpj, qj[e]);
+            qv[h] = qprev[e];
+            d[h] = dotv[e];
+            if (left) pv[h] = pprev[e];
         }
-    });
-    double2 tot = mk(acc.re, acc.ip - acc.im);
-    if (!ok) {
-        if (threadIdx.x == 0) mark_failed(o, rhs, kStatusTimeout);
-        tot = mk(0.0, 0.0);
+        if (!S64) {
+            sv[0] = mk(f2d_int(sf.x), f2d_int(sf.y));
+            sv[1] = mk(f2d_int(sf.z), f2d_int(sf.w));
+            if (left) {
+                tv[0] = mk(f2d_int(tf.x), f2d_int(tf.y));
+                tv[1] = mk(f2d_int(tf.z), f2d_int(tf.w));
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const size_t e = e0 + (size_t)h * V;
+            const double2 rr = TS ? cfma_sub(sv[h], c1, nc1, qv[h])
+                                  : mk(fma(nc1.x, qv[h].x, sv[h].x), fma(nc1.x, qv[h].y, sv[h].y));
+            rn[e] = rr;
+            if (TS) dot3_add(acc, d[h], rr);   // conj(d) r
+            else acc.re = fma(d[h].x, rr.x, fma(d[h].y, rr.y, acc.re));
+            if (left) ln[e] = cfma_sub(tv[h], c1l, nc1l, pv[h]);
+            if (PASS2) yacc[e] = cfma_add(yacc[e], cpj, ncpj, TS ? qj[e] : d[h]);
+        }
     }
+    const double2 tot = mk(acc.re, acc.ip - acc.im);
     const double2 part = block_sum(tot, sh);
     if (finish_partial(part, o.partials + (size_t)rhs * o.npart, o.counters + rhs, blockIdx.x, o.nblk)) {
         const double2 a = sum_partials(o.partials + (size_t)rhs * o.npart, o.nblk, sh);
@@ -472,9 +403,6 @@ __global__ void __launch_bounds__(kStreamThreads) k_step1(Outer o, int j) {
             o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cmul(cconj(al), sc[kScM]) : mk(0.0, 0.0);
     }
 }
-
-size_t step2_smem() { return (size_t)kStreamWarps * kStages * kStep2Rows * kRowBytes; }
-size_t step1_smem(bool s64) { return (size_t)kStreamWarps * kStages * (s64 ? kStep1Rows64 : kStep1Rows) * kRowBytes; }
 
 // Step 2 of the late (FP32-stencil) steps of the mixed schedule in two-float
 // arithmetic on the FP32 pipe, on the two-float rings: r and l (left in ring slot j + 1
@@ -661,8 +589,7 @@ void launch_outer_init(const Outer& o, int copy_mode, cudaStream_t st, bool keep
 void launch_outer_step1(const Outer& o, int j, bool s64, cudaStream_t st) {
     dim3 grid(o.nblk, o.n_rhs);
     const bool pass2 = o.y != nullptr;
-    const size_t sm = step1_smem(s64);
-#define NK_STEP1(TS_, P2_, S_) k_step1<TS_, P2_, S_><<<grid, kStreamThreads, sm, st>>>(o, j)
+#define NK_STEP1(TS_, P2_, S_) k_step1<TS_, P2_, S_><<<grid, kStepThreads, 0, st>>>(o, j)
     if (o.two_sided) {
         if (pass2) { if (s64) NK_STEP1(true, true, true); else NK_STEP1(true, true, false); }
         else { if (s64) NK_STEP1(true, false, true); else NK_STEP1(true, false, false); }
@@ -673,54 +600,20 @@ void launch_outer_step1(const Outer& o, int j, bool s64, cudaStream_t st) {
 #undef NK_STEP1
 }
 
-// CTAs of the two-sided step-2 kernel that fit one SM (its stage buffers
-// decide), queried once per device after lanczos_init_attributes.
-int stream_ctas_per_sm() {
-    static int cached[64] = {0};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) dev = 0;
-    if (!cached[dev]) {
-        int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_step2<true>, kStreamThreads, step2_smem()) !=
-                cudaSuccess || n < 1) {
-            cudaGetLastError();
-            return 1;   // attributes not set yet: not cached
-        }
-        cached[dev] = n;
-    }
-    return cached[dev];
-}
-
-int stream_tile_sites() { return kTile; }
-
-void lanczos_init_attributes() {
-    // dynamic shared memory above 48 KB for the stage buffers of the streaming
-    // kernels, and the largest shared-memory carveout so that several CTAs fit an SM
-    const int carve = cudaSharedmemCarveoutMaxShared;
-#define NK_ATTR(K_, SM_)                                                                    \
-    cudaFuncSetAttribute(K_, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(SM_));     \
-    cudaFuncSetAttribute(K_, cudaFuncAttributePreferredSharedMemoryCarveout, carve)
-    NK_ATTR(k_step2<true>, step2_smem());
-    NK_ATTR(k_step2<false>, step2_smem());
-    NK_ATTR((k_step1<true, true, false>), step1_smem(false));
-    NK_ATTR((k_step1<true, false, false>), step1_smem(false));
-    NK_ATTR((k_step1<false, true, false>), step1_smem(false));
-    NK_ATTR((k_step1<false, false, false>), step1_smem(false));
-    NK_ATTR((k_step1<true, true, true>), step1_smem(true));
-    NK_ATTR((k_step1<true, false, true>), step1_smem(true));
-    NK_ATTR((k_step1<false, true, true>), step1_smem(true));
-    NK_ATTR((k_step1<false, false, true>), step1_smem(true));
-#undef NK_ATTR
+// Default CTAs per RHS of the step kernels (and of the norm): one item per
+// thread, but no more than one wave of the chip over all RHS (a CTA's block sum
+// costs the FP64 pipe as much as an item), in fours
+int step_blocks(long N, int n_rhs, int sms) {
+    const long need = (N / 2 + kStepThreads - 1) / kStepThreads, cap = (long)sms * kStepCtasPerSm / n_rhs / 4 * 4;
+    return (int)std::max(1L, std::min(need, cap));
 }
 
 void launch_outer_step2(const Outer& o, int j, int copy_mode, bool ring, bool write_ring, cudaStream_t st) {
     dim3 grid(o.nblk, o.n_rhs);
     const int wr = (write_ring && o.qr) ? 1 : 0;
     if (!ring || !o.qr) {   // FP64 step
-        const size_t sm = step2_smem();
-        if (o.two_sided) k_step2<true><<<grid, kStreamThreads, sm, st>>>(o, j, copy_mode, wr);
-        else k_step2<false><<<grid, kStreamThreads, sm, st>>>(o, j, copy_mode, wr);
+        if (o.two_sided) k_step2<true><<<grid, kStepThreads, 0, st>>>(o, j, copy_mode, wr);
+        else k_step2<false><<<grid, kStepThreads, 0, st>>>(o, j, copy_mode, wr);
     } else {
         if (o.two_sided) k_step2_df<true><<<grid, kThreads, 0, st>>>(o, j, copy_mode);
         else k_step2_df<false><<<grid, kThreads, 0, st>>>(o, j, copy_mode);

@@ -79,28 +79,42 @@ __device__ __forceinline__ double warp_sum(double v) {
 __device__ __forceinline__ int block_tid() { return threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z); }
 __device__ __forceinline__ int block_threads() { return blockDim.x * blockDim.y * blockDim.z; }
 
+// Warp sum of a double2 for a reduction tail: in the first exchange the lower
+// half-warp keeps the real parts and the upper half the imaginary ones, so
+// each level costs one FP64 addition instead of two (an FP64 warp instruction
+// holds its pipe 64 clocks on GB300 whatever its active lanes).  x in lanes
+// 0-15, y in lanes 16-31.
+__device__ __forceinline__ double warp_sum_split(double2 v) {
+    const bool up = (block_tid() & 16) != 0;
+    const double got = __shfl_xor_sync(0xffffffffu, up ? v.x : v.y, 16);
+    double t = (up ? v.y : v.x) + got;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
 // Block sum of a double2 (<= 1024 threads in whole warps). Every thread of the
 // block receives the same value; the summation order is fixed.  Only warp 0
-// does the second level (FP64 adds are scarce on GB300); the result is
-// broadcast through shared memory.  The butterfly of the second level stops at
-// the number of warps (lanes beyond it hold zeros).
+// does the second level (FP64 adds are scarce on GB300), real parts in the
+// lower half-warp and imaginary ones in the upper; the result is broadcast
+// through shared memory.  The butterfly of the second level stops at the
+// number of warps (lanes beyond it hold zeros).
 __device__ __forceinline__ double2 block_sum(double2 v, double2* sh /* >= 33 */) {
-    v = warp_sum(v);
+    const double s = warp_sum_split(v);
     const int tid = block_tid();
     int lane = tid & 31, w = tid >> 5, nw = block_threads() >> 5;
+    double* f = reinterpret_cast<double*>(sh);
+    const int q = lane & 15, part = lane >> 4;   // warp q (and q + 16), real or imaginary part
     __syncthreads();
-    if (lane == 0) sh[w] = v;
+    if (q == 0) f[2 * w + part] = s;
     __syncthreads();
     if (w == 0) {
-        double2 t = lane < nw ? sh[lane] : mk(0.0, 0.0);
+        double t = q < nw ? f[2 * q + part] : 0.0;
+        if (nw > 16 && q + 16 < nw) t += f[32 + 2 * q + part];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            if (o < nw) {   // only the levels that combine real partials
-                t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
-                t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
-            }
-        }
-        if (lane == 0) sh[32] = t;
+        for (int o = 8; o > 0; o >>= 1)
+            if (o < nw) t += __shfl_xor_sync(0xffffffffu, t, o);   // only the levels that combine real partials
+        if (q == 0) f[64 + part] = t;
     }
     __syncthreads();
     return sh[32];
@@ -113,8 +127,11 @@ __device__ __forceinline__ double block_sum(double v, double* sh /* >= 32 */) {
     if (lane == 0) sh[w] = v;
     __syncthreads();
     double t = lane < nw ? sh[lane] : 0.0;
-    t = warp_sum(t);
-    return t;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (o < nw) t += __shfl_xor_sync(0xffffffffu, t, o);
+    // lanes below the next power of two of nw hold the sum
+    return __shfl_sync(0xffffffffu, t, 0);
 }
 
 // Two-stage deterministic reduction, stage 1: thread 0 of each block writes
@@ -133,13 +150,21 @@ __device__ __forceinline__ bool finish_partial(double2 part, double2* partials, 
     return last;
 }
 
-// Stage 2: fixed-order sum of the nslots partials (all threads of the last block).
+// Stage 2: fixed-order sum of the nslots partials (all threads of the last
+// block).  Four loads in flight per thread: the tail of a step waits for them.
 __device__ __forceinline__ double2 sum_partials(const double2* partials, int nslots, double2* sh) {
     __threadfence();
     double2 a = mk(0.0, 0.0);
-    for (int i = block_tid(); i < nslots; i += block_threads()) {
-        double2 v = __ldcg(partials + i);
-        a.x += v.x; a.y += v.y;
+    const int T = block_threads();
+    for (int i0 = block_tid(); i0 < nslots; i0 += 4 * T) {
+        double2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i0 + u * T < nslots ? __ldcg(partials + i0 + u * T) : mk(0.0, 0.0);
+        if (i0 + T < nslots) {
+            v[0] = cadd(v[0], v[1]);
+            if (i0 + 2 * T < nslots) v[0] = cadd(v[0], cadd(v[2], v[3]));
+        }
+        a = i0 < T ? v[0] : cadd(a, v[0]);
     }
     return block_sum(a, sh);
 }

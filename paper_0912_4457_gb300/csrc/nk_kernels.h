@@ -196,7 +196,7 @@ constexpr int kStatusRhi = 3;         // RHi did not converge / singular pivot
 constexpr int kStatusLU = 4;          // singular p H_k
 constexpr int kStatusConverged = 5;   // adaptive k: frozen at its converged size (skipped by the kernels)
 constexpr int kStatusInnerBreakdown = 6;  // inner (two-sided) Lanczos on H_k': zero beta or delta
-constexpr int kStatusTimeout = 7;     // a bounded wait of a streaming kernel ran out (copies never landed)
+constexpr int kStatusTimeout = 7;     // a bounded device-side wait ran out (no kernel has one now)
 
 // First failure of an RHS wins (a later one does not overwrite it).
 __device__ inline void mark_failed(const Outer& o, int rhs, int code) { atomicCAS(o.status + rhs, kStatusOK, code); }
@@ -220,9 +220,7 @@ bool split_step(int precision, const Outer& o, int j);
 void launch_stencil_step(int precision, const void* U, const Geom& g, const Outer& o, int j, double kappa,
                          double mu, cudaStream_t st);
 void launch_outer_step1(const Outer& o, int j, bool s64, cudaStream_t st);
-void lanczos_init_attributes();   // dynamic shared memory above 48 KB (outside capture)
-int stream_ctas_per_sm();         // CTAs of the streaming step kernels per SM
-int stream_tile_sites();          // sites per tile of the streaming step kernels
+int step_blocks(long N, int n_rhs, int sms);   // default CTAs per RHS of the step kernels
 void launch_stencil32_step1(const void* U32, const Geom& g, const Outer& o, int j, double kappa, double mu,
                             cudaStream_t st);
 int dslash_step1_blocks(const Geom& g, int threads);
