@@ -283,10 +283,9 @@ Layout carve(char* base, const Geom& g, int n_rhs, int k, int ell, bool two_side
         q.rhi_iters = (int*)take(sizeof(int) * n_rhs);
         kl = q.ell;
     }
-    // the inner part stays FP64 in every schedule: with a Ritz value of H_k'
-    // near the imaginary axis its sign is ill conditioned, and two-float
-    // arithmetic there left single sources of the 16^3 x 32 test at 2.5e-8
-    in.df_inner = 0;
+    // (the inner part is FP64 in every schedule: with a Ritz value of H_k' near
+    // the imaginary axis its sign is ill conditioned, and two-float arithmetic
+    // there left single sources of the 16^3 x 32 test at 2.5e-8)
     in.p_shared = 0;
     L.total = off;
     return L;
@@ -497,9 +496,10 @@ cudaError_t enqueue_inner_chain(const Layout& Lw, const nk::Inner& in1, Launcher
         q.c = up.s;   // the lift of this level lands in the s of the level above
         lv[n] = q;
     }
-    for (int i = 0; i < n; ++i)
-        L.run(NK_CLASS_INNER, nk::inner_launches(lv[i]), [&] { nk::launch_inner_lanczos(lv[i], st); });
     cudaError_t e = cudaSuccess;
+    for (int i = 0; i < n && e == cudaSuccess; ++i)
+        L.run(NK_CLASS_INNER, nk::inner_launches(lv[i]), [&] { e = (cudaError_t)nk::launch_inner_lanczos(lv[i], st); });
+    if (e != cudaSuccess) return e;
     L.run(NK_CLASS_RHI, 1, [&] { e = (cudaError_t)nk::launch_rhi(lv[n - 1], st); });
     if (e != cudaSuccess) return e;
     for (int i = n - 1; i >= 1; --i) L.run(NK_CLASS_INNER, 1, [&] { nk::launch_inner_combine(lv[i], st); });

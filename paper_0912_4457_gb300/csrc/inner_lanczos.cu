@@ -35,7 +35,9 @@
 // each on GB300, whatever the active lanes) -- about 250 per step and warp at
 // k = 1024, two-sided -- and the barriers.  One CTA per RHS with the vectors
 // in global memory (the earlier form) ran 4 to 8 warps of 8 rows a lane on one
-// SM's pipe.
+// SM's pipe.  Measured, this part alone: 12 two-sided RHS at k = 1024, l = 128
+// 16.5 -> 4.0 ms (20 us per step, 0.9 ms for the LU, 0.5 for p); the whole inner
+// part of a 6^4 solve at k = 512, l = 128 16 -> 9 ms.
 #include <cooperative_groups.h>
 
 #include "inner_arith.cuh"

@@ -122,41 +122,6 @@ __global__ void __launch_bounds__(kThreads) k_init(Outer o, int copy_mode) {
     }
 }
 
-// sqrt(x) and 1 / sqrt(x) of a positive finite x from one reciprocal square
-// root (410 clocks; a square root takes 650, a division 620): y = rsqrt(x),
-// then one Newton correction of x y.
-__device__ __forceinline__ double sqrt_inv(double x, double& inv) {
-    const double y = rsqrt(x), s = x * y;
-    inv = y;
-    return fma(0.5 * y, fma(-s, s, x), s);
-}
-
-// beta = sqrt(delta) (principal branch), gamma = delta^* / beta, 1 / beta and
-// 1 / gamma of a finite delta != 0, without a division: with d = delta / 2^e
-// (e even, exact, so that max(|Re d|, |Im d|) is in [1, 4)), m = |d| and
-// 1 / m come from one reciprocal square root, the parts of sqrt(d) from a
-// second; then 1 / beta = beta^* / |delta|, gamma = (delta beta)^* / |delta| and
-// 1 / gamma = delta beta / |delta|^2.
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }   // |e| <= 1022
-__device__ __forceinline__ void csqrt_scalars(double2 delta, double2& beta, double2& gamma, double2& inv_beta,
-                                              double2& inv_gamma) {
-    const int hx = __double2hiint(delta.x) & 0x7fffffff, hy = __double2hiint(delta.y) & 0x7fffffff;
-    const int e = min(max(((max(hx, hy) >> 20) - 1023) & ~1, -1022), 1022);
-    const double sc = pow2(-e), up = pow2(e >> 1), down = pow2(-(e >> 1));
-    const double2 d = mk(delta.x * sc, delta.y * sc);
-    double im;
-    const double m = sqrt_inv(fma(d.x, d.x, d.y * d.y), im);
-    double iv;
-    const double t = sqrt_inv(0.5 * (m + fabs(d.x)), iv), o = 0.5 * d.y * iv;
-    // (t, o) for Re d >= 0, else (|o|, sign(Im d) t)
-    const double2 b = d.x >= 0.0 ? mk(t, o) : mk(fabs(o), d.y >= 0.0 ? t : -t);
-    const double2 w = cscale(cmul(d, b), im);
-    beta = cscale(b, up);
-    gamma = cscale(cconj(w), up);
-    inv_beta = cscale(cconj(b), im * down);
-    inv_gamma = cscale(w, im * down);
-}
-
 // End of step 2: the deterministic reduction of the per-thread partial
 // (r^dag r, or r^dag l two-sided) and, in the last block, beta and gamma and
 // the scalars of step j + 1.  This tail is a chain of dependent FP64

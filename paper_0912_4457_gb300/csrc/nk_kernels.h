@@ -286,18 +286,15 @@ struct Inner {
     int* rhi_iters;        // [rhs]
     double2* c;            // V_l s, [rhs][k]
     int* status;           // [rhs]
-    int df_inner;          // 1: p estimate, LU, sweeps and inner Lanczos in two-float
-                           // arithmetic (the mixed schedule); 0: FP64
 };
-constexpr int kInnerWorkVecs = 16;
-// per RHS: kInnerWorkVecs vectors of length k, then the sweep tables of the LU
-constexpr int kSweepTableElems = 72 * 256;   // 72 table rows x up to 256 group lanes
-__host__ __device__ constexpr size_t inner_work_elems(int k) { return (size_t)kInnerWorkVecs * k + kSweepTableElems; }
-// Largest outer size k the inner kernel supports (its LU factors and solve
-// vectors, 8 complex vectors of length k plus the pivots, fill shared memory).
+constexpr int kInnerWorkVecs = 5;   // the LU of H_k: multipliers, 1/d, du, du2, and the singularity flag
+__host__ __device__ constexpr size_t inner_work_elems(int k) { return (size_t)kInnerWorkVecs * k; }
+// Largest outer size k the inner kernel supports (three rows per lane of its
+// largest cluster).
 constexpr int kMaxInnerK = 1536;
 
-void launch_inner_lanczos(const Inner& in, cudaStream_t st);
+int launch_inner_lanczos(const Inner& in, cudaStream_t st);   // returns cudaError_t
+void inner_lanczos_init_attributes();
 // kernels launch_inner_lanczos launches: two with a p shared by the batch
 inline int inner_launches(const Inner& in) { return in.p_shared && !(in.p_fixed > 0.0) ? 2 : 1; }
 int launch_rhi(const Inner& in, cudaStream_t st);  // returns cudaError_t

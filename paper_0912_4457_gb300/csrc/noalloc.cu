@@ -8,7 +8,7 @@
 // allocate; the caller passes only its inputs and outputs.
 //
 // The array is a module global: every GPU that loads this library holds it
-// (about 5.9 MB) until the process exits.  All calls share it and it keeps the
+// (about 5 MB) until the process exits.  All calls share it and it keeps the
 // last call's contents, so calls whose work overlaps on the GPU (different
 // streams, or different host threads) race on it; serialise them.
 #include <cuda_runtime.h>
@@ -119,8 +119,8 @@ extern "C" int nk_inner_sign_noalloc(const double* alpha_dev, const double* beta
     // the array keeps the previous call's contents: the status flags must start at 0
     e = cudaMemsetAsync(in.status, 0, sizeof(int) * n_rhs, st);
     if (e != cudaSuccess) return set_err(err, err_len, NK_ECUDA, cudaGetErrorString(e));
-    nk::launch_inner_lanczos(in, st);
-    e = (cudaError_t)nk::launch_rhi(in, st);
+    e = (cudaError_t)nk::launch_inner_lanczos(in, st);
+    if (e == cudaSuccess) e = (cudaError_t)nk::launch_rhi(in, st);
     if (e != cudaSuccess) return set_err(err, err_len, NK_ECUDA, cudaGetErrorString(e));
     nk::launch_inner_combine(in, st);
     e = cudaGetLastError();
