@@ -469,7 +469,7 @@ int nk_set_predictor(nk_ctx* ctx, nk_mlp* m);
  * arrays owned by the caller (alpha_dev, beta_dev, gamma_dev, c_dev in the
  * nk_outer_lanczos_dev layout, complex doubles [r*k + j]) and every other
  * buffer it needs lives in one static device array of the library (about
- * 5.9 MB, held by every GPU that loads the library until the process exits).
+ * 5 MB, held by every GPU that loads the library until the process exits).
  * It calls no cudaMalloc/cudaFree and needs no context.
  * Limits: n_rhs <= NK_NOALLOC_MAX_RHS, k <= NK_NOALLOC_MAX_K,
  * l <= NK_NOALLOC_MAX_ELL; larger sizes return NK_EINVAL with a message.

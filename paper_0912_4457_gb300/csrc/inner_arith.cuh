@@ -59,6 +59,32 @@ __device__ __forceinline__ double2 shfl_from(double2 v, int src) {
     return mk(__shfl_sync(kFull, v.x, src), __shfl_sync(kFull, v.y, src));
 }
 
+// 1/n for n in [1, 16): an FP32 reciprocal (its conversions on the integer
+// pipe) and two Newton steps r <- r + r (1 - n r), four FP64 instructions where
+// a division takes about ten.  About one ulp.
+__device__ __forceinline__ double rcp_unit(double n) {
+    double r = f2d_int(__frcp_rn(d2f_int(n)));
+    r = fma(r, fma(-n, r, 1.0), r);
+    return fma(r, fma(-n, r, 1.0), r);
+}
+// 1/a of a pivot.  Scaled by a power of two (exact) into the range of rcp_unit;
+// complex as conj(a) / |a|^2, which then neither over- nor underflows.  Near
+// the ends of the exponent range, and for zero, infinity and NaN: t_inv.
+__device__ __forceinline__ double pivot_inv(double a) {
+    const int e = ((__double2hiint(a) & 0x7fffffff) >> 20) - 1023;
+    if (e < -1000 || e > 1000) return t_inv(a);
+    const double s = pow2(-e), r = rcp_unit(fabs(a) * s) * s;
+    return a < 0.0 ? -r : r;
+}
+__device__ __forceinline__ double2 pivot_inv(double2 a) {
+    const int hx = __double2hiint(a.x) & 0x7fffffff, hy = __double2hiint(a.y) & 0x7fffffff;
+    const int e = (max(hx, hy) >> 20) - 1023;
+    if (e < -1000 || e > 1000) return t_inv(a);
+    const double s = pow2(-e), x = a.x * s, y = a.y * s;
+    const double r = rcp_unit(fma(x, x, y * y)) * s;
+    return mk(x * r, -y * r);
+}
+
 // |x| as ordered bits: compares magnitudes without an FP64 comparison
 __device__ __forceinline__ unsigned long long abs_bits(double x) {
     return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
