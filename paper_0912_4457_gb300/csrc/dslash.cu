@@ -413,6 +413,7 @@ void launch_stencil_step(int precision, const void* U, const Geom& g, const Oute
         s.n_a = o.n_rhs;
         s.n_d = n_d;
         s.scale = o.sc;
+        s.out_abi = false;
         launch_stencil_df(U, g, s, kappa, mu, st);
         return;
     }
@@ -544,22 +545,26 @@ __global__ void f32pair_to_abi(const float4* __restrict__ in, long in_stride, do
     out[(size_t)vec * out_stride + (size_t)site * 12 + 2 * pr + 1] = make_double2(v.z, v.w);
 }
 
-__global__ void to_df(const double2* __restrict__ in, long in_stride, dfc* __restrict__ out, long out_stride,
-                      long N, int n) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (size_t)N * n) return;
-    int vec = (int)(i / N);
-    size_t j = i % N;
-    double2 v = in[(size_t)vec * in_stride + j];
+// ABI spinor [site][12] -> two-float [12][V], n vectors
+__global__ void abi_to_df(const double2* __restrict__ in, long in_stride, dfc* __restrict__ out, long out_stride,
+                          int V, int n) {
+    pdl_trigger();
+    pdl_wait();
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;   // (vector, site, component)
+    const size_t per = (size_t)V * 12;
+    if (i >= per * n) return;
+    const int vec = (int)(i / per);
+    const unsigned j = (unsigned)(i - vec * per), site = j / 12u, c = j % 12u;
+    const double2 v = in[(size_t)vec * in_stride + j];
     dfc w;
     w.x = df_from_double(v.x);
     w.y = df_from_double(v.y);
-    out[(size_t)vec * out_stride + j] = w;
+    out[(size_t)vec * out_stride + (size_t)c * V + site] = w;
 }
 
-void launch_to_df(const double2* in, long in_stride, dfc* out, long out_stride, long N, int n, cudaStream_t st) {
-    size_t tot = (size_t)N * n;
-    to_df<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(in, in_stride, out, out_stride, N, n);
+void launch_abi_to_df(const double2* in, long in_stride, dfc* out, long out_stride, int V, int n, cudaStream_t st) {
+    const size_t tot = (size_t)V * 12 * n;
+    launch_kernel(abi_to_df, (unsigned)((tot + 255) / 256), 256, 0, st, true, in, in_stride, out, out_stride, V, n);
 }
 
 void launch_abi_to_f32pair(const double2* in, long in_stride, float4* out, long out_stride, int V, int n,

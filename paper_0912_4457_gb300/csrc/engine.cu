@@ -1896,26 +1896,24 @@ int nk_dslash_dev(nk_ctx* c, const double* in_dev, double* out_dev, int n_vec, i
         return NK_OK;
     }
     if (precision == 48) {
-        // scratch: SoA input, its two-float copy and SoA output
-        size_t bytes = align_up(sizeof(double2) * N * n_vec) * 3;
+        // scratch: the two-float copy of the input; the output goes straight to
+        // the ABI layout (the stencil reads only the copy, so out may be in)
+        const size_t bytes = align_up(sizeof(double2) * N * n_vec);
         int rc = ensure(c, c->staging, std::max(bytes, c->staging.bytes));
         if (rc) return rc;
-        double2* in_soa = (double2*)c->staging.p;
-        double2* out_soa = (double2*)((char*)c->staging.p + align_up(sizeof(double2) * N * n_vec));
-        nk::dfc* in_df = (nk::dfc*)((char*)out_soa + align_up(sizeof(double2) * N * n_vec));
-        nk::launch_abi_to_soa((const double2*)in_dev, N, in_soa, N, c->V, n_vec, st);
+        nk::dfc* in_df = (nk::dfc*)c->staging.p;
+        nk::launch_abi_to_df((const double2*)in_dev, N, in_df, N, c->V, n_vec, st);
         // the multi-RHS two-float stencil of the solver's early steps
-        nk::launch_to_df(in_soa, N, in_df, N, N, n_vec, st);
         nk::StencilDfSet sd;
         sd.in_a = sd.in_d = in_df;
         sd.in_stride = N;
-        sd.out_a = sd.out_d = out_soa;
+        sd.out_a = sd.out_d = (double2*)out_dev;
         sd.out_stride = N;
         sd.n_a = dagger ? 0 : n_vec;
         sd.n_d = dagger ? n_vec : 0;
         sd.scale = nullptr;
+        sd.out_abi = true;
         nk::launch_stencil_df(c->Udf, geom_of(c), sd, kappa_of(c), c->mu, st);
-        nk::launch_soa_to_abi(out_soa, N, (double2*)out_dev, N, nullptr, 0, c->V, n_vec, st);
         NK_CUDA(c, cudaGetLastError());
         return NK_OK;
     }

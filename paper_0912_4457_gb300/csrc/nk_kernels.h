@@ -38,7 +38,8 @@ void launch_links_to_device_layout(const double2* in, double2* u64, float2* u32,
                                    cudaStream_t st);
 int plaquette_blocks(const Geom& g);
 void launch_plaquette(const double2* U, const Geom& g, double* partial, cudaStream_t st);
-void launch_to_df(const double2* in, long in_stride, dfc* out, long out_stride, long N, int n, cudaStream_t st);
+// ABI spinors ([site][12]) -> two-float vectors [12][V], n vectors
+void launch_abi_to_df(const double2* in, long in_stride, dfc* out, long out_stride, int V, int n, cudaStream_t st);
 void launch_abi_to_soa(const double2* in, long in_stride, double2* out, long out_stride, int V,
                        int n, cudaStream_t st);
 void launch_soa_to_abi(const double2* in, long in_stride, double2* out, long out_stride,
@@ -82,6 +83,7 @@ struct StencilDfSet {
     long in_stride, out_stride;
     int n_a, n_d;
     const double2* scale;
+    bool out_abi;   // output in the ABI layout [V][12]
 };
 void launch_stencil_df(const void* Udf, const Geom& g, const StencilDfSet& s, double kappa, double mu,
                        cudaStream_t st);

@@ -193,8 +193,11 @@ __global__ void __launch_bounds__(384, 2) k_stencil32(const float2* __restrict__
         const int side = v < s.n_a ? 0 : 1;
         return (side ? s.in_d : s.in_a) + (size_t)(side ? v - s.n_a : v) * s.vstride;
     };
+    pdl_trigger();
+    // the links (written by nothing that a stream may still run here) are staged before the wait
     s32_stage_begin(U, g, site0, S);
     s32_stage_end();
+    pdl_wait();
     for (int v = threadIdx.y; v < nv; v += blockDim.y) {
         const int side = v < s.n_a ? 0 : 1;
         const int vi = side ? v - s.n_a : v;
@@ -433,8 +436,9 @@ void launch_stencil32(const void* U, const Geom& g, const Stencil32Set& s, doubl
     if (nv == 0) return;
     const dim3 block = s32_block(nv);
     const unsigned grid = (unsigned)((g.V + block.x - 1) / block.x);
-    k_stencil32<<<grid, block, s32_smem(block.x, block.x * block.y), st>>>((const float2*)U, g, s, (float)kappa,
-                                                                           (float)exp(mu), (float)exp(-mu));
+    // alone (no step scalars): a dependent launch
+    launch_kernel(k_stencil32, grid, block, s32_smem(block.x, block.x * block.y), st, !s.scale, (const float2*)U, g, s,
+                  (float)kappa, (float)exp(mu), (float)exp(-mu));
 }
 
 template <bool TS, bool PASS2, bool RING>

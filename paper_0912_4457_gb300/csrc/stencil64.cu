@@ -158,6 +158,8 @@ template <int S, bool ABI>
 __global__ void __launch_bounds__(16 * S) k_stencil64(const double2* __restrict__ U, Geom g, DslashSet s0, DslashSet s1,
                                                       double kappa, double emu, double emu_inv) {
     __shared__ double2 sx[48 * S];
+    pdl_trigger();
+    pdl_wait();
     const int nvec = s0.n + s1.n;
     const int vec = blockIdx.x % nvec, site0 = (blockIdx.x / nvec) * S;
     const DslashSet& D = vec < s0.n ? s0 : s1;
@@ -332,8 +334,8 @@ void launch_stencil64(const void* U64, const Geom& g, const DslashSet& s0, const
     if (nvec == 0) return;
     constexpr int S = 8;
     const unsigned grid = (unsigned)((g.V + S - 1) / S) * (unsigned)nvec;
-    if (abi) k_stencil64<S, true><<<grid, 16 * S, 0, st>>>((const double2*)U64, g, s0, s1, kappa, exp(mu), exp(-mu));
-    else k_stencil64<S, false><<<grid, 16 * S, 0, st>>>((const double2*)U64, g, s0, s1, kappa, exp(mu), exp(-mu));
+    if (abi) launch_kernel(k_stencil64<S, true>, grid, 16 * S, 0, st, true, (const double2*)U64, g, s0, s1, kappa, exp(mu), exp(-mu));
+    else launch_kernel(k_stencil64<S, false>, grid, 16 * S, 0, st, true, (const double2*)U64, g, s0, s1, kappa, exp(mu), exp(-mu));
 }
 
 }  // namespace nk

@@ -19,7 +19,7 @@
 // psi_1.re), UI = (psi_0.im, psi_1.im), DR, DI (spins 2, 3).
 //
 // Input: two-float vectors (dfc, [vector][12][V]); output: FP64 vectors
-// ([vector][12][V]) of gamma5 (psi - kappa hops), optionally scaled by the
+// ([vector][12][V], or the ABI layout [vector][V][12]) of gamma5 (psi - kappa hops), optionally scaled by the
 // step scalar 1/n_j (A) or 1/m_j (A^dagger) in two-float arithmetic -- the
 // input of the FP64 step-1 kernel.
 #include "nk_common.cuh"
@@ -73,7 +73,8 @@ __device__ __forceinline__ void df_stage(const dfc* __restrict__ U, const Geom& 
         }
     }
     __syncthreads();
-    for (int q = ty; q < 72; q += vg) {
+#pragma unroll 2
+    for (int q = ty; q < 72; q += vg) {   // (two elements in flight: few vectors make many rounds)
         const int h = q / 9, e = q % 9, nu = h >> 1, a = e / 3, b = e % 3;
         const bool fwd = (h & 1) != 0;
         // M_ab = U(x - nu)_ab backward, conj(U(x)_ba) forward
@@ -213,7 +214,9 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
     const DfSmem S = df_carve(smem);
     const int site0 = blockIdx.x * kDfSites;
     const int site = min(site0 + (int)threadIdx.x, g.V - 1);
-    df_stage(U, g, site0, S);
+    pdl_trigger();
+    df_stage(U, g, site0, S);   // (the links: nothing that a stream may still run here writes them)
+    pdl_wait();
     const int v = threadIdx.y;
     if (v >= s.n_a + s.n_d) return;
     const int side = v < s.n_a ? 0 : 1;
@@ -263,8 +266,9 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
             double r0, r1, i0, i1;
             p2_to_double(orr, r0, r1);
             p2_to_double(oii, i0, i1);
-            out[(size_t)(3 * (2 * hf) + a) * g.V + site] = make_double2(r0, i0);
-            out[(size_t)(3 * (2 * hf + 1) + a) * g.V + site] = make_double2(r1, i1);
+            const int c0 = 3 * (2 * hf) + a, c1 = c0 + 3;
+            out[s.out_abi ? (size_t)site * 12 + c0 : (size_t)c0 * g.V + site] = make_double2(r0, i0);
+            out[s.out_abi ? (size_t)site * 12 + c1 : (size_t)c1 * g.V + site] = make_double2(r1, i1);
         }
     }
 }
@@ -288,8 +292,8 @@ void launch_stencil_df(const void* Udf, const Geom& g, const StencilDfSet& s, do
     if (nv == 0) return;
     const dim3 block(kDfSites, nv);
     const unsigned grid = (unsigned)((g.V + kDfSites - 1) / kDfSites);
-    k_stencil_df<<<grid, block, df_smem(), st>>>((const dfc*)Udf, g, s, df_of_host(kappa), df_of_host(exp(mu)),
-                                                  df_of_host(exp(-mu)));
+    launch_kernel(k_stencil_df, grid, block, df_smem(), st, !s.scale, (const dfc*)Udf, g, s, df_of_host(kappa),
+                  df_of_host(exp(mu)), df_of_host(exp(-mu)));
 }
 
 }  // namespace nk

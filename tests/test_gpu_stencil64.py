@@ -83,3 +83,37 @@ def test_fused_step_shapes(mu, threads, order, split):
     y2, _, _ = ctx.sign_apply(b, k, 8, p=1.0, flags=NK_FP64 | NK_DOUBLE_PASS)
     assert rel(y2, y1) < 1e-13
     ctx.close()
+
+
+def test_operators_back_to_back():
+    """Consecutive calls may overlap on the device (dependent launches): a
+    chain of applications, each reading the last one's result, equals the same
+    chain with a synchronisation after every call, in every precision."""
+    dims, n = (5, 4, 3, 6), 3
+    ctx, _ = make_ctx(dims, 0.2)
+    x = torch.from_numpy(inputs.gaussian_sources(dims, 45, n_rhs=n)).cuda()
+    V = int(np.prod(dims))
+    f = torch.randn(2 * n, 6, V, 4, device="cuda")
+
+    def chain(sync):
+        out = []
+        for prec in (64, 48, 32):
+            a, b = x.clone(), torch.zeros_like(x)
+            for i in range(6):
+                ctx.dslash_dev(a, b, n, dagger=bool(i & 1), precision=prec)
+                if sync:
+                    torch.cuda.synchronize()
+                a, b = b, a
+            out.append(a.clone())
+        p, q = f.clone(), torch.zeros_like(f)
+        for i in range(6):
+            ctx.stencil32_dev(p, q, n)
+            if sync:
+                torch.cuda.synchronize()
+            p, q = q, p
+        out.append(p.clone())
+        torch.cuda.synchronize()
+        return out
+    for u, v in zip(chain(True), chain(False)):
+        assert torch.equal(u, v)
+    ctx.close()
