@@ -52,8 +52,9 @@ extern "C" {
 #define NK_ENOTCONV (-4)    /* adaptive k: tolerance not met at k_max */
 #define NK_ERHI (-5)        /* Roberts-Higham iteration did not converge */
 #define NK_ECUDA (-6)       /* CUDA runtime error */
-#define NK_ETIMEOUT (-7)    /* a bounded device-side wait ran out (kept for callers that test for it: no
-                               kernel waits on another one or on its own copies now; the clusters
+#define NK_ETIMEOUT (-7)    /* a bounded device-side wait ran out: the grid barriers of the cooperative
+                               launch that runs the FP64 steps of a small batch wait at most one
+                               second each; that RHS is failed (the clusters of the inner part
                                synchronise with hardware cluster barriers) */
 #define NK_ESTATE (-8)      /* call out of order (e.g. no links loaded) */
 
@@ -268,6 +269,10 @@ int nk_set_adapt_start(nk_ctx* ctx, int k_first);
  *                   two-float recurrence (nk_set_df_recurrence): sites per CTA,
  *                   one thread (early_split = 3: one per colour) per site and
  *                   vector.  The multi-RHS stencils of NK_MIXED have one shape.
+ * An FP64 recurrence on a small batch (V n_rhs, times 2 for mu != 0, up to 32768)
+ * with no shape set or tuned runs all its steps in one cooperative launch instead
+ * (needs every one of its CTAs, at most one per SM, resident at once; a device
+ * without cooperative launches runs step by step).
  * A shape belongs to (n_rhs, sidedness of the current mu (mu != 0), the
  * NK_MIXED bit of flags).  Different shapes sum in different orders, so
  * results differ at rounding level; one shape is bitwise reproducible.

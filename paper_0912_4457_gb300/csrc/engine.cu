@@ -57,6 +57,8 @@ struct nk_ctx {
     long N;
     int antiperiodic;
     int device;
+    int sms = 152;         // multiprocessors
+    bool coop = false;     // the device takes cooperative launches
     double mu = 0.0, m_w = 0.0;
     bool mu_set = false;
     int j0 = -1;
@@ -173,6 +175,8 @@ Geom geom_of(const nk_ctx* c) {
 double kappa_of(const nk_ctx* c) { return 1.0 / (8.0 + 2.0 * c->m_w); }
 
 // Carves the solve workspace; returns total bytes (dry run when base == nullptr).
+constexpr int kRunMaxCtas = 160;   // CTAs of a cooperative run of outer steps
+
 struct Layout {
     nk::Outer o;
     nk::Inner in;
@@ -212,6 +216,7 @@ Layout carve(char* base, const Geom& g, int n_rhs, int k, int ell, bool two_side
     o.st_split_df = lc.early_split;
     o.npart = std::max(nblk, nk::dslash_step1_blocks(g, std::min(lc.stencil_threads, lc.early_threads)));
     o.npart = std::max(o.npart, nk::stencil32_blocks(g, two_sided ? 2 * n_rhs : n_rhs));
+    o.npart = std::max(o.npart, 2 * kRunMaxCtas);
     o.npart = std::max(o.npart, nk::stencil64_blocks(g, lc.stencil_threads, two_sided ? 2 * n_rhs : n_rhs));
     o.q_ring = double_pass ? 1 : 0;
     o.qcols = double_pass ? 3 : k + 1;   // single pass: k basis vectors + one scratch column
@@ -235,6 +240,7 @@ Layout carve(char* base, const Geom& g, int n_rhs, int k, int ell, bool two_side
     o.gamma = (double2*)take(sizeof(double2) * (size_t)k * n_rhs);
     o.partials = (double2*)take(sizeof(double2) * (size_t)o.npart * n_rhs);
     o.counters = (unsigned*)take(sizeof(unsigned) * n_rhs);
+    o.run_bar = (unsigned*)take(sizeof(unsigned) * n_rhs);
     o.sc = (double2*)take(sizeof(double2) * nk::kScalars * n_rhs);
     o.status = (int*)take(sizeof(int) * n_rhs);
     o.xnorm = (double*)take(sizeof(double) * n_rhs);
@@ -407,6 +413,18 @@ int copy_mode_for(const Schedule& s, int j) {
     return p == 32 ? nk::kCopy32 : (p == 48 ? nk::kCopyDF : nk::kCopyNone);
 }
 
+// Whether the FP64 steps of this recurrence run as one cooperative launch
+// (k_run64): a small batch -- up to kRunSiteVecs sites times vectors, beyond which
+// the FP64 pipe hides the step kernels' launches and tails and their finer grain
+// wins (measured us per step, run against step kernels: 6^4 x 2 vectors 16.7 / 21.3,
+// 10^4 x 2 53.9 / 58.3, 6^4 x 24 78.8 / 80.3, 8^4 x 12 114.7 / 112.4) -- with no launch shape of
+// its own (a set or tuned shape names the kernels of a step).
+constexpr long kRunSiteVecs = 32768;
+bool run_in_one(const nk_ctx* c, const nk::Outer& o) {
+    if (!c->coop || (long)c->V * o.n_rhs * (o.two_sided ? 2 : 1) > kRunSiteVecs) return false;
+    return c->tune.count(std::make_tuple(o.n_rhs, o.two_sided ? 1 : 0, 0)) == 0;
+}
+
 void enqueue_outer_init(const nk::Outer& o, const Schedule& s, Launcher& L, bool keep_status = false) {
     cudaStream_t st = L.st;
     L.run(NK_CLASS_OTHER, 2, [&] { nk::launch_outer_init(o, copy_mode_for(s, 0), st, keep_status); });
@@ -422,6 +440,14 @@ void enqueue_outer_steps(nk_ctx* c, const nk::Outer& o, const Schedule& s, int j
     const Geom g = geom_of(c);
     const double kap = kappa_of(c);
     cudaStream_t st = L.st;
+    if (!s.mixed && !L.profile && j_end > j_begin && run_in_one(c, o)) {
+        bool ok = true;
+        L.run(NK_CLASS_DSLASH64, 1, [&] {
+            ok = nk::launch_run64(c->U64, g, o, j_begin, j_end, kap, c->mu, std::min(c->sms, kRunMaxCtas), st);
+        });
+        if (ok) return;
+        cudaGetLastError();   // no cooperative launch here: step by step
+    }
     for (int j = j_begin; j < j_end; ++j) {
         const int prec = s.prec(j);
         const void* U = prec == 64 ? (const void*)c->U64 : (prec == 48 ? (const void*)c->Udf : (const void*)c->U32);
@@ -994,6 +1020,9 @@ int nk_create_lattice(const int dims[4], int bc_t_antiperiodic, nk_ctx** out) {
         delete c;
         return NK_ECUDA;
     }
+    int attr = 0;
+    if (cudaDeviceGetAttribute(&attr, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess && attr > 0) c->sms = attr;
+    if (cudaDeviceGetAttribute(&attr, cudaDevAttrCooperativeLaunch, c->device) == cudaSuccess) c->coop = attr != 0;
     nk::init_kernel_attributes();
     cudaGetLastError();
     for (auto& e : c->ph) {

@@ -32,6 +32,7 @@
 
 #include "nk_common.cuh"
 #include "nk_kernels.h"
+#include "nk_step.cuh"
 
 namespace nk {
 
@@ -134,39 +135,16 @@ __device__ __forceinline__ void step2_finish(const Outer& o, int rhs, int j, dou
     double2 part = block_sum(acc, sh);
     if (finish_partial(part, o.partials + (size_t)rhs * o.npart, o.counters + rhs, blockIdx.x, o.nblk)) {
         double2* sc = o.sc + (size_t)rhs * kScalars;
-        const double2 inv_n = sc[kScN], inv_m = sc[kScM];   // 1/n_j, 1/m_j
-        double2 d = sum_partials(o.partials + (size_t)rhs * o.npart, o.nblk, sh);
+        const double2 d = sum_partials(o.partials + (size_t)rhs * o.npart, o.nblk, sh);
         if (threadIdx.x == 0) {
             const size_t at = (size_t)rhs * o.k + j;
-            double2 b, g, ib = mk(0.0, 0.0), ig = mk(0.0, 0.0);
-            bool ok = true;
-            if (!TS) {
-                // beta <- sqrt(r^dag r)
-                ok = d.x > 0.0 && isfinite(d.x);
-                double inv = 0.0;
-                const double bb = ok ? sqrt_inv(d.x, inv) : sqrt(d.x);
-                b = g = mk(bb, 0.0);
-                ib = ig = mk(inv, 0.0);
-                if (!ok) mark_failed(o, rhs, kStatusBreakdown);
-            } else if ((d.x == 0.0 && d.y == 0.0) || !isfinite(d.x) || !isfinite(d.y)) {
-                // serious breakdown: delta = 0 (App. B); a non-finite delta is treated alike
-                mark_failed(o, rhs, kStatusBreakdown);
-                b = g = mk(0.0, 0.0);
-                ok = false;
-            } else {
-                csqrt_scalars(d, b, g, ib, ig);          // beta <- sqrt(delta), gamma <- delta^* / beta
-            }
-            o.beta[at] = b;
-            o.gamma[at] = g;
+            const StepScalars t = step_scalars<TS>(d);
+            if (!t.ok) mark_failed(o, rhs, kStatusBreakdown);
+            o.beta[at] = t.beta;
+            o.gamma[at] = t.gamma;
             o.counters[rhs] = 0u;
             // step j + 1: n_{j+1} = beta_j, m_{j+1} = gamma_j^*
-            if (ok && j + 1 < o.k && o.status[rhs] == kStatusOK) {
-                sc[kScN] = ib;
-                sc[kScC1] = cmul(g, inv_n);              // gamma (Hermitian: beta) / n_j
-                sc[kScD] = ig;
-                sc[kScM] = cconj(ig);
-                sc[kScC1L] = cmul(cconj(b), inv_m);
-            }
+            if (t.ok && j + 1 < o.k && o.status[rhs] == kStatusOK) next_scalars<TS>(sc, t);
         }
     }
 }

@@ -34,6 +34,11 @@ void launch_stencil64(const void* U64, const Geom& g, const DslashSet& s0, const
 void launch_stencil64_step1(const void* U64, const Geom& g, const Outer& o, int j, double kappa, double mu,
                             cudaStream_t st);
 int stencil64_blocks(const Geom& g, int threads, int nvec);   // CTAs, hence partial sums, per vector
+// Steps [j_lo, j_hi) of an FP64 recurrence in one cooperative launch of at most
+// `sms` CTAs (two partial sums per CTA and RHS: npart >= 2 sms / n_rhs).
+// False if the launch failed (cudaGetLastError has the reason).
+bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int j_hi, double kappa, double mu, int sms,
+                  cudaStream_t st);
 void launch_links_to_device_layout(const double2* in, double2* u64, float2* u32, dfc* udf, int V,
                                    cudaStream_t st);
 int plaquette_blocks(const Geom& g);
@@ -120,6 +125,7 @@ struct Outer {
     double2* beta;   // H(j+1,j), [rhs][k]
     double2* gamma;  // H(j,j+1), [rhs][k]
     double2* partials;  // [rhs][npart]
+    unsigned* run_bar;  // [rhs]: arrivals at the grid barriers of k_run64 (stencil64.cu)
     unsigned* counters; // [rhs]; the all-RHS kernels (k_stencil32_step1) use counters[0]
     double2* sc;        // [rhs][kScalars]: scalars of the current outer step (below)
     int* status;        // [rhs]
@@ -198,7 +204,14 @@ constexpr int kStatusRhi = 3;         // RHi did not converge / singular pivot
 constexpr int kStatusLU = 4;          // singular p H_k
 constexpr int kStatusConverged = 5;   // adaptive k: frozen at its converged size (skipped by the kernels)
 constexpr int kStatusInnerBreakdown = 6;  // inner (two-sided) Lanczos on H_k': zero beta or delta
-constexpr int kStatusTimeout = 7;     // a bounded device-side wait ran out (no kernel has one now)
+constexpr int kStatusTimeout = 7;     // a bounded wait at a grid barrier of k_run64 ran out
+
+// beta_j, gamma_j and their inverses from delta = r^dag l (Hermitian: r^dag r,
+// in its real part); ok = false: breakdown.
+struct StepScalars {
+    double2 beta, gamma, inv_beta, inv_gamma;
+    bool ok;
+};
 
 // First failure of an RHS wins (a later one does not overwrite it).
 __device__ inline void mark_failed(const Outer& o, int rhs, int code) { atomicCAS(o.status + rhs, kStatusOK, code); }

@@ -29,6 +29,7 @@
 // the default S = 8 (6^4 28 against 32 us) and level with it at S = 4, 4^4.
 #include "nk_common.cuh"
 #include "nk_kernels.h"
+#include "nk_step.cuh"
 
 namespace nk {
 
@@ -56,11 +57,11 @@ __device__ __forceinline__ size_t comp_at(int c, int site, int V) {
 // Phase 1: thread (s, h, c[, a]) of the CTA's sites leaves row(s) a of
 // M (psi_up + s C psi_dn)_c of hop h in sx[((h * 2 + c) * 3 + a) * S + s].
 // The coordinate of `site` along nu decides the neighbour; sites past V use V - 1.
-template <int S, int SPLIT, bool ABI>
+// CG: read `in` past the L1 cache (vectors that the running kernel itself writes).
+template <int S, int SPLIT, bool ABI, bool CG = false>
 __device__ __forceinline__ void s64_hops(const double2* __restrict__ U, const double2* __restrict__ in, const Geom& g,
-                                         int site0, double2* __restrict__ sx) {
+                                         int site0, double2* __restrict__ sx, int tid) {
     constexpr int ROWS = 3 / SPLIT;
-    const int tid = threadIdx.x;
     const int s = tid % S, hc = (tid / S) & 15, a0 = SPLIT == 1 ? 0 : tid / (16 * S);
     const int h = hc >> 1, c = hc & 1, nu = h >> 1;
     const bool fwd = (h & 1) != 0;
@@ -82,8 +83,9 @@ __device__ __forceinline__ void s64_hops(const double2* __restrict__ U, const do
     const int q = (nu == 0 ? 3 : nu == 1 ? (c ? 0 : 2) : nu == 2 ? (c ? 1 : 3) : 0) + (fwd ? 2 : 0);
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        up[b] = in[comp_at<ABI>(3 * c + b, sn, V)];
-        dn[b] = in[comp_at<ABI>(3 * ic + b, sn, V)];
+        const double2 *pu = in + comp_at<ABI>(3 * c + b, sn, V), *pd = in + comp_at<ABI>(3 * ic + b, sn, V);
+        up[b] = CG ? __ldcg(pu) : *pu;
+        dn[b] = CG ? __ldcg(pd) : *pd;
     }
 #pragma unroll
     for (int r = 0; r < ROWS; ++r)
@@ -165,7 +167,7 @@ __global__ void __launch_bounds__(16 * S) k_stencil64(const double2* __restrict_
     const DslashSet& D = vec < s0.n ? s0 : s1;
     const int vi = vec < s0.n ? vec : vec - s0.n;
     const double2* __restrict__ in = reinterpret_cast<const double2*>(D.in) + (size_t)vi * D.in_stride;
-    s64_hops<S, 1, ABI>(U, in, g, site0, sx);
+    s64_hops<S, 1, ABI>(U, in, g, site0, sx, threadIdx.x);
     // component-fastest threads in the ABI layout, site-fastest in the device one (coalesced
     // stores).  12 of 16 threads sum: which warps idle rotates with the block of sites, as
     // the FP64 pipe of an SM sub-partition serves the warps of one residue mod 4
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(16 * S * SPLIT, SPLIT == 1 ? kS64Sites / S : 1
     const unsigned sg = sp < 2 ? 0u : 0x80000000u;   // gamma5 = diag(1, 1, -1, -1)
     double2 dot = make_double2(0.0, 0.0);
     for (int b = b_lo; b < b_hi; ++b) {
-        s64_hops<S, SPLIT, false>(U, in, g, b * S, sx);
+        s64_hops<S, SPLIT, false>(U, in, g, b * S, sx, threadIdx.x);
         const int site = b * S + s;
         const bool live = comp < 12 && site < V;
         const size_t idx = (size_t)comp * V + site;
@@ -284,6 +286,206 @@ __global__ void __launch_bounds__(16 * S * SPLIT, SPLIT == 1 ? kS64Sites / S : 1
     }
 }
 
+// ---- a run of outer steps in one launch ----------------------------------------------
+// Steps [j_lo, j_hi) of an FP64 recurrence.  A step of a small lattice is two
+// kernels of 5 to 15 us whose launches, cold starts and one-CTA tails (partial
+// sums, beta, gamma and the scalars on one lane, then a kernel boundary before
+// anyone may use them) are half of it.  Here the CTAs stay: one cooperative
+// launch, at most one CTA per SM and RHS share, and per step two grid barriers
+// of the RHS's CTAs; after each every CTA adds the partial sums and forms the
+// scalars for itself (the same values in the same order everywhere), so nothing
+// waits for a second hop through memory.  64 threads work on four sites as in
+// k_stencil64_step1 (group of the CTA with its own named barrier), then all on
+// (component pair, site) items as in k_step2.  Vectors written by the launch are
+// read past L1.
+// The barriers' waits are bounded: a CTA whose wait runs out marks its RHS
+// kStatusTimeout and leaves; the others' waits then run out too.
+// Measured, us per step against the step kernels: 4^4, mu = 0 13.5 -> 10.0; 6^4, mu = 0.1
+// 21.3 -> 16.7; 10^4, mu = 0.2 58.3 -> 53.9 (all one source).  256 or 512 threads per CTA:
+// 18.3 and 16.7 at 6^4 (two rounds of groups with 256), 57.4 and 54.3 at 10^4.
+constexpr int kRunThreads = 384, kRunGroups = kRunThreads / 64, kRunSites = 4;
+constexpr unsigned long long kRunWaitNs = 1000000000ull;   // one second
+
+__device__ __forceinline__ unsigned long long run_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+// All CTAs of one RHS (n of them; the counter counts arrivals since the launch).
+__device__ __forceinline__ bool run_barrier(unsigned* counter, unsigned target, bool* ok_sh) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+        bool ok = true;
+        if (ld_acquire(counter) < target) {
+            const unsigned long long t0 = run_ns();
+            while (ld_acquire(counter) < target)
+                if (run_ns() - t0 > kRunWaitNs) { ok = false; break; }
+        }
+        *ok_sh = ok;
+    }
+    __syncthreads();
+    return *ok_sh;
+}
+
+template <bool TS, bool PASS2>
+__global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict__ U, Geom g, Outer o, int j_lo, int j_hi,
+                                                          double kappa, double emu, double emu_inv) {
+    __shared__ double2 sx[kRunGroups][48 * kRunSites];
+    __shared__ double2 sh[33];
+    __shared__ double2 sc[kScalars];
+    __shared__ bool ok_sh;
+    const int rhs = blockIdx.x % o.n_rhs, cta = blockIdx.x / o.n_rhs, ncta = gridDim.x / o.n_rhs;
+    if (o.status[rhs] != kStatusOK) return;
+    const int tid = threadIdx.x, grp = tid / 64, gt = tid % 64, warp = tid / 32, lane = tid % 32;
+    const int V = g.V, nsb = (V + kRunSites - 1) / kRunSites;
+    const unsigned items = 6u * (unsigned)V;
+    unsigned* counter = o.run_bar + rhs;
+    unsigned target = 0;
+    double2* part1 = o.partials + (size_t)rhs * o.npart;
+    double2* part2 = part1 + ncta;
+    if (tid < kScalars) sc[tid] = o.sc[(size_t)rhs * kScalars + tid];
+    __syncthreads();
+    // sum of the ncta partials in warp 0 of every CTA (all its lanes)
+    auto total = [&](const double2* part) -> double2 {
+        double2 a = make_double2(0.0, 0.0);
+        for (int i = lane; i < ncta; i += 32) {
+            const double2 v = __ldcg(part + i);
+            a = i == lane ? v : cadd(a, v);
+        }
+        const double t = warp_sum_split(a);
+        return make_double2(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 16));
+    };
+    const int s = gt % kRunSites, comp = gt / kRunSites, sp = comp / 3, a = comp % 3;
+    const unsigned sg = sp < 2 ? 0u : 0x80000000u;
+    for (int j = j_lo; j < j_hi; ++j) {
+        const int jp = j > 0 ? j - 1 : j;
+        const bool left = TS && j < o.k - 1;
+        // ---- stencil and step 1 ----
+        double2 dot = make_double2(0.0, 0.0);
+        for (int u = cta + ncta * grp; u < (left ? 2 : 1) * nsb; u += ncta * kRunGroups) {
+            const int side = u >= nsb ? 1 : 0, b = u - side * nsb;
+            const double2* in = side ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
+            s64_hops<kRunSites, 1, false, true>(U, in, g, b * kRunSites, sx[grp], gt);
+            const int site = b * kRunSites + s;
+            const bool live = comp < 12 && site < V;
+            const size_t idx = (size_t)comp * V + site;
+            double2 p = make_double2(0.0, 0.0), pv = p, d = p;
+            if (live) {
+                p = __ldcg(in + idx);
+                pv = __ldcg((side ? outer_p(o, rhs, jp) : outer_q(o, rhs, jp)) + idx);
+                if (side == 0) d = __ldcg((TS ? outer_p(o, rhs, j) : outer_q(o, rhs, j)) + idx);
+            }
+            asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");
+            if (live) {
+                double wp, wm;
+                t_weights(g, site, side, emu, emu_inv, wp, wm);
+                const double2 acc = s64_sum<kRunSites>(sx[grp], s, sp, a, wp, wm);
+                const double2 v = make_double2(flip(fma(-kappa, acc.x, p.x), sg), flip(fma(-kappa, acc.y, p.y), sg));
+                const double2 scl = sc[side ? kScM : kScN], c1 = sc[side ? kScC1L : kScC1];
+                double2 rr;
+                if (TS) {
+                    rr = make_double2(v.x * scl.x - v.y * scl.y, v.x * scl.y + v.y * scl.x);
+                    rr = caxpy_neg(rr, c1, pv);
+                } else {
+                    rr = make_double2(v.x * scl.x, v.y * scl.x);
+                    rr = make_double2(fma(-c1.x, pv.x, rr.x), fma(-c1.x, pv.y, rr.y));
+                }
+                (side ? outer_p(o, rhs, j + 1) : outer_q(o, rhs, j + 1))[idx] = rr;
+                if (side == 0) {
+                    dot.x = fma(d.x, rr.x, fma(d.y, rr.y, dot.x));      // conj(d) r
+                    if (TS) dot.y = fma(d.x, rr.y, fma(-d.y, rr.x, dot.y));
+                    if (PASS2) {
+                        double2* y = o.y + (size_t)rhs * o.N + idx;
+                        *y = caxpy_pos(*y, o.cp[(size_t)rhs * o.k + j], TS ? p : d);
+                    }
+                }
+            }
+            asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");   // sx is rewritten
+        }
+        dot = block_sum(dot, sh);
+        if (tid == 0) part1[cta] = dot;
+        target += (unsigned)ncta;
+        if (!run_barrier(counter, target, &ok_sh)) {
+            if (tid == 0) mark_failed(o, rhs, kStatusTimeout);
+            return;
+        }
+        if (warp == 0) {   // one warp: an FP64 warp instruction costs its pipe as much as any
+            const double2 tot = total(part1);
+            // Hermitian: H(j,j) = Re(q_j^dag r) / n_j, real (App. C); two-sided: (p_j^dag r) / m_j^*
+            const double2 al = TS ? cmul(sc[kScD], tot) : make_double2(tot.x * sc[kScD].x, 0.0);
+            if (lane == 0) {
+                if (cta == 0) o.alpha[(size_t)rhs * o.k + j] = al;
+                sc[kScC3] = cmul(al, sc[kScN]);
+                sc[kScC4] = TS ? cmul(cconj(al), sc[kScM]) : make_double2(0.0, 0.0);
+            }
+        }
+        __syncthreads();
+        if (j == o.k - 1) break;
+        const double2 c3 = sc[kScC3], c4 = sc[kScC4];
+        // ---- step 2 ----
+        const double2* qj = outer_q(o, rhs, j);
+        double2* r = outer_q(o, rhs, j + 1);
+        const double2* pj = TS ? outer_p(o, rhs, j) : nullptr;
+        double2* l = TS ? outer_p(o, rhs, j + 1) : nullptr;
+        double2 del = make_double2(0.0, 0.0);
+        const unsigned stride = (unsigned)ncta * kRunThreads;
+        for (unsigned i = (unsigned)(cta + ncta * warp) * 32u + lane; i < items; i += stride) {
+            const size_t e0 = (size_t)i + (size_t)(i / (unsigned)V) * V;   // component 2 cp of the item
+            double2 q[2], x[2], pv[2], w[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const size_t e = e0 + (size_t)h * V;
+                q[h] = __ldcg(qj + e);
+                x[h] = __ldcg(r + e);
+                if (TS) { pv[h] = __ldcg(pj + e); w[h] = __ldcg(l + e); }
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const size_t e = e0 + (size_t)h * V;
+                x[h] = TS ? caxpy_neg(x[h], c3, q[h])
+                          : make_double2(fma(-c3.x, q[h].x, x[h].x), fma(-c3.x, q[h].y, x[h].y));
+                r[e] = x[h];
+                if (TS) {
+                    w[h] = caxpy_neg(w[h], c4, pv[h]);
+                    l[e] = w[h];
+                    del.x = fma(x[h].x, w[h].x, fma(x[h].y, w[h].y, del.x));   // conj(r) l
+                    del.y = fma(x[h].x, w[h].y, fma(-x[h].y, w[h].x, del.y));
+                } else {
+                    del.x = fma(x[h].x, x[h].x, fma(x[h].y, x[h].y, del.x));
+                }
+            }
+        }
+        del = block_sum(del, sh);
+        if (tid == 0) part2[cta] = del;
+        target += (unsigned)ncta;
+        if (!run_barrier(counter, target, &ok_sh)) {
+            if (tid == 0) mark_failed(o, rhs, kStatusTimeout);
+            return;
+        }
+        if (warp == 0) {
+            const StepScalars t = step_scalars<TS>(total(part2));
+            if (lane == 0) {
+                if (cta == 0) {
+                    o.beta[(size_t)rhs * o.k + j] = t.beta;
+                    o.gamma[(size_t)rhs * o.k + j] = t.gamma;
+                    if (!t.ok) mark_failed(o, rhs, kStatusBreakdown);
+                }
+                ok_sh = t.ok;
+                if (t.ok) next_scalars<TS>(sc, t);
+            }
+        }
+        __syncthreads();
+        if (!ok_sh) return;   // the same decision in every CTA of the RHS
+    }
+    if (cta == 0 && tid < kScalars && j_hi < o.k) o.sc[(size_t)rhs * kScalars + tid] = sc[tid];
+}
+
 template <int S, int SPLIT>
 void launch_s64_step1(const double2* U, const Geom& g, const Outer& o, int j, double kappa, double emu, double emu_inv,
                       cudaStream_t st) {
@@ -326,6 +528,36 @@ void launch_stencil64_step1(const void* U64, const Geom& g, const Outer& o, int 
     else if (o.st_threads == 128) NK_S64(8);
     else NK_S64(16);
 #undef NK_S64
+}
+
+bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int j_hi, double kappa, double mu, int sms,
+                  cudaStream_t st) {
+    // one CTA per SM over the RHS, fewer where there are not four groups' work for each
+    const int nvec = o.two_sided ? 2 : 1;
+    const int nsb = (g.V + kRunSites - 1) / kRunSites;
+    int ncta = sms / o.n_rhs;
+    if (ncta > nvec * nsb) ncta = nvec * nsb;
+    cudaMemsetAsync(o.run_bar, 0, sizeof(unsigned) * o.n_rhs, st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(ncta * o.n_rhs));
+    cfg.blockDim = dim3(kRunThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const double2* U = (const double2*)U64;
+    const double ep = exp(mu), em = exp(-mu);
+    const bool pass2 = o.y != nullptr;
+    cudaError_t e;
+    if (o.two_sided)
+        e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<true, true>, U, g, o, j_lo, j_hi, kappa, ep, em)
+                  : cudaLaunchKernelEx(&cfg, k_run64<true, false>, U, g, o, j_lo, j_hi, kappa, ep, em);
+    else
+        e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<false, true>, U, g, o, j_lo, j_hi, kappa, ep, em)
+                  : cudaLaunchKernelEx(&cfg, k_run64<false, false>, U, g, o, j_lo, j_hi, kappa, ep, em);
+    return e == cudaSuccess;
 }
 
 void launch_stencil64(const void* U64, const Geom& g, const DslashSet& s0, const DslashSet& s1, bool abi, double kappa,

@@ -117,3 +117,64 @@ def test_operators_back_to_back():
     for u, v in zip(chain(True), chain(False)):
         assert torch.equal(u, v)
     ctx.close()
+
+
+@pytest.mark.parametrize("mu", [0.0, 0.3])
+@pytest.mark.parametrize("dims,n", [((2, 2, 2, 2), 1), ((3, 5, 3, 7), 1), ((3, 3, 4, 5), 5), ((4, 4, 4, 4), 12)])
+def test_run_of_steps_matches_step_kernels(mu, dims, n):
+    """The cooperative launch of all steps (default shape, small batch) against the oracle and the
+    step kernels (a launch shape set), from fewer units of work than CTAs to several per CTA; and
+    the adaptive solve, which continues a recurrence in chunks, against the same solve at fixed k."""
+    k = 12
+    ctx, U = make_ctx(dims, mu)
+    b = inputs.gaussian_sources(dims, 46, n_rhs=n)
+    bd = torch.from_numpy(b).cuda()
+    run = ctx.outer_lanczos_dev(bd, n, k)
+    again = ctx.outer_lanczos_dev(bd, n, k)
+    for u, v in zip(run, again):
+        np.testing.assert_array_equal(u[..., : k - 1], v[..., : k - 1])   # bitwise reproducible
+    y2, _, _ = ctx.sign_apply(b, k, 8, p=1.0, flags=NK_FP64 | NK_DOUBLE_PASS)
+    y1, _, _ = ctx.sign_apply(b, k, 8, p=1.0)
+    assert rel(y2, y1) < 1e-13
+    # an adaptive solve that never meets its tolerance continues the recurrence in chunks of 64
+    # steps: the arithmetic of a fixed k, step for step
+    ya, sta, _ = ctx.sign_apply(b[:1], 128, 32, tol=1e-30, check=False)
+    yf, _, _ = ctx.sign_apply(b[:1], 128, 32)
+    assert sta["checks"] == 2 and rel(ya, yf) < 1e-12
+    ctx.set_launch(n, NK_FP64, 128, 0, 3)
+    steps = ctx.outer_lanczos_dev(bd, n, k)
+    A, Ad, herm = nested.operator(U, dims, mu, M_W)
+    for i in range(n):
+        ref = nested.outer_basis(A, Ad, b[i], k, herm)
+        for got in (run, steps):
+            assert rel(got[0][i], ref.alpha) < 1e-11
+            assert rel(got[1][i, : k - 1], ref.beta[: k - 1]) < 1e-11
+            assert rel(got[2][i, : k - 1], ref.gamma[: k - 1]) < 1e-11
+    ctx.close()
+
+
+def test_runs_of_two_contexts_in_flight():
+    """Two contexts' cooperative launches on two streams: each equals its solve alone."""
+    dims, k = (6, 6, 6, 6), 64
+    from paper_0912_4457_gb300.nksign import NK_ASYNC
+    pair = [make_ctx(dims, 0.2)[0] for _ in range(2)]
+    b = [torch.from_numpy(inputs.gaussian_sources(dims, 47 + i)).cuda() for i in range(2)]
+    y = [torch.zeros_like(x) for x in b]
+    alone = []
+    for c, x, o in zip(pair, b, y):
+        c.sign_apply_dev(x, o, 1, k, 16)
+        alone.append(o.clone())
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for _ in range(5):
+        for c, x, o, s in zip(pair, b, y, streams):
+            o.zero_()
+            torch.cuda.synchronize()
+        for c, x, o, s in zip(pair, b, y, streams):
+            c.sign_apply_dev(x, o, 1, k, 16, flags=NK_FP64 | NK_ASYNC, stream=s)
+        for c in pair:
+            c.wait()
+        for o, ref in zip(y, alone):
+            assert torch.equal(o, ref)
+    for c in pair:
+        c.close()
