@@ -457,7 +457,12 @@ __global__ void k_adapt_delta(Outer o, const double2* __restrict__ c, double2* _
     if (threadIdx.x == 0) dn[rhs] = mk(sqrt(t.x), sqrt(t.y));
 }
 
-// y_r = sum_j c'_r[j] q_j  (reads every basis vector once)
+// y_r = sum_j c'_r[j] q_j  (reads every basis vector once).  REAL: the
+// coefficients are real (the Hermitian recurrence: c = V_l sgn(H_l) e_1 and the
+// scales are), which halves the FP64 work that bounds the lift: 12 sources at 8^4,
+// k = 768, 3.13 -> 1.61 ms against 1.49 on the FP64 pipe and 1.1 for the basis over
+// HBM.  The two-sided lift is at its FP64 time: 10^4 x 12, k = 1024, 9.78 ms.
+template <bool REAL>
 __global__ void __launch_bounds__(kThreads) k_lift(Outer o, const double2* __restrict__ cp,
                                                     const int* __restrict__ kused, double2* __restrict__ y) {
     const int rhs = blockIdx.y;
@@ -475,8 +480,13 @@ __global__ void __launch_bounds__(kThreads) k_lift(Outer o, const double2* __res
     for (int j = 0; j < ku; ++j) {
         const double2 cj = __ldg(cr + j);
         const double2 v = Qr[(size_t)j * o.N + i];
-        acc.x = fma(cj.x, v.x, fma(neg_bits(cj.y), v.y, acc.x));
-        acc.y = fma(cj.x, v.y, fma(cj.y, v.x, acc.y));
+        if (REAL) {
+            acc.x = fma(cj.x, v.x, acc.x);
+            acc.y = fma(cj.x, v.y, acc.y);
+        } else {
+            acc.x = fma(cj.x, v.x, fma(neg_bits(cj.y), v.y, acc.x));
+            acc.y = fma(cj.x, v.y, fma(cj.y, v.x, acc.y));
+        }
     }
     yo[i] = acc;
 }
@@ -574,7 +584,8 @@ void launch_lift(const Outer& o, const double2* cp, const int* kused, double2* y
     // basis columns; an FP64 recurrence is lifted in FP64
     if (o.q_ring) k_zero_bad<<<grid, kThreads, 0, st>>>(o, y);
     else if (o.qr && o.q_df_from < o.k) k_lift_df<<<grid, kThreads, sizeof(dfc) * (size_t)o.k, st>>>(o, cp, kused, y);
-    else k_lift<<<grid, kThreads, 0, st>>>(o, cp, kused, y);
+    else if (o.two_sided) k_lift<false><<<grid, kThreads, 0, st>>>(o, cp, kused, y);
+    else k_lift<true><<<grid, kThreads, 0, st>>>(o, cp, kused, y);
 }
 
 __global__ void k_fill_int(int* p, int n, int v) {
