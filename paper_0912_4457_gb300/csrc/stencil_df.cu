@@ -92,13 +92,15 @@ struct DSpin {
 };
 
 // the two-float spinor of site s (components 3 sp + b, each (re.hi, re.lo,
-// im.hi, im.lo)) in the spin-pair lanes
-__device__ __forceinline__ void load_dspin(const dfc* __restrict__ in, int V, int s, DSpin& p) {
-    const float4* f = reinterpret_cast<const float4*>(in);
+// im.hi, im.lo)) in the spin-pair lanes; SWAP exchanges the lanes of the lower pair
+__device__ __forceinline__ void load_dspin(const dfc* __restrict__ in, int V, int s, DSpin& p, bool swap) {
+    const float4* f = reinterpret_cast<const float4*>(in) + s;
+    const float4* f2 = f + (size_t)(swap ? 9 : 6) * V;
+    const float4* f3 = f + (size_t)(swap ? 6 : 9) * V;
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        const float4 s0 = __ldg(f + (size_t)b * V + s), s1 = __ldg(f + (size_t)(3 + b) * V + s);
-        const float4 s2 = __ldg(f + (size_t)(6 + b) * V + s), s3 = __ldg(f + (size_t)(9 + b) * V + s);
+        const float4 s0 = __ldg(f + (size_t)b * V), s1 = __ldg(f + (size_t)(3 + b) * V);
+        const float4 s2 = __ldg(f2 + (size_t)b * V), s3 = __ldg(f3 + (size_t)b * V);
         p.ur[b] = {pk(s0.x, s1.x), pk(s0.y, s1.y)};
         p.ui[b] = {pk(s0.z, s1.z), pk(s0.w, s1.w)};
         p.dr[b] = {pk(s2.x, s3.x), pk(s2.y, s3.y)};
@@ -106,13 +108,9 @@ __device__ __forceinline__ void load_dspin(const dfc* __restrict__ in, int V, in
     }
 }
 
-// lane signs (S0, S1) in {+1, -1} times the hop sign s (forward hops: -1),
-// exact: m is the sign-bit mask of s in both lanes
-template <int S0, int S1>
-__device__ __forceinline__ P2 sgn(P2 a, f2p m) {
-    constexpr f2p k = (S0 < 0 ? 0x0000000080000000ull : 0ull) | (S1 < 0 ? 0x8000000000000000ull : 0ull);
-    return {a.s ^ m ^ k, a.e ^ m ^ k};
-}
+// sign-bit masks of the two lanes
+constexpr f2p kNeg0 = 0x0000000080000000ull, kNeg1 = 0x8000000000000000ull, kNeg = kNeg0 | kNeg1;
+__device__ __forceinline__ P2 sgn(P2 a, f2p m) { return {a.s ^ m, a.e ^ m}; }
 
 // One hop into the accumulators: acc += w (1 + s gamma_nu) M psi_n with
 // s = +1 backward (M = U(x - nu)), -1 forward (M = U(x)^dagger), in the
@@ -121,40 +119,38 @@ __device__ __forceinline__ P2 sgn(P2 a, f2p m) {
 //                      z: -i psi_2, i psi_3;       t: psi_2, psi_3
 //   (B m)_{0,1}:       nu = x: i m_1, i m_0;        y: m_1, -m_0;
 //                      z: i m_0, -i m_1;           t: m_0, m_1
-// (i z = (-z.im, z.re)); the spin swaps of x and y become swaps of the lanes.
-// One instantiation per direction; the forward and backward hops of it share
-// the code (fwd a runtime value), which halves the kernel's instruction
-// footprint -- the fully unrolled eight hops overflowed the instruction cache.
-template <int NU>
+// (i z = (-z.im, z.re)).  x and y exchange the two lower spins: their lower
+// pair is loaded, and the accumulators' lower pair held, with the lanes
+// swapped.  With that, x and z (EVEN) have the same form but for lane signs,
+// and so have y and t: two instantiations for the eight hops, direction and
+// sense as sign masks.  Instruction fetch is what this saves: eight unrolled
+// hops overflowed the instruction cache, and with one instantiation per
+// direction a warp still waited 0.7 of 6 cycles per instruction for it.
+template <bool EVEN>
 __device__ __forceinline__ void df_hop(DSpin& acc, const dfc* __restrict__ in, int V, const DfSmem& S, df wp_t,
-                                       df wm_t, int fwd) {
-    constexpr int SG = 1;   // lane signs below are for the backward hop; m flips them forward
-    const int H = 2 * NU + fwd;
-    const f2p m = fwd ? 0x8000000080000000ull : 0ull;
+                                       df wm_t, bool swap, int fwd) {
+    const int H = 2 * ((swap ? 0 : 2) + (EVEN ? 0 : 1)) + fwd;
+    const f2p m = fwd ? kNeg : 0ull;
+    const f2p k = m ^ (EVEN ? (swap ? 0ull : kNeg1) : (swap ? kNeg0 : 0ull));
     const int tx = threadIdx.x;
     DSpin p;
-    load_dspin(in, V, S.nb[H * kDfSites + tx], p);
+    load_dspin(in, V, S.nb[H * kDfSites + tx], p, swap);
     // projection: HR = (h0.re, h1.re), HI = (h0.im, h1.im) per colour, and -HI
     P2 hr[3], hi[3], nhi[3];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        if (NU == 0) {        // c0 = -i psi3 = (psi3.im, -psi3.re), c1 = -i psi2
-            hr[b] = p2_add(p.ur[b], sgn<SG, SG>(p2_swp(p.di[b]), m));
-            hi[b] = p2_add(p.ui[b], sgn<-SG, -SG>(p2_swp(p.dr[b]), m));
-        } else if (NU == 1) { // c0 = -psi3, c1 = psi2
-            hr[b] = p2_add(p.ur[b], sgn<-SG, SG>(p2_swp(p.dr[b]), m));
-            hi[b] = p2_add(p.ui[b], sgn<-SG, SG>(p2_swp(p.di[b]), m));
-        } else if (NU == 2) { // c0 = -i psi2 = (psi2.im, -psi2.re), c1 = i psi3 = (-psi3.im, psi3.re)
-            hr[b] = p2_add(p.ur[b], sgn<SG, -SG>(p.di[b], m));
-            hi[b] = p2_add(p.ui[b], sgn<-SG, SG>(p.dr[b], m));
-        } else {              // c0 = psi2, c1 = psi3
-            hr[b] = p2_add(p.ur[b], sgn<SG, SG>(p.dr[b], m));
-            hi[b] = p2_add(p.ui[b], sgn<SG, SG>(p.di[b], m));
+        if (EVEN) {   // x: c = -i (psi3, psi2); z: c = -i (psi2, -psi3)
+            hr[b] = p2_add(p.ur[b], sgn(p.di[b], k));
+            hi[b] = p2_add(p.ui[b], sgn(p.dr[b], k ^ kNeg));
+        } else {      // y: c = (-psi3, psi2); t: c = (psi2, psi3)
+            hr[b] = p2_add(p.ur[b], sgn(p.dr[b], k));
+            hi[b] = p2_add(p.ui[b], sgn(p.di[b], k));
         }
         nhi[b] = p2_neg(hi[b]);
     }
-    P2 wt;   // the temporal weight e^{+-mu} with the boundary sign (t hops only)
-    if (NU == 3) {
+    const bool temporal = !EVEN && !swap;
+    P2 wt = {0ull, 0ull};   // the temporal weight e^{+-mu} with the boundary sign (t hops only)
+    if (temporal) {
         const df w = fwd ? wm_t : wp_t;
         const float f = S.fl[H * kDfSites + tx];
         wt = {pk(w.hi * f, w.hi * f), pk(w.lo * f, w.lo * f)};
@@ -177,24 +173,20 @@ __device__ __forceinline__ void df_hop(DSpin& acc, const dfc* __restrict__ in, i
             p2_add_prod(xr, mi, nhi[b]);   // re: mr hr - mi hi
             p2_add_prod(xi, mi, hr[b]);    // im: mr hi + mi hr
         }
-        if (NU == 3) {
-            xr = p2_prod(wt, xr);
-            xi = p2_prod(wt, xi);
+        if (!EVEN) {
+            if (temporal) {
+                xr = p2_prod(wt, xr);
+                xi = p2_prod(wt, xi);
+            }
         }
         acc.ur[a] = p2_add(acc.ur[a], xr);
         acc.ui[a] = p2_add(acc.ui[a], xi);
-        if (NU == 0) {        // b0 = i x1, b1 = i x0: (-x1.im, -x0.im), (x1.re, x0.re)
-            acc.dr[a] = p2_add(acc.dr[a], sgn<-SG, -SG>(p2_swp(xi), m));
-            acc.di[a] = p2_add(acc.di[a], sgn<SG, SG>(p2_swp(xr), m));
-        } else if (NU == 1) { // b0 = x1, b1 = -x0
-            acc.dr[a] = p2_add(acc.dr[a], sgn<SG, -SG>(p2_swp(xr), m));
-            acc.di[a] = p2_add(acc.di[a], sgn<SG, -SG>(p2_swp(xi), m));
-        } else if (NU == 2) { // b0 = i x0 = (-x0.im, x0.re), b1 = -i x1 = (x1.im, -x1.re)
-            acc.dr[a] = p2_add(acc.dr[a], sgn<-SG, SG>(xi, m));
-            acc.di[a] = p2_add(acc.di[a], sgn<SG, -SG>(xr, m));
-        } else {              // b0 = x0, b1 = x1
-            acc.dr[a] = p2_add(acc.dr[a], sgn<SG, SG>(xr, m));
-            acc.di[a] = p2_add(acc.di[a], sgn<SG, SG>(xi, m));
+        if (EVEN) {   // lanes as accumulated, x: (b1, b0) = i (x0, x1); z: (b0, b1) = i (x0, -x1)
+            acc.dr[a] = p2_add(acc.dr[a], sgn(xi, k ^ kNeg));
+            acc.di[a] = p2_add(acc.di[a], sgn(xr, k));
+        } else {      // y: (b1, b0) = (-x0, x1); t: (b0, b1) = (x0, x1)
+            acc.dr[a] = p2_add(acc.dr[a], sgn(xr, k));
+            acc.di[a] = p2_add(acc.di[a], sgn(xi, k));
         }
     }
 }
@@ -228,16 +220,23 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
 #pragma unroll
     for (int a = 0; a < 3; ++a) acc.ur[a] = acc.ui[a] = acc.dr[a] = acc.di[a] = P2{0ull, 0ull};
 #pragma unroll 1
-    for (int f = 0; f < 2; ++f) df_hop<0>(acc, in, g.V, S, wp_t, wm_t, f);
+    for (int pair = 0; pair < 2; ++pair) {   // x, y, then z, t
+        const bool swap = pair == 0;
 #pragma unroll 1
-    for (int f = 0; f < 2; ++f) df_hop<1>(acc, in, g.V, S, wp_t, wm_t, f);
+        for (int f = 0; f < 2; ++f) df_hop<true>(acc, in, g.V, S, wp_t, wm_t, swap, f);
 #pragma unroll 1
-    for (int f = 0; f < 2; ++f) df_hop<2>(acc, in, g.V, S, wp_t, wm_t, f);
-#pragma unroll 1
-    for (int f = 0; f < 2; ++f) df_hop<3>(acc, in, g.V, S, wp_t, wm_t, f);
+        for (int f = 0; f < 2; ++f) df_hop<false>(acc, in, g.V, S, wp_t, wm_t, swap, f);
+        if (swap) {   // the lower accumulators in their own lanes from here on
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                acc.dr[a] = p2_swp(acc.dr[a]);
+                acc.di[a] = p2_swp(acc.di[a]);
+            }
+        }
+    }
     if (site0 + (int)threadIdx.x >= g.V) return;
     DSpin p;
-    load_dspin(in, g.V, site, p);
+    load_dspin(in, g.V, site, p, false);
     const P2 K = {pk(kappa.hi, kappa.hi), pk(kappa.lo, kappa.lo)};
     P2 SR, SI;   // the scale 1/n_j (1/m_j), two-float from its FP64 value
     const bool scaled = s.scale != nullptr;
