@@ -4,7 +4,8 @@
 // steps cannot recover.
 //
 // One CTA owns a block of kDfSites consecutive sites for every vector of the
-// launch (threadIdx.x = site in the block, threadIdx.y = vector).  Before any
+// launch (threadIdx.x = site in the block, threadIdx.y = vector, for few vectors
+// two threads of one).  Before any
 // vector is touched the CTA stages, in shared memory, the links of its sites'
 // eight hops in the form the arithmetic uses -- M = U(x - nu) for the backward
 // hops, M = U(x)^dagger for the forward ones, each element's real and
@@ -200,6 +201,25 @@ __device__ __forceinline__ void p2_to_double(P2 v, double& l0, double& l1) {
     l1 = f2d_int(s1) + f2d_int(e1);
 }
 
+// the value of the lane 8 away, within the 16 lanes of one vector
+__device__ __forceinline__ P2 shfl_half(P2 v) {
+    const unsigned lanes = 0xffffu << (threadIdx.y & 2 ? 16 : 0);
+    return {__shfl_xor_sync(lanes, (unsigned long long)v.s, 8), __shfl_xor_sync(lanes, (unsigned long long)v.e, 8)};
+}
+
+// SPLIT = 2: two threads share a site and vector, one takes the backward and one
+// the forward hops, and each finishes one spin pair (24 words exchanged, 6 sums).
+// Half the work a thread fills a launch of few vectors' lanes and halves its last
+// wave; it costs the exchange and a CTA of twice the threads.  Measured, one
+// application, 1 -> 2 threads: 10^4 sites, 1 vector 32.8 -> 20.0 us, 3 31.3 ->
+// 27.0, 6 45.9 -> 37.1, 8 46.9 -> 44.4; 16^3 x 32, 1 461 -> 251, 6 500 -> 452.
+// Where many waves hide the last one only the exchange is left: 8 at 16384 sites
+// 67.3 -> 68.7, at 131072 506 -> 528; 12 at 8^4 inside a step 31 -> 33.
+constexpr int kDfSplit = 6;            // vectors up to which two threads always win,
+constexpr int kDfSplitSmall = 8;       // and up to which they do on a lattice of
+constexpr int kDfSplitSites = 12288;   // at most this many sites
+
+template <int SPLIT>
 __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __restrict__ U, Geom g, StencilDfSet s,
                                                               df kappa, df emu, df emu_inv) {
     extern __shared__ __align__(16) char smem[];
@@ -209,7 +229,7 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
     pdl_trigger();
     df_stage(U, g, site0, S);   // (the links: nothing that a stream may still run here writes them)
     pdl_wait();
-    const int v = threadIdx.y;
+    const int v = threadIdx.y / SPLIT, half = threadIdx.y % SPLIT;
     if (v >= s.n_a + s.n_d) return;
     const int side = v < s.n_a ? 0 : 1;
     const int vi = side ? v - s.n_a : v;
@@ -223,9 +243,9 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
     for (int pair = 0; pair < 2; ++pair) {   // x, y, then z, t
         const bool swap = pair == 0;
 #pragma unroll 1
-        for (int f = 0; f < 2; ++f) df_hop<true>(acc, in, g.V, S, wp_t, wm_t, swap, f);
+        for (int f = half; f < 2; f += SPLIT) df_hop<true>(acc, in, g.V, S, wp_t, wm_t, swap, f);
 #pragma unroll 1
-        for (int f = 0; f < 2; ++f) df_hop<false>(acc, in, g.V, S, wp_t, wm_t, swap, f);
+        for (int f = half; f < 2; f += SPLIT) df_hop<false>(acc, in, g.V, S, wp_t, wm_t, swap, f);
         if (swap) {   // the lower accumulators in their own lanes from here on
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -234,9 +254,15 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
             }
         }
     }
+    if (SPLIT == 2) {   // this thread's spin pair (in ur, ui), summed over both senses
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const P2 gr = shfl_half(half ? acc.ur[a] : acc.dr[a]), gi = shfl_half(half ? acc.ui[a] : acc.di[a]);
+            acc.ur[a] = p2_add(half ? acc.dr[a] : acc.ur[a], gr);
+            acc.ui[a] = p2_add(half ? acc.di[a] : acc.ui[a], gi);
+        }
+    }
     if (site0 + (int)threadIdx.x >= g.V) return;
-    DSpin p;
-    load_dspin(in, g.V, site, p, false);
     const P2 K = {pk(kappa.hi, kappa.hi), pk(kappa.lo, kappa.lo)};
     P2 SR, SI;   // the scale 1/n_j (1/m_j), two-float from its FP64 value
     const bool scaled = s.scale != nullptr;
@@ -246,26 +272,28 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
         SR = {pk(zr.hi, zr.hi), pk(zr.lo, zr.lo)};
         SI = {pk(zi.hi, zi.hi), pk(zi.lo, zi.lo)};
     }
+    const float4* __restrict__ f = reinterpret_cast<const float4*>(in) + site;
     double2* __restrict__ out = (side ? s.out_d : s.out_a) + (size_t)vi * s.out_stride;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        // gamma5 = diag(1, 1, -1, -1): upper spins psi - kappa acc, lower kappa acc - psi
-        P2 yr[2], yi[2];
-        yr[0] = p2_add(p.ur[a], p2_neg(p2_prod(K, acc.ur[a])));
-        yi[0] = p2_add(p.ui[a], p2_neg(p2_prod(K, acc.ui[a])));
-        yr[1] = p2_add(p2_prod(K, acc.dr[a]), p2_neg(p.dr[a]));
-        yi[1] = p2_add(p2_prod(K, acc.di[a]), p2_neg(p.di[a]));
 #pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-            P2 orr = yr[hf], oii = yi[hf];
+        for (int q = 0; q < 2; q += SPLIT) {
+            const int hf = SPLIT == 2 ? half : q;   // spins 2 hf, 2 hf + 1
+            const int c0 = 6 * hf + a, c1 = c0 + 3;
+            const float4 s0 = __ldg(f + (size_t)c0 * g.V), s1 = __ldg(f + (size_t)c1 * g.V);
+            const P2 pr = {pk(s0.x, s1.x), pk(s0.y, s1.y)}, pi = {pk(s0.z, s1.z), pk(s0.w, s1.w)};
+            const P2 kr = p2_prod(K, q ? acc.dr[a] : acc.ur[a]), ki = p2_prod(K, q ? acc.di[a] : acc.ui[a]);
+            // gamma5 = diag(1, 1, -1, -1): upper spins psi - kappa acc, lower kappa acc - psi
+            P2 orr = hf ? p2_add(kr, p2_neg(pr)) : p2_add(pr, p2_neg(kr));
+            P2 oii = hf ? p2_add(ki, p2_neg(pi)) : p2_add(pi, p2_neg(ki));
             if (scaled) {   // (yr + i yi)(sr + i si)
-                orr = p2_add(p2_prod(SR, yr[hf]), p2_prod(SI, p2_neg(yi[hf])));
-                oii = p2_add(p2_prod(SI, yr[hf]), p2_prod(SR, yi[hf]));
+                const P2 yr = orr, yi = oii;
+                orr = p2_add(p2_prod(SR, yr), p2_prod(SI, p2_neg(yi)));
+                oii = p2_add(p2_prod(SI, yr), p2_prod(SR, yi));
             }
             double r0, r1, i0, i1;
             p2_to_double(orr, r0, r1);
             p2_to_double(oii, i0, i1);
-            const int c0 = 3 * (2 * hf) + a, c1 = c0 + 3;
             out[s.out_abi ? (size_t)site * 12 + c0 : (size_t)c0 * g.V + site] = make_double2(r0, i0);
             out[s.out_abi ? (size_t)site * 12 + c1 : (size_t)c1 * g.V + site] = make_double2(r1, i1);
         }
@@ -282,17 +310,21 @@ df df_of_host(double d) {
 }  // namespace
 
 void stencil_df_init_attributes() {
-    cudaFuncSetAttribute(k_stencil_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)df_smem());
+    cudaFuncSetAttribute(k_stencil_df<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)df_smem());
+    cudaFuncSetAttribute(k_stencil_df<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)df_smem());
 }
 
 void launch_stencil_df(const void* Udf, const Geom& g, const StencilDfSet& s, double kappa, double mu,
                        cudaStream_t st) {
     const int nv = s.n_a + s.n_d;
     if (nv == 0) return;
-    const dim3 block(kDfSites, nv);
     const unsigned grid = (unsigned)((g.V + kDfSites - 1) / kDfSites);
-    launch_kernel(k_stencil_df, grid, block, df_smem(), st, !s.scale, (const dfc*)Udf, g, s, df_of_host(kappa),
-                  df_of_host(exp(mu)), df_of_host(exp(-mu)));
+#define NK_DF(SPLIT_)                                                                                        \
+    launch_kernel(k_stencil_df<SPLIT_>, grid, dim3(kDfSites, SPLIT_ * nv), df_smem(), st, !s.scale, (const dfc*)Udf, \
+                  g, s, df_of_host(kappa), df_of_host(exp(mu)), df_of_host(exp(-mu)))
+    if (nv <= kDfSplit || (nv <= kDfSplitSmall && g.V <= kDfSplitSites)) NK_DF(2);
+    else NK_DF(1);
+#undef NK_DF
 }
 
 }  // namespace nk
