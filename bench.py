@@ -434,13 +434,13 @@ def dominant_roofline(dom, tc, nc, w, peaks, sm_mhz):
         r = {"kernel": kernel, "bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
              "frac": tf / FP64_PEAK_TFLOPS, "ms_per_launch": ms, "flops_per_launch": flops,
              "peak_derivation": "nominal dense FP64 rate of GB300 (1.25 TFLOP/s, 152 SMs); a DFMA throughput "
-                                "test on this pool measured 0.59-0.63 T DFMA/s, i.e. the same"}
+                                "test measured 0.59-0.63 T DFMA/s, i.e. the same"}
         r.update(extra or {})
         return r
 
     if dom == "step2":
         t1, t2 = profiled_traffic("k_step1"), profiled_traffic("k_step2")   # the FP32-step pair
-        return alu64("k_step1 / k_step2 (FP64 recurrence, operands staged by bulk copies)",
+        return alu64("k_step1 / k_step2 (FP64 recurrence)",
                      (24 if two else 8) * N * n_rhs,
                      {"traffic": (t1 + t2) / 2 if (t1 is not None and t2 is not None) else None,
                       "algorithmic_bytes_per_launch": (104 if two else 56) * N * n_rhs})
@@ -451,7 +451,7 @@ def dominant_roofline(dom, tc, nc, w, peaks, sm_mhz):
                 "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm, "ms_per_launch": ms,
                 "bytes_per_launch": nbytes, "traffic": profiled_traffic("k_stencil32@10x10x10x10")}
     if dom == "lift":
-        return alu64("k_lift (FP64)", 8.0 * N * n_rhs * w["k"], {"traffic": None})
+        return alu64("k_lift (FP64)", (8.0 if two else 4.0) * N * n_rhs * w["k"], {"traffic": None})
     if dom == "dslash_df":
         flops = 1320.0 * V * nv
         tf = flops / (ms * 1e-3) / 1e12

@@ -12,7 +12,7 @@
 // complex multiply-adds per CTA: 4096 clocks of the FP64 pipe at l = 128, C = 8)
 // and a chain of dependent steps -- multipliers, the next column, the pivot
 // search, the inverse of the pivot, the exchange through the cluster.  Run one after the other
-// (the earlier form: 6 us per pivot at l = 128) the chain costs as much again
+// (the earlier form: 8 us per pivot at l = 128) the chain costs as much again
 // as the update, so here it runs one pivot ahead: four warps per CTA form the
 // next pivot column from the rows as they are, choose their candidate, update
 // and publish its row (and row c + 1) and arrive at the cluster barrier; then
