@@ -215,9 +215,18 @@ __device__ __forceinline__ P2 shfl_half(P2 v) {
 // 27.0, 6 45.9 -> 37.1, 8 46.9 -> 44.4; 16^3 x 32, 1 461 -> 251, 6 500 -> 452.
 // Where many waves hide the last one only the exchange is left: 8 at 16384 sites
 // 67.3 -> 68.7, at 131072 506 -> 528; 12 at 8^4 inside a step 31 -> 33.
+// At 9 to 12 vectors a CTA of one thread each is three warps, which fill the four
+// schedulers unevenly: there two threads win once many waves follow one another
+// (12 vectors: 228 -> 208 us at 32768, 455 -> 409 at 65536; a step of
+// 12^4, 6 two-sided sources, 209 -> 202), and not before (10^4, 12 sources 98 -> 100).
 constexpr int kDfSplit = 6;            // vectors up to which two threads always win,
-constexpr int kDfSplitSmall = 8;       // and up to which they do on a lattice of
-constexpr int kDfSplitSites = 12288;   // at most this many sites
+constexpr int kDfSplitSmall = 8;       // up to which on a lattice of at most,
+constexpr int kDfSplitLarge = 12;      // up to which on one of more than
+constexpr int kDfSplitSites = 12288;   // this many sites
+
+bool df_split(int nv, int V) {
+    return nv <= kDfSplit || (nv <= kDfSplitSmall ? V <= kDfSplitSites : nv <= kDfSplitLarge && V > kDfSplitSites);
+}
 
 template <int SPLIT>
 __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __restrict__ U, Geom g, StencilDfSet s,
@@ -322,7 +331,7 @@ void launch_stencil_df(const void* Udf, const Geom& g, const StencilDfSet& s, do
 #define NK_DF(SPLIT_)                                                                                        \
     launch_kernel(k_stencil_df<SPLIT_>, grid, dim3(kDfSites, SPLIT_ * nv), df_smem(), st, !s.scale, (const dfc*)Udf, \
                   g, s, df_of_host(kappa), df_of_host(exp(mu)), df_of_host(exp(-mu)))
-    if (nv <= kDfSplit || (nv <= kDfSplitSmall && g.V <= kDfSplitSites)) NK_DF(2);
+    if (df_split(nv, g.V)) NK_DF(2);
     else NK_DF(1);
 #undef NK_DF
 }

@@ -52,7 +52,7 @@ def test_alone(dims, n, antiperiodic):
 
 
 @pytest.mark.parametrize("dims", [(16, 16, 16, 3), (17, 16, 16, 3)])
-@pytest.mark.parametrize("n", [6, 7, 8])
+@pytest.mark.parametrize("n", [6, 7, 8, 9, 12, 13])
 def test_rule_by_sites(dims, n):
     """On both sides of 12288 sites, against the FP64 stencil."""
     ctx, _ = make_ctx(dims, 0.2)
