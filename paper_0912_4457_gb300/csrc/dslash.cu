@@ -545,9 +545,9 @@ __global__ void f32pair_to_abi(const float4* __restrict__ in, long in_stride, do
     out[(size_t)vec * out_stride + (size_t)site * 12 + 2 * pr + 1] = make_double2(v.z, v.w);
 }
 
-// ABI spinor [site][12] -> two-float [12][V], n vectors
-__global__ void abi_to_df(const double2* __restrict__ in, long in_stride, dfc* __restrict__ out, long out_stride,
-                          int V, int n) {
+// ABI spinor [site][12] -> two-float [12][V], n vectors (a dependent launch: `in` is read
+// by ordinary loads, nk_common.cuh)
+__global__ void abi_to_df(const double2* in, long in_stride, dfc* out, long out_stride, int V, int n) {
     pdl_trigger();
     pdl_wait();
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;   // (vector, site, component)

@@ -12,7 +12,10 @@ namespace nk {
 // kernel's CTAs are placed, and stage the links, as soon as every CTA of the
 // kernel before it in the stream has started and passed pdl_trigger; it touches
 // no vector before pdl_wait, which returns once the kernels before it have
-// completed and their writes are visible.  A caller that applies the operator again
+// completed and their writes are visible to ordinary loads.  It is alive while
+// they still write, so its vectors are no read-only data of the grid: they are
+// read by ordinary loads (no __ldg, no const __restrict__ pointer, which would
+// also let the compiler move a load above the wait).  A caller that applies the operator again
 // and again then has no launch gap and a filled last wave: FP32 stencil, 24 vectors at 10^4,
 // 22.5 -> 19.0 us.  Behind a kernel without pdl_trigger it is an ordinary launch.
 // Inside an outer recurrence the kernels are launched plainly: there the
@@ -20,6 +23,15 @@ namespace nk {
 // 33 with an early trigger; 6^4, one source, 20.9 -> 22.6).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// An ordinary load that stays below a pdl_wait before it (volatile statements keep
+// their order).
+__device__ __forceinline__ float4 ld_after_wait(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p));
+    return v;
+}
 template <typename... P, typename... A>
 inline void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool dependent,
                           A... args) {

@@ -75,10 +75,12 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
-__device__ __forceinline__ void load_spinor32(const float4* __restrict__ in, int V, int s, float2 p[4][3]) {
+// (ordinary loads: the vectors may have been written while this grid was already
+// alive, see nk_common.cuh)
+__device__ __forceinline__ void load_spinor32(const float4* in, int V, int s, float2 p[4][3]) {
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        const float4 v = __ldg(in + (size_t)i * V + s);
+        const float4 v = ld_after_wait(in + (size_t)i * V + s);
         const int c0 = 2 * i, c1 = 2 * i + 1;
         p[c0 / 3][c0 % 3] = make_float2(v.x, v.y);
         p[c1 / 3][c1 % 3] = make_float2(v.z, v.w);
@@ -131,7 +133,7 @@ __device__ __forceinline__ void s32_stage_end() {
 // One hop: the neighbour spinor straight from global memory (L1 / L2), the
 // link from shared memory.
 template <int H>
-__device__ __forceinline__ void s32_hop(float2 acc[4][3], const float4* __restrict__ in, int V, const S32Smem& S,
+__device__ __forceinline__ void s32_hop(float2 acc[4][3], const float4* in, int V, const S32Smem& S,
                                         float wp_t, float wm_t) {
     constexpr int NU = H >> 1;
     constexpr bool FWD = (H & 1) != 0;
@@ -153,7 +155,7 @@ __device__ __forceinline__ void s32_hop(float2 acc[4][3], const float4* __restri
 // out = gamma5 (psi - kappa * sum of the eight hops) at this thread's site
 // (clamped to the lattice), for the vector `in`; side 1 (A^dagger) exchanges
 // the temporal weights.
-__device__ __forceinline__ void s32_site(const float4* __restrict__ in, int V, int site, const S32Smem& S, int side,
+__device__ __forceinline__ void s32_site(const float4* in, int V, int site, const S32Smem& S, int side,
                                          float kappa, float emu, float emu_inv, float2 out[4][3]) {
     const float wp_t = side ? emu_inv : emu;
     const float wm_t = side ? emu : emu_inv;

@@ -59,7 +59,7 @@ __device__ __forceinline__ size_t comp_at(int c, int site, int V) {
 // The coordinate of `site` along nu decides the neighbour; sites past V use V - 1.
 // CG: read `in` past the L1 cache (vectors that the running kernel itself writes).
 template <int S, int SPLIT, bool ABI, bool CG = false>
-__device__ __forceinline__ void s64_hops(const double2* __restrict__ U, const double2* __restrict__ in, const Geom& g,
+__device__ __forceinline__ void s64_hops(const double2* __restrict__ U, const double2* in, const Geom& g,
                                          int site0, double2* __restrict__ sx, int tid) {
     constexpr int ROWS = 3 / SPLIT;
     const int s = tid % S, hc = (tid / S) & 15, a0 = SPLIT == 1 ? 0 : tid / (16 * S);
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(16 * S) k_stencil64(const double2* __restrict_
     const int vec = blockIdx.x % nvec, site0 = (blockIdx.x / nvec) * S;
     const DslashSet& D = vec < s0.n ? s0 : s1;
     const int vi = vec < s0.n ? vec : vec - s0.n;
-    const double2* __restrict__ in = reinterpret_cast<const double2*>(D.in) + (size_t)vi * D.in_stride;
+    const double2* in = reinterpret_cast<const double2*>(D.in) + (size_t)vi * D.in_stride;   // ordinary loads (nk_common.cuh)
     s64_hops<S, 1, ABI>(U, in, g, site0, sx, threadIdx.x);
     // component-fastest threads in the ABI layout, site-fastest in the device one (coalesced
     // stores).  12 of 16 threads sum: which warps idle rotates with the block of sites, as

@@ -93,15 +93,17 @@ struct DSpin {
 };
 
 // the two-float spinor of site s (components 3 sp + b, each (re.hi, re.lo,
-// im.hi, im.lo)) in the spin-pair lanes; SWAP exchanges the lanes of the lower pair
-__device__ __forceinline__ void load_dspin(const dfc* __restrict__ in, int V, int s, DSpin& p, bool swap) {
+// im.hi, im.lo)) in the spin-pair lanes; SWAP exchanges the lanes of the lower pair.
+// Ordinary loads: the vectors may have been written while this grid was already alive
+// (nk_common.cuh).
+__device__ __forceinline__ void load_dspin(const dfc* in, int V, int s, DSpin& p, bool swap) {
     const float4* f = reinterpret_cast<const float4*>(in) + s;
     const float4* f2 = f + (size_t)(swap ? 9 : 6) * V;
     const float4* f3 = f + (size_t)(swap ? 6 : 9) * V;
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-        const float4 s0 = __ldg(f + (size_t)b * V), s1 = __ldg(f + (size_t)(3 + b) * V);
-        const float4 s2 = __ldg(f2 + (size_t)b * V), s3 = __ldg(f3 + (size_t)b * V);
+        const float4 s0 = ld_after_wait(f + (size_t)b * V), s1 = ld_after_wait(f + (size_t)(3 + b) * V);
+        const float4 s2 = ld_after_wait(f2 + (size_t)b * V), s3 = ld_after_wait(f3 + (size_t)b * V);
         p.ur[b] = {pk(s0.x, s1.x), pk(s0.y, s1.y)};
         p.ui[b] = {pk(s0.z, s1.z), pk(s0.w, s1.w)};
         p.dr[b] = {pk(s2.x, s3.x), pk(s2.y, s3.y)};
@@ -128,7 +130,7 @@ __device__ __forceinline__ P2 sgn(P2 a, f2p m) { return {a.s ^ m, a.e ^ m}; }
 // hops overflowed the instruction cache, and with one instantiation per
 // direction a warp still waited 0.7 of 6 cycles per instruction for it.
 template <bool EVEN>
-__device__ __forceinline__ void df_hop(DSpin& acc, const dfc* __restrict__ in, int V, const DfSmem& S, df wp_t,
+__device__ __forceinline__ void df_hop(DSpin& acc, const dfc* in, int V, const DfSmem& S, df wp_t,
                                        df wm_t, bool swap, int fwd) {
     const int H = 2 * ((swap ? 0 : 2) + (EVEN ? 0 : 1)) + fwd;
     const f2p m = fwd ? kNeg : 0ull;
@@ -242,7 +244,7 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
     if (v >= s.n_a + s.n_d) return;
     const int side = v < s.n_a ? 0 : 1;
     const int vi = side ? v - s.n_a : v;
-    const dfc* __restrict__ in = (side ? s.in_d : s.in_a) + (size_t)vi * s.in_stride;
+    const dfc* in = (side ? s.in_d : s.in_a) + (size_t)vi * s.in_stride;
     // temporal weights: A uses (e^{mu}, e^{-mu}); A^dagger exchanges them
     const df wp_t = side ? emu_inv : emu, wm_t = side ? emu : emu_inv;
     DSpin acc;
@@ -281,15 +283,15 @@ __global__ void __launch_bounds__(kDfMaxThreads, 2) k_stencil_df(const dfc* __re
         SR = {pk(zr.hi, zr.hi), pk(zr.lo, zr.lo)};
         SI = {pk(zi.hi, zi.hi), pk(zi.lo, zi.lo)};
     }
-    const float4* __restrict__ f = reinterpret_cast<const float4*>(in) + site;
-    double2* __restrict__ out = (side ? s.out_d : s.out_a) + (size_t)vi * s.out_stride;
+    const float4* f = reinterpret_cast<const float4*>(in) + site;
+    double2* out = (side ? s.out_d : s.out_a) + (size_t)vi * s.out_stride;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
 #pragma unroll
         for (int q = 0; q < 2; q += SPLIT) {
             const int hf = SPLIT == 2 ? half : q;   // spins 2 hf, 2 hf + 1
             const int c0 = 6 * hf + a, c1 = c0 + 3;
-            const float4 s0 = __ldg(f + (size_t)c0 * g.V), s1 = __ldg(f + (size_t)c1 * g.V);
+            const float4 s0 = ld_after_wait(f + (size_t)c0 * g.V), s1 = ld_after_wait(f + (size_t)c1 * g.V);
             const P2 pr = {pk(s0.x, s1.x), pk(s0.y, s1.y)}, pi = {pk(s0.z, s1.z), pk(s0.w, s1.w)};
             const P2 kr = p2_prod(K, q ? acc.dr[a] : acc.ur[a]), ki = p2_prod(K, q ? acc.di[a] : acc.ui[a]);
             // gamma5 = diag(1, 1, -1, -1): upper spins psi - kappa acc, lower kappa acc - psi
