@@ -339,7 +339,8 @@ __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict
     __shared__ double2 sx[kRunGroups][48 * kRunSites];
     __shared__ double2 sh[33];
     __shared__ double2 sc[kScalars];
-    __shared__ bool ok_sh;
+    __shared__ bool ok_sh;   // a barrier's outcome (written inside run_barrier only)
+    __shared__ bool go_sh;   // no breakdown at this step
     const int rhs = blockIdx.x % o.n_rhs, cta = blockIdx.x / o.n_rhs, ncta = gridDim.x / o.n_rhs;
     if (o.status[rhs] != kStatusOK) return;
     const int tid = threadIdx.x, grp = tid / 64, gt = tid % 64, warp = tid / 32, lane = tid % 32;
@@ -476,12 +477,12 @@ __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict
                     o.gamma[(size_t)rhs * o.k + j] = t.gamma;
                     if (!t.ok) mark_failed(o, rhs, kStatusBreakdown);
                 }
-                ok_sh = t.ok;
+                go_sh = t.ok;
                 if (t.ok) next_scalars<TS>(sc, t);
             }
         }
         __syncthreads();
-        if (!ok_sh) return;   // the same decision in every CTA of the RHS
+        if (!go_sh) return;   // the same decision in every CTA of the RHS
     }
     if (cta == 0 && tid < kScalars && j_hi < o.k) o.sc[(size_t)rhs * kScalars + tid] = sc[tid];
 }
