@@ -67,7 +67,9 @@ extern "C" {
 #define NK_ASYNC 0x40u      /* nk_sign_apply_dev / nk_overlap_apply_dev with tol = 0: enqueue the
                                solve and return without waiting; nk_wait collects its outcome.
                                One pending solve per context (its workspace); two contexts on two
-                               streams keep two batches in flight.  Until nk_wait, the calls that
+                               streams keep two batches in flight (the kernels leave room for
+                               one another; a blocking solve of a small FP64 batch may hold the
+                               chip from its first step to its last).  Until nk_wait, the calls that
                                write the context's workspace, links or deflation vectors (the
                                solves, nk_load_links(_dev), nk_set_deflation, nk_eigs_smallest,
                                nk_autotune, nk_outer_lanczos_dev, nk_inner_sign, nk_features,
@@ -271,8 +273,9 @@ int nk_set_adapt_start(nk_ctx* ctx, int k_first);
  *                   vector.  The multi-RHS stencils of NK_MIXED have one shape.
  * An FP64 recurrence on a small batch (V n_rhs, times 2 for mu != 0, up to 32768)
  * with no shape set or tuned runs all its steps in one cooperative launch instead
- * (needs every one of its CTAs, at most one per SM, resident at once; a device
- * without cooperative launches runs step by step).
+ * (needs every one of its CTAs, at most one per SM, resident at once), or, with
+ * NK_ASYNC or on a device without cooperative launches, in one launch per half
+ * step of the same CTAs: the same bits either way.
  * A shape belongs to (n_rhs, sidedness of the current mu (mu != 0), the
  * NK_MIXED bit of flags).  Different shapes sum in different orders, so
  * results differ at rounding level; one shape is bitwise reproducible.

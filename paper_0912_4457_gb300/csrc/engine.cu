@@ -357,6 +357,7 @@ int check_solve_args(nk_ctx* c, int n_rhs, int k, int ell, double tol) {
 struct Launcher {
     cudaStream_t st;
     bool profile = false;
+    bool alone = true;   // nothing else is expected on the chip (no NK_ASYNC)
     int launches = 0;
     int n_class[NK_NCLASS] = {0};
     std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> marks;
@@ -416,12 +417,15 @@ int copy_mode_for(const Schedule& s, int j) {
 // Whether the FP64 steps of this recurrence run as one cooperative launch
 // (k_run64): a small batch -- up to kRunSiteVecs sites times vectors, beyond which
 // the FP64 pipe hides the step kernels' launches and tails and their finer grain
-// wins (measured us per step, run against step kernels: 6^4 x 2 vectors 16.7 / 21.3,
-// 10^4 x 2 53.9 / 58.3, 6^4 x 24 78.8 / 80.3, 8^4 x 12 114.7 / 112.4) -- with no launch shape of
-// its own (a set or tuned shape names the kernels of a step).
+// wins (measured us per step, run against step kernels: 6^4 x 2 vectors 17.4 / 21.0,
+// 10^4 x 2 52.2 / 58.1, 6^4 x 24 74.5 / 79.4, 8^4 x 8 74.8 / 79.6, 8^4 x 12 114.7 / 112.4) -- with
+// no launch shape of its own (a set or tuned shape names the kernels of a step).
+// A cooperative launch keeps its SMs for the whole run, so a solve beside others
+// (NK_ASYNC) takes a launch per half step of the same CTAs instead, with the
+// same bits (k_run64_half: eight 6^4 solves in flight 9.5 -> 5.0 ms each, one 16.0 -> 17.5).
 constexpr long kRunSiteVecs = 32768;
 bool run_in_one(const nk_ctx* c, const nk::Outer& o) {
-    if (!c->coop || (long)c->V * o.n_rhs * (o.two_sided ? 2 : 1) > kRunSiteVecs) return false;
+    if ((long)c->V * o.n_rhs * (o.two_sided ? 2 : 1) > kRunSiteVecs) return false;
     return c->tune.count(std::make_tuple(o.n_rhs, o.two_sided ? 1 : 0, 0)) == 0;
 }
 
@@ -441,12 +445,22 @@ void enqueue_outer_steps(nk_ctx* c, const nk::Outer& o, const Schedule& s, int j
     const double kap = kappa_of(c);
     cudaStream_t st = L.st;
     if (!s.mixed && !L.profile && j_end > j_begin && run_in_one(c, o)) {
-        bool ok = true;
-        L.run(NK_CLASS_DSLASH64, 1, [&] {
-            ok = nk::launch_run64(c->U64, g, o, j_begin, j_end, kap, c->mu, std::min(c->sms, kRunMaxCtas), st);
-        });
-        if (ok) return;
-        cudaGetLastError();   // no cooperative launch here: step by step
+        const int ctas = std::min(c->sms, kRunMaxCtas);
+        if (c->coop && L.alone) {
+            bool ok = true;
+            L.run_counted(NK_CLASS_DSLASH64, [&] {
+                ok = nk::launch_run64(c->U64, g, o, j_begin, j_end, kap, c->mu, ctas, st);
+                return ok ? 1 : 0;
+            });
+            if (ok) return;
+            cudaGetLastError();   // no cooperative launch here
+        }
+        for (int j = j_begin; j < j_end; ++j) {
+            L.run(NK_CLASS_DSLASH64, 1, [&] { nk::launch_run64_half(c->U64, g, o, 0, j, kap, c->mu, ctas, st); });
+            if (j == o.k - 1) break;
+            L.run(NK_CLASS_STEP2, 1, [&] { nk::launch_run64_half(c->U64, g, o, 1, j, kap, c->mu, ctas, st); });
+        }
+        return;
     }
     for (int j = j_begin; j < j_end; ++j) {
         const int prec = s.prec(j);
@@ -784,6 +798,7 @@ int solve_core(nk_ctx* c, const double* b_dev, int n_rhs, int k, int ell, double
     Launcher L;
     L.st = st;
     L.profile = profile;
+    L.alone = !async;
     std::vector<int> kused_h(n_rhs, k), notconv(n_rhs, 0);
     int checks = 0;
     double tph[3] = {0.0, 0.0, 0.0};
@@ -802,6 +817,7 @@ int solve_core(nk_ctx* c, const double* b_dev, int n_rhs, int k, int ell, double
             NK_CUDA(c, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
             Launcher Lc;
             Lc.st = cs;
+            Lc.alone = !async;
             cudaError_t e = enqueue_solve(c, Lw, b_dev, y_dev, n_rhs, p, flags, overlap, Lc);
             cudaGraph_t graph;
             cudaError_t e2 = cudaStreamEndCapture(cs, &graph);

@@ -334,16 +334,16 @@ __global__ void __launch_bounds__(kStepThreads, kStepCtasPerSm) k_step1(Outer o,
     if (finish_partial(part, o.partials + (size_t)rhs * o.npart, o.counters + rhs, blockIdx.x, o.nblk)) {
         const double2 a = sum_partials(o.partials + (size_t)rhs * o.npart, o.nblk, sh);
         // Hermitian: H(j,j) = Re(q_j^dag r) / n_j, real (App. C); two-sided: (p_j^dag r) / m_j^*
-        const double2 al = TS ? cmul(sc[kScD], a) : mk(a.x * sc[kScD].x, 0.0);
+        const double2 al = TS ? cmul_fma(sc[kScD], a) : mk(a.x * sc[kScD].x, 0.0);
         const int w = threadIdx.x >> 5;
         if (threadIdx.x == 0) {
             o.alpha[(size_t)rhs * o.k + j] = al;
             o.counters[rhs] = 0u;
         }
         // the step-2 scalars H(j,j)/n_j and H(j,j)^*/m_j from the inverses kScN and kScM
-        if ((threadIdx.x & 31) == 0 && w == 1) o.sc[(size_t)rhs * kScalars + kScC3] = cmul(al, sc[kScN]);
+        if ((threadIdx.x & 31) == 0 && w == 1) o.sc[(size_t)rhs * kScalars + kScC3] = cmul_fma(al, sc[kScN]);
         if ((threadIdx.x & 31) == 0 && w == 2)
-            o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cmul(cconj(al), sc[kScM]) : mk(0.0, 0.0);
+            o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cmul_fma(cconj(al), sc[kScM]) : mk(0.0, 0.0);
     }
 }
 

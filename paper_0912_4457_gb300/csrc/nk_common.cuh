@@ -60,6 +60,11 @@ __host__ __device__ __forceinline__ double2 csub(double2 a, double2 b) { return 
 __host__ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+// a * b as explicit fused multiply-adds: the same bits in every kernel (in a * b - c * d the
+// compiler chooses which product it rounds)
+__device__ __forceinline__ double2 cmul_fma(double2 a, double2 b) {
+    return mk(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
+}
 // conj(a) * b
 __host__ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
     return mk(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
@@ -116,7 +121,7 @@ __device__ __forceinline__ void csqrt_scalars(double2 delta, double2& beta, doub
     const double t = sqrt_inv(0.5 * (m + fabs(d.x)), iv), o = 0.5 * d.y * iv;
     // (t, o) for Re d >= 0, else (|o|, sign(Im d) t)
     const double2 b = d.x >= 0.0 ? mk(t, o) : mk(fabs(o), d.y >= 0.0 ? t : -t);
-    const double2 w = cscale(cmul(d, b), im);
+    const double2 w = cscale(cmul_fma(d, b), im);
     beta = cscale(b, up);
     gamma = cscale(cconj(w), up);
     inv_beta = cscale(cconj(b), im * down);

@@ -39,6 +39,9 @@ int stencil64_blocks(const Geom& g, int threads, int nvec);   // CTAs, hence par
 // False if the launch failed (cudaGetLastError has the reason).
 bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int j_hi, double kappa, double mu, int sms,
                   cudaStream_t st);
+// The same, a launch per half step (same CTAs, same bits): half 0 or 1 of step j.
+void launch_run64_half(const void* U64, const Geom& g, const Outer& o, int half, int j, double kappa, double mu, int sms,
+                       cudaStream_t st);
 void launch_links_to_device_layout(const double2* in, double2* u64, float2* u32, dfc* udf, int V,
                                    cudaStream_t st);
 int plaquette_blocks(const Geom& g);

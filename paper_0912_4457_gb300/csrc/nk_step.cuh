@@ -36,10 +36,10 @@ template <bool TS>
 __device__ __forceinline__ void next_scalars(double2* sc, const StepScalars& t) {
     const double2 inv_n = sc[kScN], inv_m = sc[kScM];
     sc[kScN] = t.inv_beta;
-    sc[kScC1] = cmul(t.gamma, inv_n);              // gamma (Hermitian: beta) / n_j
+    sc[kScC1] = cmul_fma(t.gamma, inv_n);           // gamma (Hermitian: beta) / n_j
     sc[kScD] = t.inv_gamma;
     sc[kScM] = cconj(t.inv_gamma);
-    sc[kScC1L] = cmul(cconj(t.beta), inv_m);
+    sc[kScC1L] = cmul_fma(cconj(t.beta), inv_m);
 }
 
 }  // namespace nk

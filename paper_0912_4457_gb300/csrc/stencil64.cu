@@ -27,6 +27,8 @@
 // colour row of the product its own thread: a third of the chain per thread
 // for 22% more FP64 work (the projection is repeated); it was never faster at
 // the default S = 8 (6^4 28 against 32 us) and level with it at S = 4, 4^4.
+#include <algorithm>
+
 #include "nk_common.cuh"
 #include "nk_kernels.h"
 #include "nk_step.cuh"
@@ -252,8 +254,7 @@ __global__ void __launch_bounds__(16 * S * SPLIT, SPLIT == 1 ? kS64Sites / S : 1
             const double2 v = make_double2(flip(fma(-kappa, acc.x, p.x), sg), flip(fma(-kappa, acc.y, p.y), sg));
             double2 rr;
             if (TS) {
-                rr = make_double2(v.x * scl.x - v.y * scl.y, v.x * scl.y + v.y * scl.x);
-                rr = caxpy_neg(rr, c1, pv);
+                rr = caxpy_neg(cmul_fma(v, scl), c1, pv);
             } else {
                 rr = make_double2(v.x * scl.x, v.y * scl.x);
                 rr = make_double2(fma(-c1.x, pv.x, rr.x), fma(-c1.x, pv.y, rr.y));
@@ -274,13 +275,13 @@ __global__ void __launch_bounds__(16 * S * SPLIT, SPLIT == 1 ? kS64Sites / S : 1
         // Hermitian: H(j,j) = Re(q_j^dag r) / n_j, real (App. C); two-sided: (p_j^dag r) / m_j^*;
         // the step-2 scalars H(j,j)/n_j (warp 1) and H(j,j)^*/m_j (warp 0) side by side
         if (tid == 0 || tid == 32) {
-            const double2 al = TS ? cmul(sc[kScD], tot) : make_double2(tot.x * sc[kScD].x, 0.0);
+            const double2 al = TS ? cmul_fma(sc[kScD], tot) : make_double2(tot.x * sc[kScD].x, 0.0);
             if (tid == 0) {
                 o.alpha[(size_t)rhs * o.k + j] = al;
                 o.counters[rhs] = 0u;
-                o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cmul(cconj(al), sc[kScM]) : make_double2(0.0, 0.0);
+                o.sc[(size_t)rhs * kScalars + kScC4] = TS ? cmul_fma(cconj(al), sc[kScM]) : make_double2(0.0, 0.0);
             } else {
-                o.sc[(size_t)rhs * kScalars + kScC3] = cmul(al, sc[kScN]);
+                o.sc[(size_t)rhs * kScalars + kScC3] = cmul_fma(al, sc[kScN]);
             }
         }
     }
@@ -294,16 +295,18 @@ __global__ void __launch_bounds__(16 * S * SPLIT, SPLIT == 1 ? kS64Sites / S : 1
 // launch, at most one CTA per SM and RHS share, and per step two grid barriers
 // of the RHS's CTAs; after each every CTA adds the partial sums and forms the
 // scalars for itself (the same values in the same order everywhere), so nothing
-// waits for a second hop through memory.  64 threads work on four sites as in
+// waits for a second hop through memory.  128 threads work on eight sites as in
 // k_stencil64_step1 (group of the CTA with its own named barrier), then all on
 // (component pair, site) items as in k_step2.  Vectors written by the launch are
 // read past L1.
 // The barriers' waits are bounded: a CTA whose wait runs out marks its RHS
 // kStatusTimeout and leaves; the others' waits then run out too.
-// Measured, us per step against the step kernels: 4^4, mu = 0 13.5 -> 10.0; 6^4, mu = 0.1
-// 21.3 -> 16.7; 10^4, mu = 0.2 58.3 -> 53.9 (all one source).  256 or 512 threads per CTA:
-// 18.3 and 16.7 at 6^4 (two rounds of groups with 256), 57.4 and 54.3 at 10^4.
-constexpr int kRunThreads = 384, kRunGroups = kRunThreads / 64, kRunSites = 4;
+// Measured, us per step against the step kernels: 4^4, mu = 0 13.5 -> 9.7; 6^4, mu = 0.1
+// 21.0 -> 17.4; 10^4, mu = 0.2 58.1 -> 52.2 (all one source).  Registers capped for two
+// CTAs per SM cost 4% at 10^4 (62.7 -> 65.2 ms a solve of k = 1024); 256 threads per CTA 18.5
+// at 6^4, 55.5 at 10^4.  Groups of 64 threads on four sites leave a quarter of the lanes
+// idle in the sum over the hops: 54 at 10^4.
+constexpr int kRunSites = 8, kRunGroup = 16 * kRunSites, kRunThreads = 384, kRunGroups = kRunThreads / kRunGroup;
 constexpr unsigned long long kRunWaitNs = 1000000000ull;   // one second
 
 __device__ __forceinline__ unsigned long long run_ns() {
@@ -333,6 +336,153 @@ __device__ __forceinline__ bool run_barrier(unsigned* counter, unsigned target, 
     return *ok_sh;
 }
 
+// What the two forms of a run share.  Every CTA of an RHS (`ncta` of them) holds the
+// step's scalars in sc; part1 and part2 are its partial sums of H(j,j) and of delta.
+// The sums below have one order whatever the form, and products of complex
+// scalars are written as explicit fused multiply-adds, so that both forms give
+// the same bits.
+
+// Sum of the ncta partials in every lane of one warp.
+__device__ __forceinline__ double2 run_total(const double2* part, int ncta) {
+    const int lane = threadIdx.x % 32;
+    double2 a = make_double2(0.0, 0.0);
+    for (int i = lane; i < ncta; i += 32) {
+        const double2 v = __ldcg(part + i);
+        a = i == lane ? v : cadd(a, v);
+    }
+    const double t = warp_sum_split(a);
+    return make_double2(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 16));
+}
+
+// First half of step j, stencil and step 1 on this CTA's share of the site blocks;
+// returns the thread's part of H(j,j).
+template <bool TS, bool PASS2>
+__device__ __forceinline__ double2 run_half1(const double2* __restrict__ U, const Geom& g, const Outer& o, int rhs, int j,
+                                             int cta, int ncta, const double2* sc, double2 (*sx)[48 * kRunSites],
+                                             double kappa, double emu, double emu_inv) {
+    const int tid = threadIdx.x, grp = tid / kRunGroup, gt = tid % kRunGroup;
+    const int V = g.V, nsb = (V + kRunSites - 1) / kRunSites;
+    const int jp = j > 0 ? j - 1 : j;
+    const bool left = TS && j < o.k - 1;
+    // the warp that idles in the sum differs from group to group (FP64 pipes, as in k_stencil64)
+    const int t2 = (gt + 32 * (grp & 3)) % kRunGroup;
+    const int s = t2 % kRunSites, comp = t2 / kRunSites, sp = comp / 3, a = comp % 3;
+    const unsigned sg = sp < 2 ? 0u : 0x80000000u;
+    double2 dot = make_double2(0.0, 0.0);
+    for (int u = cta + ncta * grp; u < (left ? 2 : 1) * nsb; u += ncta * kRunGroups) {
+        const int side = u >= nsb ? 1 : 0, b = u - side * nsb;
+        const double2* in = side ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
+        s64_hops<kRunSites, 1, false, true>(U, in, g, b * kRunSites, sx[grp], gt);
+        const int site = b * kRunSites + s;
+        const bool live = comp < 12 && site < V;
+        const size_t idx = (size_t)comp * V + site;
+        double2 p = make_double2(0.0, 0.0), pv = p, d = p;
+        if (live) {
+            p = __ldcg(in + idx);
+            pv = __ldcg((side ? outer_p(o, rhs, jp) : outer_q(o, rhs, jp)) + idx);
+            if (side == 0) d = __ldcg((TS ? outer_p(o, rhs, j) : outer_q(o, rhs, j)) + idx);
+        }
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kRunGroup) : "memory");
+        if (live) {
+            double wp, wm;
+            t_weights(g, site, side, emu, emu_inv, wp, wm);
+            const double2 acc = s64_sum<kRunSites>(sx[grp], s, sp, a, wp, wm);
+            const double2 v = make_double2(flip(fma(-kappa, acc.x, p.x), sg), flip(fma(-kappa, acc.y, p.y), sg));
+            const double2 scl = sc[side ? kScM : kScN], c1 = sc[side ? kScC1L : kScC1];
+            double2 rr;
+            if (TS) {
+                rr = caxpy_neg(cmul_fma(v, scl), c1, pv);
+            } else {
+                rr = make_double2(v.x * scl.x, v.y * scl.x);
+                rr = make_double2(fma(-c1.x, pv.x, rr.x), fma(-c1.x, pv.y, rr.y));
+            }
+            (side ? outer_p(o, rhs, j + 1) : outer_q(o, rhs, j + 1))[idx] = rr;
+            if (side == 0) {
+                dot.x = fma(d.x, rr.x, fma(d.y, rr.y, dot.x));      // conj(d) r
+                if (TS) dot.y = fma(d.x, rr.y, fma(-d.y, rr.x, dot.y));
+                if (PASS2) {
+                    double2* y = o.y + (size_t)rhs * o.N + idx;
+                    *y = caxpy_pos(*y, o.cp[(size_t)rhs * o.k + j], TS ? p : d);
+                }
+            }
+        }
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kRunGroup) : "memory");   // sx is rewritten
+    }
+    return dot;
+}
+
+// H(j,j) and the step-2 scalars, by one warp (an FP64 warp instruction costs its
+// pipe as much as any).  Hermitian: H(j,j) = Re(q_j^dag r) / n_j, real (App. C);
+// two-sided: (p_j^dag r) / m_j^*.
+template <bool TS>
+__device__ __forceinline__ void run_alpha(const Outer& o, int rhs, int j, bool write, int ncta, const double2* part1, double2* sc) {
+    const double2 tot = run_total(part1, ncta);
+    const double2 al = TS ? cmul_fma(sc[kScD], tot) : make_double2(tot.x * sc[kScD].x, 0.0);
+    if (threadIdx.x % 32 == 0) {
+        if (write) o.alpha[(size_t)rhs * o.k + j] = al;
+        sc[kScC3] = cmul_fma(al, sc[kScN]);
+        sc[kScC4] = TS ? cmul_fma(cconj(al), sc[kScM]) : make_double2(0.0, 0.0);
+    }
+}
+
+// Second half of step j on this CTA's share of the (component pair, site) items;
+// returns the thread's part of delta.
+template <bool TS>
+__device__ __forceinline__ double2 run_half2(const Outer& o, int rhs, int j, int cta, int ncta, const double2* sc) {
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const unsigned V = (unsigned)(o.N / 12), items = 6u * V;
+    const double2 c3 = sc[kScC3], c4 = sc[kScC4];
+    const double2* qj = outer_q(o, rhs, j);
+    double2* r = outer_q(o, rhs, j + 1);
+    const double2* pj = TS ? outer_p(o, rhs, j) : nullptr;
+    double2* l = TS ? outer_p(o, rhs, j + 1) : nullptr;
+    double2 del = make_double2(0.0, 0.0);
+    const unsigned stride = (unsigned)ncta * kRunThreads;
+    for (unsigned i = (unsigned)(cta + ncta * warp) * 32u + lane; i < items; i += stride) {
+        const size_t e0 = (size_t)i + (size_t)(i / V) * V;   // component 2 cp of the item
+        double2 q[2], x[2], pv[2], w[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const size_t e = e0 + (size_t)h * V;
+            q[h] = __ldcg(qj + e);
+            x[h] = __ldcg(r + e);
+            if (TS) { pv[h] = __ldcg(pj + e); w[h] = __ldcg(l + e); }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const size_t e = e0 + (size_t)h * V;
+            x[h] = TS ? caxpy_neg(x[h], c3, q[h])
+                      : make_double2(fma(-c3.x, q[h].x, x[h].x), fma(-c3.x, q[h].y, x[h].y));
+            r[e] = x[h];
+            if (TS) {
+                w[h] = caxpy_neg(w[h], c4, pv[h]);
+                l[e] = w[h];
+                del.x = fma(x[h].x, w[h].x, fma(x[h].y, w[h].y, del.x));   // conj(r) l
+                del.y = fma(x[h].x, w[h].y, fma(-x[h].y, w[h].x, del.y));
+            } else {
+                del.x = fma(x[h].x, x[h].x, fma(x[h].y, x[h].y, del.x));
+            }
+        }
+    }
+    return del;
+}
+
+// beta_j, gamma_j and the scalars of step j + 1, by one warp; *go: no breakdown.
+template <bool TS>
+__device__ __forceinline__ void run_beta(const Outer& o, int rhs, int j, bool write, int ncta, const double2* part2, double2* sc,
+                                         bool* go) {
+    const StepScalars t = step_scalars<TS>(run_total(part2, ncta));
+    if (threadIdx.x % 32 == 0) {
+        if (write) {
+            o.beta[(size_t)rhs * o.k + j] = t.beta;
+            o.gamma[(size_t)rhs * o.k + j] = t.gamma;
+            if (!t.ok) mark_failed(o, rhs, kStatusBreakdown);
+        }
+        *go = t.ok;
+        if (t.ok) next_scalars<TS>(sc, t);
+    }
+}
+
 template <bool TS, bool PASS2>
 __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict__ U, Geom g, Outer o, int j_lo, int j_hi,
                                                           double kappa, double emu, double emu_inv) {
@@ -343,148 +493,80 @@ __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict
     __shared__ bool go_sh;   // no breakdown at this step
     const int rhs = blockIdx.x % o.n_rhs, cta = blockIdx.x / o.n_rhs, ncta = gridDim.x / o.n_rhs;
     if (o.status[rhs] != kStatusOK) return;
-    const int tid = threadIdx.x, grp = tid / 64, gt = tid % 64, warp = tid / 32, lane = tid % 32;
-    const int V = g.V, nsb = (V + kRunSites - 1) / kRunSites;
-    const unsigned items = 6u * (unsigned)V;
+    const int tid = threadIdx.x;
     unsigned* counter = o.run_bar + rhs;
     unsigned target = 0;
     double2* part1 = o.partials + (size_t)rhs * o.npart;
     double2* part2 = part1 + ncta;
     if (tid < kScalars) sc[tid] = o.sc[(size_t)rhs * kScalars + tid];
     __syncthreads();
-    // sum of the ncta partials in warp 0 of every CTA (all its lanes)
-    auto total = [&](const double2* part) -> double2 {
-        double2 a = make_double2(0.0, 0.0);
-        for (int i = lane; i < ncta; i += 32) {
-            const double2 v = __ldcg(part + i);
-            a = i == lane ? v : cadd(a, v);
-        }
-        const double t = warp_sum_split(a);
-        return make_double2(__shfl_sync(0xffffffffu, t, 0), __shfl_sync(0xffffffffu, t, 16));
-    };
-    const int s = gt % kRunSites, comp = gt / kRunSites, sp = comp / 3, a = comp % 3;
-    const unsigned sg = sp < 2 ? 0u : 0x80000000u;
     for (int j = j_lo; j < j_hi; ++j) {
-        const int jp = j > 0 ? j - 1 : j;
-        const bool left = TS && j < o.k - 1;
-        // ---- stencil and step 1 ----
-        double2 dot = make_double2(0.0, 0.0);
-        for (int u = cta + ncta * grp; u < (left ? 2 : 1) * nsb; u += ncta * kRunGroups) {
-            const int side = u >= nsb ? 1 : 0, b = u - side * nsb;
-            const double2* in = side ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
-            s64_hops<kRunSites, 1, false, true>(U, in, g, b * kRunSites, sx[grp], gt);
-            const int site = b * kRunSites + s;
-            const bool live = comp < 12 && site < V;
-            const size_t idx = (size_t)comp * V + site;
-            double2 p = make_double2(0.0, 0.0), pv = p, d = p;
-            if (live) {
-                p = __ldcg(in + idx);
-                pv = __ldcg((side ? outer_p(o, rhs, jp) : outer_q(o, rhs, jp)) + idx);
-                if (side == 0) d = __ldcg((TS ? outer_p(o, rhs, j) : outer_q(o, rhs, j)) + idx);
-            }
-            asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");
-            if (live) {
-                double wp, wm;
-                t_weights(g, site, side, emu, emu_inv, wp, wm);
-                const double2 acc = s64_sum<kRunSites>(sx[grp], s, sp, a, wp, wm);
-                const double2 v = make_double2(flip(fma(-kappa, acc.x, p.x), sg), flip(fma(-kappa, acc.y, p.y), sg));
-                const double2 scl = sc[side ? kScM : kScN], c1 = sc[side ? kScC1L : kScC1];
-                double2 rr;
-                if (TS) {
-                    rr = make_double2(v.x * scl.x - v.y * scl.y, v.x * scl.y + v.y * scl.x);
-                    rr = caxpy_neg(rr, c1, pv);
-                } else {
-                    rr = make_double2(v.x * scl.x, v.y * scl.x);
-                    rr = make_double2(fma(-c1.x, pv.x, rr.x), fma(-c1.x, pv.y, rr.y));
-                }
-                (side ? outer_p(o, rhs, j + 1) : outer_q(o, rhs, j + 1))[idx] = rr;
-                if (side == 0) {
-                    dot.x = fma(d.x, rr.x, fma(d.y, rr.y, dot.x));      // conj(d) r
-                    if (TS) dot.y = fma(d.x, rr.y, fma(-d.y, rr.x, dot.y));
-                    if (PASS2) {
-                        double2* y = o.y + (size_t)rhs * o.N + idx;
-                        *y = caxpy_pos(*y, o.cp[(size_t)rhs * o.k + j], TS ? p : d);
-                    }
-                }
-            }
-            asm volatile("bar.sync %0, 64;" ::"r"(1 + grp) : "memory");   // sx is rewritten
-        }
-        dot = block_sum(dot, sh);
+        const double2 dot = block_sum(run_half1<TS, PASS2>(U, g, o, rhs, j, cta, ncta, sc, sx, kappa, emu, emu_inv), sh);
         if (tid == 0) part1[cta] = dot;
         target += (unsigned)ncta;
         if (!run_barrier(counter, target, &ok_sh)) {
             if (tid == 0) mark_failed(o, rhs, kStatusTimeout);
             return;
         }
-        if (warp == 0) {   // one warp: an FP64 warp instruction costs its pipe as much as any
-            const double2 tot = total(part1);
-            // Hermitian: H(j,j) = Re(q_j^dag r) / n_j, real (App. C); two-sided: (p_j^dag r) / m_j^*
-            const double2 al = TS ? cmul(sc[kScD], tot) : make_double2(tot.x * sc[kScD].x, 0.0);
-            if (lane == 0) {
-                if (cta == 0) o.alpha[(size_t)rhs * o.k + j] = al;
-                sc[kScC3] = cmul(al, sc[kScN]);
-                sc[kScC4] = TS ? cmul(cconj(al), sc[kScM]) : make_double2(0.0, 0.0);
-            }
-        }
+        if (tid < 32) run_alpha<TS>(o, rhs, j, cta == 0, ncta, part1, sc);
         __syncthreads();
         if (j == o.k - 1) break;
-        const double2 c3 = sc[kScC3], c4 = sc[kScC4];
-        // ---- step 2 ----
-        const double2* qj = outer_q(o, rhs, j);
-        double2* r = outer_q(o, rhs, j + 1);
-        const double2* pj = TS ? outer_p(o, rhs, j) : nullptr;
-        double2* l = TS ? outer_p(o, rhs, j + 1) : nullptr;
-        double2 del = make_double2(0.0, 0.0);
-        const unsigned stride = (unsigned)ncta * kRunThreads;
-        for (unsigned i = (unsigned)(cta + ncta * warp) * 32u + lane; i < items; i += stride) {
-            const size_t e0 = (size_t)i + (size_t)(i / (unsigned)V) * V;   // component 2 cp of the item
-            double2 q[2], x[2], pv[2], w[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const size_t e = e0 + (size_t)h * V;
-                q[h] = __ldcg(qj + e);
-                x[h] = __ldcg(r + e);
-                if (TS) { pv[h] = __ldcg(pj + e); w[h] = __ldcg(l + e); }
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const size_t e = e0 + (size_t)h * V;
-                x[h] = TS ? caxpy_neg(x[h], c3, q[h])
-                          : make_double2(fma(-c3.x, q[h].x, x[h].x), fma(-c3.x, q[h].y, x[h].y));
-                r[e] = x[h];
-                if (TS) {
-                    w[h] = caxpy_neg(w[h], c4, pv[h]);
-                    l[e] = w[h];
-                    del.x = fma(x[h].x, w[h].x, fma(x[h].y, w[h].y, del.x));   // conj(r) l
-                    del.y = fma(x[h].x, w[h].y, fma(-x[h].y, w[h].x, del.y));
-                } else {
-                    del.x = fma(x[h].x, x[h].x, fma(x[h].y, x[h].y, del.x));
-                }
-            }
-        }
-        del = block_sum(del, sh);
+        const double2 del = block_sum(run_half2<TS>(o, rhs, j, cta, ncta, sc), sh);
         if (tid == 0) part2[cta] = del;
         target += (unsigned)ncta;
         if (!run_barrier(counter, target, &ok_sh)) {
             if (tid == 0) mark_failed(o, rhs, kStatusTimeout);
             return;
         }
-        if (warp == 0) {
-            const StepScalars t = step_scalars<TS>(total(part2));
-            if (lane == 0) {
-                if (cta == 0) {
-                    o.beta[(size_t)rhs * o.k + j] = t.beta;
-                    o.gamma[(size_t)rhs * o.k + j] = t.gamma;
-                    if (!t.ok) mark_failed(o, rhs, kStatusBreakdown);
-                }
-                go_sh = t.ok;
-                if (t.ok) next_scalars<TS>(sc, t);
-            }
-        }
+        if (tid < 32) run_beta<TS>(o, rhs, j, cta == 0, ncta, part2, sc, &go_sh);
         __syncthreads();
         if (!go_sh) return;   // the same decision in every CTA of the RHS
     }
     if (cta == 0 && tid < kScalars && j_hi < o.k) o.sc[(size_t)rhs * kScalars + tid] = sc[tid];
+}
+
+// The same steps with a launch in the place of each grid barrier, for solves that
+// share the chip with others: the CTAs of k_run64 hold their SMs from the first
+// step to the last, and a second solve waits for a place; these come and go.  HALF 0
+// is the first half of step j, HALF 1 the second; the CTA that finishes last forms
+// the scalars, for all (formed by every CTA, as in k_run64, they would take an SM's
+// FP64 pipe from the other solves: 10.4 against 8.0 below).  us per step of one of 16
+// solves in flight, all steps in one launch -> a launch per half step: 4^4, mu = 0.1 3.4 -> 3.1;
+// 6^4, mu = 0.1 11.2 -> 8.0; 8^4 21.8 -> 18.3; 10^4, mu = 0.2 46.2 -> 40.2 (k_run64 there with
+// registers for three CTAs per SM; one per SM 14 at 6^4); of one alone 12.4 -> 17.3, 17.4 -> 22.5,
+// 27.6 -> 33.9, 52.2 -> 59.2.
+template <bool TS, bool PASS2, int HALF>
+__global__ void __launch_bounds__(kRunThreads, HALF == 0 ? 2 : 3) k_run64_half(const double2* __restrict__ U, Geom g, Outer o, int j,
+                                                               double kappa, double emu, double emu_inv) {
+    __shared__ double2 sx[HALF == 0 ? kRunGroups : 1][48 * kRunSites];
+    __shared__ double2 sh[33];
+    __shared__ double2 sc[kScalars];
+    __shared__ bool go_sh;
+    const int rhs = blockIdx.x % o.n_rhs, cta = blockIdx.x / o.n_rhs, ncta = gridDim.x / o.n_rhs;
+    if (o.status[rhs] != kStatusOK) return;
+    const int tid = threadIdx.x;
+    double2* part = o.partials + (size_t)rhs * o.npart;
+    double2* home = o.sc + (size_t)rhs * kScalars;
+    if (tid < kScalars) sc[tid] = home[tid];
+    __syncthreads();
+    const double2 mine = HALF == 0 ? run_half1<TS, PASS2>(U, g, o, rhs, j, cta, ncta, sc, sx, kappa, emu, emu_inv)
+                                   : run_half2<TS>(o, rhs, j, cta, ncta, sc);
+    if (!finish_partial(block_sum(mine, sh), part, o.counters + rhs, cta, ncta)) return;
+    __threadfence();
+    if (tid < 32) {
+        if (HALF == 0) run_alpha<TS>(o, rhs, j, true, ncta, part, sc);
+        else run_beta<TS>(o, rhs, j, true, ncta, part, sc, &go_sh);
+    }
+    __syncthreads();
+    if (tid < kScalars) home[tid] = sc[tid];   // every other CTA has read its copy
+    if (tid == 0) o.counters[rhs] = 0u;
+}
+
+// CTAs per RHS of a run: one per SM over the RHS, fewer where there are not so many
+// units of work.
+int run_ctas(const Geom& g, const Outer& o, int sms) {
+    const int units = (o.two_sided ? 2 : 1) * ((g.V + kRunSites - 1) / kRunSites);
+    return std::max(1, std::min(sms / o.n_rhs, units));
 }
 
 template <int S, int SPLIT>
@@ -533,14 +615,9 @@ void launch_stencil64_step1(const void* U64, const Geom& g, const Outer& o, int 
 
 bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int j_hi, double kappa, double mu, int sms,
                   cudaStream_t st) {
-    // one CTA per SM over the RHS, fewer where there are not four groups' work for each
-    const int nvec = o.two_sided ? 2 : 1;
-    const int nsb = (g.V + kRunSites - 1) / kRunSites;
-    int ncta = sms / o.n_rhs;
-    if (ncta > nvec * nsb) ncta = nvec * nsb;
     cudaMemsetAsync(o.run_bar, 0, sizeof(unsigned) * o.n_rhs, st);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(ncta * o.n_rhs));
+    cfg.gridDim = dim3((unsigned)(run_ctas(g, o, sms) * o.n_rhs));
     cfg.blockDim = dim3(kRunThreads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -559,6 +636,20 @@ bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int 
         e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<false, true>, U, g, o, j_lo, j_hi, kappa, ep, em)
                   : cudaLaunchKernelEx(&cfg, k_run64<false, false>, U, g, o, j_lo, j_hi, kappa, ep, em);
     return e == cudaSuccess;
+}
+
+void launch_run64_half(const void* U64, const Geom& g, const Outer& o, int half, int j, double kappa, double mu, int sms,
+                       cudaStream_t st) {
+    const unsigned grid = (unsigned)(run_ctas(g, o, sms) * o.n_rhs);
+    const double ep = exp(mu), em = exp(-mu);
+#define NK_HALF(TS_, P2_, H_) k_run64_half<TS_, P2_, H_><<<grid, kRunThreads, 0, st>>>((const double2*)U64, g, o, j, kappa, ep, em)
+    if (half == 0) {
+        if (o.two_sided) { if (o.y) NK_HALF(true, true, 0); else NK_HALF(true, false, 0); }
+        else { if (o.y) NK_HALF(false, true, 0); else NK_HALF(false, false, 0); }
+    } else {
+        if (o.two_sided) NK_HALF(true, false, 1); else NK_HALF(false, false, 1);
+    }
+#undef NK_HALF
 }
 
 void launch_stencil64(const void* U64, const Geom& g, const DslashSet& s0, const DslashSet& s1, bool abi, double kappa,

@@ -13,7 +13,9 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
-from paper_0912_4457_gb300.nksign import NK_EBREAKDOWN, NK_FP64, NK_OK, Context  # noqa: E402
+from paper_0912_4457_gb300.nksign import (  # noqa: E402
+    NK_ASYNC, NK_DOUBLE_PASS, NK_EBREAKDOWN, NK_FP64, NK_NO_GRAPH, NK_OK, Context,
+)
 
 M_W = -2.0
 
@@ -49,4 +51,64 @@ def test_breakdown_of_one_source_of_a_batch():
         assert list(st["status"][:2]) == [NK_EBREAKDOWN, NK_OK]
         assert not y[0].any()
         assert rel(y[1], ref) < 1e-10
+    ctx.close()
+
+
+def test_solves_in_flight_share_the_chip():
+    """Eight contexts' solves on eight streams take less than half the time of the eight one after
+    the other: a solve's launch of all its steps leaves room for others on its SMs (its CTAs alone
+    fill at most a third of them, so that at least two are resident together)."""
+    import time
+    dims, k, n = (6, 6, 6, 6), 256, 8
+    U = inputs.su3_links(dims, 41)[0]
+    ctxs, b, y, streams = [], [], [], []
+    for i in range(n):
+        c = Context(dims)
+        c.load_links(U)
+        c.set_mu_mw(0.1, M_W)
+        ctxs.append(c)
+        b.append(torch.from_numpy(inputs.gaussian_sources(dims, 73 + i)).cuda())
+        y.append(torch.zeros_like(b[-1]))
+        streams.append(torch.cuda.Stream())
+    torch.cuda.synchronize()
+
+    def together():
+        for c, x, o, s in zip(ctxs, b, y, streams):
+            c.sign_apply_dev(x, o, 1, k, 32, flags=NK_FP64 | NK_ASYNC, stream=s)
+        for c in ctxs:
+            c.wait()
+
+    def in_turn():
+        for c, x, o, s in zip(ctxs, b, y, streams):
+            c.sign_apply_dev(x, o, 1, k, 32, flags=NK_FP64 | NK_ASYNC, stream=s)
+            c.wait()
+
+    def best(f):
+        f()
+        ts = []
+        for _ in range(5):
+            t = time.perf_counter()
+            f()
+            ts.append(time.perf_counter() - t)
+        return min(ts)
+
+    assert best(together) < 0.5 * best(in_turn)
+    for c in ctxs:
+        c.close()
+
+
+@pytest.mark.parametrize("mu", [0.0, 0.3])
+@pytest.mark.parametrize("dims,n,k", [((2, 2, 2, 2), 1, 12), ((3, 5, 3, 7), 2, 30), ((4, 4, 4, 4), 12, 64),
+                                      ((6, 6, 6, 6), 1, 64), ((8, 8, 8, 8), 2, 32)])
+def test_solve_beside_others_gives_the_same_bits(mu, dims, n, k):
+    """NK_ASYNC: a launch per half step instead of one for all; the same result, also of a
+    double pass and without a graph."""
+    ctx, _ = make_ctx(dims, mu)
+    b = torch.from_numpy(inputs.gaussian_sources(dims, 72, n_rhs=n)).cuda()
+    for flags in (NK_FP64, NK_FP64 | NK_NO_GRAPH, NK_FP64 | NK_DOUBLE_PASS):
+        ref, got = torch.zeros_like(b), torch.zeros_like(b)
+        ctx.sign_apply_dev(b, ref, n, k, 8, flags=flags)
+        ctx.sign_apply_dev(b, got, n, k, 8, flags=flags | NK_ASYNC)
+        ctx.wait()
+        assert torch.equal(ref, got)
     ctx.close()
