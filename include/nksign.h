@@ -78,7 +78,10 @@ extern "C" {
                                the extremes of the per-RHS estimates over the batch: every RHS
                                shares A), instead of one per RHS; p > 0 overrides both */
 #define NK_PROFILE 0x20u    /* kernel by kernel, with CUDA events around every launch; fills
-                               nk_stats.t_class_ms / n_class (implies NK_NO_GRAPH) */
+                               nk_stats.t_class_ms / n_class (implies NK_NO_GRAPH).  The result
+                               has the same bits; where a small FP64 batch runs all its steps in
+                               one launch (nk_launch below), they are launched and timed by
+                               halves, which takes longer than the one launch */
 #define NK_PREFIX_FP64 0x100u /* with NK_MIXED: the outer steps before j0 apply the FP64 stencil
                                instead of the two-float one (nk_set_precision) */
 #define NK_EPS_EST 0x200u   /* also estimate the error of every result as in Sec. 3: apply the
@@ -274,7 +277,7 @@ int nk_set_adapt_start(nk_ctx* ctx, int k_first);
  * An FP64 recurrence on a small batch (V n_rhs, times 2 for mu != 0, up to 32768)
  * with no shape set or tuned runs all its steps in one cooperative launch instead
  * (needs every one of its CTAs, at most one per SM, resident at once), or, with
- * NK_ASYNC or on a device without cooperative launches, in one launch per half
+ * NK_ASYNC, NK_PROFILE or on a device without cooperative launches, in one launch per half
  * step of the same CTAs: the same bits either way.
  * A shape belongs to (n_rhs, sidedness of the current mu (mu != 0), the
  * NK_MIXED bit of flags).  Different shapes sum in different orders, so

@@ -422,7 +422,8 @@ int copy_mode_for(const Schedule& s, int j) {
 // no launch shape of its own (a set or tuned shape names the kernels of a step).
 // A cooperative launch keeps its SMs for the whole run, so a solve beside others
 // (NK_ASYNC) takes a launch per half step of the same CTAs instead, with the
-// same bits (k_run64_half: eight 6^4 solves in flight 9.5 -> 5.0 ms each, one 16.0 -> 17.5).
+// same bits (k_run64_half: eight 6^4 solves in flight 9.5 -> 5.0 ms each, one 16.0 -> 17.5);
+// so does NK_PROFILE, to time the halves.
 constexpr long kRunSiteVecs = 32768;
 bool run_in_one(const nk_ctx* c, const nk::Outer& o) {
     if ((long)c->V * o.n_rhs * (o.two_sided ? 2 : 1) > kRunSiteVecs) return false;
@@ -444,9 +445,9 @@ void enqueue_outer_steps(nk_ctx* c, const nk::Outer& o, const Schedule& s, int j
     const Geom g = geom_of(c);
     const double kap = kappa_of(c);
     cudaStream_t st = L.st;
-    if (!s.mixed && !L.profile && j_end > j_begin && run_in_one(c, o)) {
+    if (!s.mixed && j_end > j_begin && run_in_one(c, o)) {
         const int ctas = std::min(c->sms, kRunMaxCtas);
-        if (c->coop && L.alone) {
+        if (c->coop && L.alone && !L.profile) {
             bool ok = true;
             L.run_counted(NK_CLASS_DSLASH64, [&] {
                 ok = nk::launch_run64(c->U64, g, o, j_begin, j_end, kap, c->mu, ctas, st);

@@ -14,7 +14,7 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
 from paper_0912_4457_gb300.nksign import (  # noqa: E402
-    NK_ASYNC, NK_DOUBLE_PASS, NK_EBREAKDOWN, NK_FP64, NK_NO_GRAPH, NK_OK, Context,
+    NK_ASYNC, NK_DOUBLE_PASS, NK_EBREAKDOWN, NK_FP64, NK_NO_GRAPH, NK_OK, NK_PROFILE, Context,
 )
 
 M_W = -2.0
@@ -111,4 +111,20 @@ def test_solve_beside_others_gives_the_same_bits(mu, dims, n, k):
         ctx.sign_apply_dev(b, got, n, k, 8, flags=flags | NK_ASYNC)
         ctx.wait()
         assert torch.equal(ref, got)
+    ctx.close()
+
+
+@pytest.mark.parametrize("mu", [0.0, 0.3])
+def test_profile_times_the_arithmetic_of_the_solve(mu):
+    """NK_PROFILE: the bits of the solve without it, fixed and adaptive k (a recurrence continued
+    in chunks), and one launch per half step in the classes of the halves."""
+    dims, n, k = (4, 4, 4, 4), 2, 128
+    ctx, _ = make_ctx(dims, mu)
+    b = inputs.gaussian_sources(dims, 74, n_rhs=n)
+    for tol in (0.0, 1e-30):
+        y, _, _ = ctx.sign_apply(b, k, 32, tol=tol, check=False)
+        yp, st, _ = ctx.sign_apply(b, k, 32, tol=tol, flags=NK_FP64 | NK_PROFILE, check=False)
+        np.testing.assert_array_equal(y, yp)
+        assert st["n_class"]["dslash64"] == k and st["n_class"]["step2"] == k - 1
+        assert st["t_class_ms"]["dslash64"] > 0.0 and st["t_class_ms"]["step2"] > 0.0
     ctx.close()
