@@ -54,8 +54,8 @@ extern "C" {
 #define NK_ECUDA (-6)       /* CUDA runtime error */
 #define NK_ETIMEOUT (-7)    /* a bounded device-side wait ran out: the grid barriers of the cooperative
                                launch that runs the FP64 steps of a small batch wait at most one
-                               second each; that RHS is failed (the clusters of the inner part
-                               synchronise with hardware cluster barriers) */
+                               second each (nk_set_wait_limit); that RHS is failed (the clusters of
+                               the inner part synchronise with hardware cluster barriers) */
 #define NK_ESTATE (-8)      /* call out of order (e.g. no links loaded) */
 
 /* Solve flags (bitwise or). */
@@ -253,6 +253,11 @@ int nk_set_nesting(nk_ctx* ctx, int n_deeper, const int* ells);
  * NK_ADAPT_FIRST(l)).  A predicted k (nk_predict_sizes) minus two check
  * intervals goes here, so that a good prediction costs three checks. */
 int nk_set_adapt_start(nk_ctx* ctx, int k_first);
+
+/* The longest that a wait of this context's kernels on one another may take, in
+ * seconds (0 to 10; 1 at creation); with 0 a wait runs out at once.  An RHS whose
+ * wait runs out is failed with NK_ETIMEOUT. */
+int nk_set_wait_limit(nk_ctx* ctx, double seconds);
 
 /*
  * Launch shape of the outer recurrence (batching of the RHS and the

@@ -59,6 +59,7 @@ struct nk_ctx {
     int device;
     int sms = 152;         // multiprocessors
     bool coop = false;     // the device takes cooperative launches
+    unsigned long long wait_ns = 1000000000ull;   // limit of a device-side wait (nk_set_wait_limit)
     double mu = 0.0, m_w = 0.0;
     bool mu_set = false;
     int j0 = -1;
@@ -450,7 +451,7 @@ void enqueue_outer_steps(nk_ctx* c, const nk::Outer& o, const Schedule& s, int j
         if (c->coop && L.alone && !L.profile) {
             bool ok = true;
             L.run_counted(NK_CLASS_DSLASH64, [&] {
-                ok = nk::launch_run64(c->U64, g, o, j_begin, j_end, kap, c->mu, ctas, st);
+                ok = nk::launch_run64(c->U64, g, o, j_begin, j_end, kap, c->mu, ctas, c->wait_ns, st);
                 return ok ? 1 : 0;
             });
             if (ok) return;
@@ -708,6 +709,8 @@ int status_to_code(int s) {
     }
 }
 
+const char* const kTimeoutMsg = "outer recurrence: a device-side wait ran out";
+
 // Per-RHS outcome of a finished solve (device arrays read after the stream
 // has been synchronised) into codes and stats.
 int collect_outcome(nk_ctx* c, int n_rhs, int k_used_max, const std::vector<int>& kused_h,
@@ -742,6 +745,7 @@ int collect_outcome(nk_ctx* c, int n_rhs, int k_used_max, const std::vector<int>
     }
     if (worst == NK_EBREAKDOWN) return fail(c, worst, "two-sided Lanczos: serious breakdown (delta = 0)");
     if (worst == NK_ERHI) return fail(c, worst, "Roberts-Higham iteration did not converge (or p H_k singular)");
+    if (worst == NK_ETIMEOUT) return fail(c, worst, kTimeoutMsg);
     if (worst == NK_ENOTCONV) return fail(c, worst, "adaptive k: tolerance not met at k_max for some RHS");
     return worst;
 }
@@ -931,7 +935,10 @@ int predicted_solve(nk_ctx* c, const double* b_dev, int n_rhs, int k, int ell, d
     return rc;
 }
 
-bool solve_failed_hard(int rc) { return rc != NK_OK && rc != NK_EBREAKDOWN && rc != NK_ERHI && rc != NK_ENOTCONV; }
+// A failure of the whole call, not of single RHS (whose status says so; the others have their results)
+bool solve_failed_hard(int rc) {
+    return rc != NK_OK && rc != NK_EBREAKDOWN && rc != NK_ERHI && rc != NK_ENOTCONV && rc != NK_ETIMEOUT;
+}
 
 // LR deflation (App. C steps 1 and 6) around a solve: the Krylov part runs on
 // x_minus = b - sum_i <l_i, b> r_i, and sum_i sgn(lambda_i) <l_i, b> r_i is
@@ -1313,6 +1320,7 @@ int nk_eigs_smallest(nk_ctx* c, const double* b, int k, int m, double tol, doubl
     NK_CUDA(c, cudaMemcpy(&xn, Lw.o.xnorm, sizeof(double), cudaMemcpyDeviceToHost));
     NK_CUDA(c, cudaMemcpy(&status, Lw.o.status, sizeof(int), cudaMemcpyDeviceToHost));
     if (status == nk::kStatusZeroSource) return fail(c, NK_EINVAL, "zero start vector");
+    if (status == nk::kStatusTimeout) return fail(c, NK_ETIMEOUT, kTimeoutMsg);
     if (status != nk::kStatusOK) return fail(c, NK_EBREAKDOWN, "Lanczos breakdown before step k");
     // H_k: diagonal H(j,j), sub-diagonal H(j+1,j) = beta_j, super-diagonal H(j,j+1) = gamma_j
     std::vector<nk::cplx> a(k), sub(k - 1), sup(k - 1);
@@ -1639,6 +1647,14 @@ static void clear_graphs(nk_ctx* c) {
     c->graphs.clear();
 }
 
+int nk_set_wait_limit(nk_ctx* c, double seconds) {
+    if (!c) return NK_EINVAL;
+    if (!(seconds >= 0.0) || seconds > 10.0) return fail(c, NK_EINVAL, "the wait limit must be in [0, 10] seconds");
+    c->wait_ns = (unsigned long long)(seconds * 1e9);
+    clear_graphs(c);
+    return NK_OK;
+}
+
 static int shape_args(nk_ctx* c, int n_rhs) {
     if (!c) return NK_EINVAL;
     if (n_rhs < 1 || n_rhs > NK_MAX_RHS) return fail(c, NK_EINVAL, "bad n_rhs");
@@ -1866,7 +1882,7 @@ static int host_solve(nk_ctx* c, const double* b, int n_rhs, int k, int ell, dou
     double* yd = bd + 2 * (size_t)c->N * NK_MAX_RHS;
     NK_CUDA(c, cudaMemcpy(bd, b, bytes, cudaMemcpyHostToDevice));
     rc = solve_dev(c, bd, n_rhs, k, ell, tol, p, flags, yd, st, 0, overlap);
-    if (rc != NK_OK && rc != NK_EBREAKDOWN && rc != NK_ERHI && rc != NK_ENOTCONV) return rc;
+    if (solve_failed_hard(rc)) return rc;
     cudaError_t e = cudaMemcpy(y, yd, bytes, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemcpy y");
     return rc;
@@ -2016,9 +2032,11 @@ int nk_outer_lanczos_dev(nk_ctx* c, const double* b_dev, int n_rhs, int k, unsig
     std::vector<int> status(n_rhs);
     NK_CUDA(c, cudaMemcpyAsync(status.data(), Lw.o.status, sizeof(int) * n_rhs, cudaMemcpyDeviceToHost, st));
     NK_CUDA(c, cudaStreamSynchronize(st));
-    for (int r = 0; r < n_rhs; ++r)
+    for (int r = 0; r < n_rhs; ++r) {
         if (status[r] == nk::kStatusBreakdown)
             return fail(c, NK_EBREAKDOWN, "two-sided Lanczos: serious breakdown (delta = 0)");
+        if (status[r] == nk::kStatusTimeout) return fail(c, NK_ETIMEOUT, kTimeoutMsg);
+    }
     return NK_OK;
 }
 

@@ -36,9 +36,10 @@ void launch_stencil64_step1(const void* U64, const Geom& g, const Outer& o, int 
 int stencil64_blocks(const Geom& g, int threads, int nvec);   // CTAs, hence partial sums, per vector
 // Steps [j_lo, j_hi) of an FP64 recurrence in one cooperative launch of at most
 // `sms` CTAs (two partial sums per CTA and RHS: npart >= 2 sms / n_rhs).
+// A wait at a grid barrier ends after wait_ns and fails that RHS (kStatusTimeout).
 // False if the launch failed (cudaGetLastError has the reason).
 bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int j_hi, double kappa, double mu, int sms,
-                  cudaStream_t st);
+                  unsigned long long wait_ns, cudaStream_t st);
 // The same, a launch per half step (same CTAs, same bits): half 0 or 1 of step j.
 void launch_run64_half(const void* U64, const Geom& g, const Outer& o, int half, int j, double kappa, double mu, int sms,
                        cudaStream_t st);

@@ -307,7 +307,6 @@ __global__ void __launch_bounds__(16 * S * SPLIT, SPLIT == 1 ? kS64Sites / S : 1
 // at 6^4, 55.5 at 10^4.  Groups of 64 threads on four sites leave a quarter of the lanes
 // idle in the sum over the hops: 54 at 10^4.
 constexpr int kRunSites = 8, kRunGroup = 16 * kRunSites, kRunThreads = 384, kRunGroups = kRunThreads / kRunGroup;
-constexpr unsigned long long kRunWaitNs = 1000000000ull;   // one second
 
 __device__ __forceinline__ unsigned long long run_ns() {
     unsigned long long t;
@@ -320,7 +319,8 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
     return v;
 }
 // All CTAs of one RHS (n of them; the counter counts arrivals since the launch).
-__device__ __forceinline__ bool run_barrier(unsigned* counter, unsigned target, bool* ok_sh) {
+// False if it waited for wait_ns.
+__device__ __forceinline__ bool run_barrier(unsigned* counter, unsigned target, unsigned long long wait_ns, bool* ok_sh) {
     __syncthreads();
     if (threadIdx.x == 0) {
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
@@ -328,7 +328,7 @@ __device__ __forceinline__ bool run_barrier(unsigned* counter, unsigned target, 
         if (ld_acquire(counter) < target) {
             const unsigned long long t0 = run_ns();
             while (ld_acquire(counter) < target)
-                if (run_ns() - t0 > kRunWaitNs) { ok = false; break; }
+                if (run_ns() - t0 >= wait_ns) { ok = false; break; }
         }
         *ok_sh = ok;
     }
@@ -485,7 +485,8 @@ __device__ __forceinline__ void run_beta(const Outer& o, int rhs, int j, bool wr
 
 template <bool TS, bool PASS2>
 __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict__ U, Geom g, Outer o, int j_lo, int j_hi,
-                                                          double kappa, double emu, double emu_inv) {
+                                                          double kappa, double emu, double emu_inv,
+                                                          unsigned long long wait_ns) {
     __shared__ double2 sx[kRunGroups][48 * kRunSites];
     __shared__ double2 sh[33];
     __shared__ double2 sc[kScalars];
@@ -504,7 +505,7 @@ __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict
         const double2 dot = block_sum(run_half1<TS, PASS2>(U, g, o, rhs, j, cta, ncta, sc, sx, kappa, emu, emu_inv), sh);
         if (tid == 0) part1[cta] = dot;
         target += (unsigned)ncta;
-        if (!run_barrier(counter, target, &ok_sh)) {
+        if (!run_barrier(counter, target, wait_ns, &ok_sh)) {
             if (tid == 0) mark_failed(o, rhs, kStatusTimeout);
             return;
         }
@@ -514,7 +515,7 @@ __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict
         const double2 del = block_sum(run_half2<TS>(o, rhs, j, cta, ncta, sc), sh);
         if (tid == 0) part2[cta] = del;
         target += (unsigned)ncta;
-        if (!run_barrier(counter, target, &ok_sh)) {
+        if (!run_barrier(counter, target, wait_ns, &ok_sh)) {
             if (tid == 0) mark_failed(o, rhs, kStatusTimeout);
             return;
         }
@@ -614,7 +615,7 @@ void launch_stencil64_step1(const void* U64, const Geom& g, const Outer& o, int 
 }
 
 bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int j_hi, double kappa, double mu, int sms,
-                  cudaStream_t st) {
+                  unsigned long long wait_ns, cudaStream_t st) {
     cudaMemsetAsync(o.run_bar, 0, sizeof(unsigned) * o.n_rhs, st);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(run_ctas(g, o, sms) * o.n_rhs));
@@ -630,11 +631,11 @@ bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int 
     const bool pass2 = o.y != nullptr;
     cudaError_t e;
     if (o.two_sided)
-        e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<true, true>, U, g, o, j_lo, j_hi, kappa, ep, em)
-                  : cudaLaunchKernelEx(&cfg, k_run64<true, false>, U, g, o, j_lo, j_hi, kappa, ep, em);
+        e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<true, true>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns)
+                  : cudaLaunchKernelEx(&cfg, k_run64<true, false>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns);
     else
-        e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<false, true>, U, g, o, j_lo, j_hi, kappa, ep, em)
-                  : cudaLaunchKernelEx(&cfg, k_run64<false, false>, U, g, o, j_lo, j_hi, kappa, ep, em);
+        e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<false, true>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns)
+                  : cudaLaunchKernelEx(&cfg, k_run64<false, false>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns);
     return e == cudaSuccess;
 }
 

@@ -49,7 +49,7 @@ ERROR_NAMES = {
 
 EXPORTED = [
     "nk_create_lattice", "nk_load_links", "nk_load_links_dev", "nk_set_mu_mw", "nk_set_precision", "nk_set_df_recurrence",
-    "nk_set_adapt_start", "nk_set_nesting", "nk_set_deflation", "nk_eigs_smallest", "nk_overlap_solve",
+    "nk_set_adapt_start", "nk_set_wait_limit", "nk_set_nesting", "nk_set_deflation", "nk_eigs_smallest", "nk_overlap_solve",
     "nk_sign_apply", "nk_sign_apply_dev", "nk_overlap_apply", "nk_overlap_apply_dev",
     "nk_dslash_dev", "nk_stencil32_dev", "nk_outer_lanczos_dev", "nk_inner_sign", "nk_inner_sign_noalloc", "nk_last_error",
     "nk_destroy",
@@ -148,6 +148,7 @@ def load_library(path: str = LIB_PATH):
         "nk_set_precision": ([P, I], I),
         "nk_set_df_recurrence": ([P, I], I),
         "nk_set_adapt_start": ([P, I], I),
+        "nk_set_wait_limit": ([P, D], I),
         "nk_set_nesting": ([P, I, P], I),
         "nk_set_deflation": ([P, I, P, P, P], I),
         "nk_eigs_smallest": ([P, dp, I, I, D, dp, dp, P, P, P], I),
@@ -271,6 +272,9 @@ class Context:
 
     def set_adapt_start(self, k_first: int):
         self._check(self._lib.nk_set_adapt_start(self.h, int(k_first)))
+
+    def set_wait_limit(self, seconds: float):
+        self._check(self._lib.nk_set_wait_limit(self.h, float(seconds)))
 
     def overlap_solve(self, b, k, ell, mass=0.0, tol_cg=1e-8, maxit=500, tol_sign=0.0, flags=NK_FP64, check=True):
         """nk_overlap_solve: x = (D_ov + mass)^-1 b by CG on the normal

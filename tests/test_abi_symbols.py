@@ -103,3 +103,9 @@ def test_noalloc_binding_refuses_undersized_tensors_before_any_launch():
     # the right sizes pass the check and then need a CUDA tensor
     with pytest.raises(TypeError):
         nksign.inner_sign_noalloc(ok, ok, ok, ok, 2, k, 16, 0.0, True)
+
+
+def test_wait_limit_rejects_a_null_context(lib):
+    f = lib.nk_set_wait_limit
+    f.argtypes, f.restype = [ctypes.c_void_p, ctypes.c_double], ctypes.c_int
+    assert f(None, 1.0) == -1

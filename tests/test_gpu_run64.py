@@ -14,7 +14,8 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
 from paper_0912_4457_gb300.nksign import (  # noqa: E402
-    NK_ASYNC, NK_DOUBLE_PASS, NK_EBREAKDOWN, NK_FP64, NK_NO_GRAPH, NK_OK, NK_PROFILE, Context,
+    NK_ASYNC, NK_DOUBLE_PASS, NK_EBREAKDOWN, NK_EINVAL, NK_ETIMEOUT, NK_FP64, NK_NO_GRAPH, NK_OK, NK_PROFILE,
+    Context, NkError,
 )
 
 M_W = -2.0
@@ -127,4 +128,35 @@ def test_profile_times_the_arithmetic_of_the_solve(mu):
         np.testing.assert_array_equal(y, yp)
         assert st["n_class"]["dslash64"] == k and st["n_class"]["step2"] == k - 1
         assert st["t_class_ms"]["dslash64"] > 0.0 and st["t_class_ms"]["step2"] > 0.0
+    ctx.close()
+
+
+def test_a_wait_that_runs_out_is_a_timeout_in_every_call():
+    """With a limit of 0 the first CTA at a grid barrier gives up: every call that runs the steps
+    in one launch reports NK_ETIMEOUT (not success, not a breakdown), and the context goes on
+    with the next limit."""
+    from paper_0912_4457_gb300 import nksign
+    dims, n, k = (6, 6, 6, 6), 2, 64
+    ctx, _ = make_ctx(dims, 0.2)
+    b = inputs.gaussian_sources(dims, 75, n_rhs=n)
+    bd = torch.from_numpy(b).cuda()
+    ref, _, _ = ctx.sign_apply(b, k, 16)
+    ctx.set_wait_limit(0.0)
+    for flags in (NK_FP64, NK_FP64 | NK_NO_GRAPH):
+        y, st, rc = ctx.sign_apply(b, k, 16, flags=flags, check=False)
+        assert rc == NK_ETIMEOUT and list(st["status"][:n]) == [NK_ETIMEOUT] * n
+        assert not y.any()
+        assert "wait" in nksign.load_library().nk_last_error(ctx.h).decode()
+    y, st, rc = ctx.sign_apply(b, k, 16, tol=1e-8, check=False)
+    assert rc == NK_ETIMEOUT and list(st["status"][:n]) == [NK_ETIMEOUT] * n
+    with pytest.raises(NkError) as e:
+        ctx.outer_lanczos_dev(bd, n, k)
+    assert e.value.code == NK_ETIMEOUT
+    assert ctx.eigs_smallest(b[0], k, 4, check=False)[-1] == NK_ETIMEOUT
+    for bad in (-1.0, 11.0, float("nan")):
+        with pytest.raises(NkError) as e:
+            ctx.set_wait_limit(bad)
+        assert e.value.code == NK_EINVAL
+    ctx.set_wait_limit(1.0)
+    np.testing.assert_array_equal(ctx.sign_apply(b, k, 16)[0], ref)
     ctx.close()
