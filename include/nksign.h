@@ -280,14 +280,15 @@ int nk_set_wait_limit(nk_ctx* ctx, double seconds);
  *                   one thread (early_split = 3: one per colour) per site and
  *                   vector.  The multi-RHS stencils of NK_MIXED have one shape.
  * An FP64 recurrence on a small batch (V n_rhs, times 2 for mu != 0, up to 32768)
- * with no shape set or tuned runs all its steps in one cooperative launch instead
+ * with no shape set or tuned, or one that equals the unset one in stencil_threads,
+ * stencil_order, step2_blocks and stencil_split, runs all its steps in one cooperative launch instead
  * (needs every one of its CTAs, at most one per SM, resident at once), or, with
  * NK_ASYNC, NK_PROFILE or on a device without cooperative launches, in one launch per half
  * step of the same CTAs: the same bits either way.
  * A shape belongs to (n_rhs, sidedness of the current mu (mu != 0), the
  * NK_MIXED bit of flags).  Different shapes sum in different orders, so
  * results differ at rounding level; one shape is bitwise reproducible.
- * Unset shapes use 128 / 0 / min(ceil(6 V / 128), 760 / n_rhs in fours) / 128 / 0 / 1 / 1.
+ * Unset shapes use 128 / 0 / min(ceil(6 V / 128), 5 CTAs per SM / n_rhs) / 128 / 0 / 1 / 1.
  */
 typedef struct nk_launch {
     int stencil_threads;
@@ -306,7 +307,8 @@ int nk_get_launch(nk_ctx* ctx, int n_rhs, unsigned flags, nk_launch* shape);
  * stencil shapes with the FP32 stencil (NK_MIXED) or the FP64 one; in NK_MIXED mode
  * the same shapes with the two-float stencil (early_threads, early_order);
  * then step2_blocks in {b/2, b, 2b, 4b, 8b} (b the default) with the fastest
- * late stencil shape.  Keeps the fastest of each (written to *best, and the
+ * late stencil shape; and for an FP64 batch small enough for it the one launch of all
+ * steps, which the unset shape then stands for where it is fastest.  Keeps the fastest of each (written to *best, and the
  * time of one late outer step to *ms_per_step; both nullable).
  * cache_path (nullable): a text file of lines
  *   nk_launch Lx Ly Lz Lt n_rhs two_sided mixed threads order blocks

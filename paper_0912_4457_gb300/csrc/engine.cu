@@ -306,11 +306,8 @@ int blocks_per_rhs(long N, int n_rhs) {
     return nk::step_blocks(N, n_rhs, sms);
 }
 
-// The launch shape of a solve: the tuned one for (n_rhs, two-sided, mixed),
-// else the default (128 sites per CTA, vector-fastest grid, blocks_per_rhs).
-nk_launch launch_cfg(const nk_ctx* c, int n_rhs, bool ts, bool mixed) {
-    auto it = c->tune.find(std::make_tuple(n_rhs, ts ? 1 : 0, mixed ? 1 : 0));
-    if (it != c->tune.end()) return it->second;
+// The default launch shape: 128 threads per CTA, vector-fastest grid, blocks_per_rhs.
+nk_launch default_launch(const nk_ctx* c, int n_rhs) {
     nk_launch d;
     d.stencil_threads = 128;
     d.stencil_order = 0;
@@ -320,6 +317,18 @@ nk_launch launch_cfg(const nk_ctx* c, int n_rhs, bool ts, bool mixed) {
     d.stencil_split = 1;
     d.early_split = 1;
     return d;
+}
+
+// The launch shape of a solve: the tuned one for (n_rhs, two-sided, mixed), else the default.
+nk_launch launch_cfg(const nk_ctx* c, int n_rhs, bool ts, bool mixed) {
+    auto it = c->tune.find(std::make_tuple(n_rhs, ts ? 1 : 0, mixed ? 1 : 0));
+    return it != c->tune.end() ? it->second : default_launch(c, n_rhs);
+}
+
+// Whether two shapes are one for the FP64 step kernels.
+bool same_steps64(const nk_launch& a, const nk_launch& b) {
+    return a.stencil_threads == b.stencil_threads && a.stencil_order == b.stencil_order &&
+           a.step2_blocks == b.step2_blocks && a.stencil_split == b.stencil_split;
 }
 
 bool valid_launch(const nk_launch& l) {
@@ -420,15 +429,17 @@ int copy_mode_for(const Schedule& s, int j) {
 // the FP64 pipe hides the step kernels' launches and tails and their finer grain
 // wins (measured us per step, run against step kernels: 6^4 x 2 vectors 17.4 / 21.0,
 // 10^4 x 2 52.2 / 58.1, 6^4 x 24 74.5 / 79.4, 8^4 x 8 74.8 / 79.6, 8^4 x 12 114.7 / 112.4) -- with
-// no launch shape of its own (a set or tuned shape names the kernels of a step).
+// no launch shape of its own (a set or tuned shape other than the default names the
+// kernels of a step).
 // A cooperative launch keeps its SMs for the whole run, so a solve beside others
 // (NK_ASYNC) takes a launch per half step of the same CTAs instead, with the
 // same bits (k_run64_half: eight 6^4 solves in flight 9.5 -> 5.0 ms each, one 16.0 -> 17.5);
 // so does NK_PROFILE, to time the halves.
 constexpr long kRunSiteVecs = 32768;
+bool small_batch64(const nk_ctx* c, int n_rhs, bool ts) { return (long)c->V * n_rhs * (ts ? 2 : 1) <= kRunSiteVecs; }
 bool run_in_one(const nk_ctx* c, const nk::Outer& o) {
-    if ((long)c->V * o.n_rhs * (o.two_sided ? 2 : 1) > kRunSiteVecs) return false;
-    return c->tune.count(std::make_tuple(o.n_rhs, o.two_sided ? 1 : 0, 0)) == 0;
+    if (!small_batch64(c, o.n_rhs, o.two_sided)) return false;
+    return same_steps64(launch_cfg(c, o.n_rhs, o.two_sided, false), default_launch(c, o.n_rhs));
 }
 
 void enqueue_outer_init(const nk::Outer& o, const Schedule& s, Launcher& L, bool keep_status = false) {
@@ -1738,6 +1749,59 @@ static int time_kernel(nk_ctx* c, const double* src, int n_rhs, bool mixed, int 
     return NK_OK;
 }
 
+// The time per step of the one launch that runs the steps of a small FP64 batch, on the
+// same source and from the same step, each repetition from the same scalars: kTuneRun
+// steps a launch (the minimum over kTuneRounds rounds).  Negative if the recurrence does
+// not get there (then no kernel's time means anything).
+constexpr int kTuneRun = 16, kTuneRunReps = 8;
+static int time_run(nk_ctx* c, const double* src, int n_rhs, cudaStream_t st, float* per_step_ms) {
+    const bool ts = c->mu != 0.0;
+    const int k = kTuneWarm + kTuneRun + 2, ctas = std::min(c->sms, kRunMaxCtas);
+    const nk_launch lc = default_launch(c, n_rhs);
+    const Geom g = geom_of(c);
+    Layout dry = carve(nullptr, g, n_rhs, k, 2, ts, false, lc, false);
+    int rc = ensure(c, c->ws, dry.total);
+    if (rc) return rc;
+    Layout Lw = carve((char*)c->ws.p, g, n_rhs, k, 2, ts, false, lc, false);
+    NK_CUDA(c, cudaMemsetAsync(Lw.o.counters, 0, sizeof(unsigned) * n_rhs, st));
+    Launcher L;
+    L.st = st;
+    enqueue_load_sources(c, Lw.o, src, n_rhs, L);
+    enqueue_outer_init(Lw.o, Schedule(), L);
+    const double kap = kappa_of(c);
+    const size_t sb = sizeof(double2) * nk::kScalars * n_rhs;   // kept in the lift coefficients (k > kScalars)
+    bool ok = nk::launch_run64(c->U64, g, Lw.o, 0, kTuneWarm, kap, c->mu, ctas, c->wait_ns, st);
+    NK_CUDA(c, cudaMemcpyAsync(Lw.cp, Lw.o.sc, sb, cudaMemcpyDeviceToDevice, st));
+    EventPair ev;   // destroyed on every return
+    NK_CUDA(c, cudaEventCreate(&ev.e0));
+    NK_CUDA(c, cudaEventCreate(&ev.e1));
+    float best = 1e30f;
+    for (int round = 0; ok && round < kTuneRounds; ++round) {
+        NK_CUDA(c, cudaEventRecord(ev.e0, st));
+        for (int r = 0; ok && r < kTuneRunReps; ++r) {
+            NK_CUDA(c, cudaMemcpyAsync(Lw.o.sc, Lw.cp, sb, cudaMemcpyDeviceToDevice, st));
+            ok = nk::launch_run64(c->U64, g, Lw.o, kTuneWarm, kTuneWarm + kTuneRun, kap, c->mu, ctas, c->wait_ns, st);
+        }
+        NK_CUDA(c, cudaEventRecord(ev.e1, st));
+        NK_CUDA(c, cudaEventSynchronize(ev.e1));
+        float ms = 0.f;
+        NK_CUDA(c, cudaEventElapsedTime(&ms, ev.e0, ev.e1));
+        best = std::min(best, ms / (kTuneRunReps * kTuneRun));
+    }
+    if (!ok) {   // no cooperative launch here
+        cudaGetLastError();
+        *per_step_ms = 1e30f;
+        return NK_OK;
+    }
+    std::vector<int> status(n_rhs);
+    NK_CUDA(c, cudaMemcpyAsync(status.data(), Lw.o.status, sizeof(int) * n_rhs, cudaMemcpyDeviceToHost, st));
+    NK_CUDA(c, cudaStreamSynchronize(st));
+    for (int r = 0; r < n_rhs; ++r)
+        if (status[r] != nk::kStatusOK) best = -1.f;
+    *per_step_ms = best;
+    return NK_OK;
+}
+
 int nk_autotune(nk_ctx* c, int n_rhs, unsigned flags, const char* cache_path, nk_launch* out, double* ms_per_step) {
     int rc = shape_args(c, n_rhs);
     if (rc) return rc;
@@ -1842,7 +1906,21 @@ int nk_autotune(nk_ctx* c, int n_rhs, unsigned flags, const char* cache_path, nk
     }
     best = cand;
     // reported: the time of one outer step after j0 (stencil + step 2)
-    const float t_best = t_s2;
+    float t_best = t_s2;
+    const nk_launch unset = default_launch(c, n_rhs);
+    if (!mixed && c->coop && small_batch64(c, n_rhs, ts != 0)) {
+        // the steps in one launch are what the default shape stands for: they keep it where
+        // they win, and the step kernels take one CTA more than it where they win with it
+        float t;
+        rc = time_run(c, src, n_rhs, st, &t);
+        if (rc) return fail_out(rc);
+        if (t < t_best) {
+            best = unset;
+            if (t > 0.f) t_best = t;
+        } else if (same_steps64(best, unset)) {
+            best.step2_blocks += best.step2_blocks < 4096 ? 1 : -1;
+        }
+    }
     cudaStreamDestroy(st);
     c->tune[std::make_tuple(n_rhs, ts, mixed)] = best;
     clear_graphs(c);

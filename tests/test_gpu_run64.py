@@ -160,3 +160,40 @@ def test_a_wait_that_runs_out_is_a_timeout_in_every_call():
     ctx.set_wait_limit(1.0)
     np.testing.assert_array_equal(ctx.sign_apply(b, k, 16)[0], ref)
     ctx.close()
+
+
+def test_setting_the_shape_a_context_reports_changes_nothing():
+    """nk_set_launch of what nk_get_launch gives keeps the one launch of all steps (same bits, same
+    number of launches); another shape takes the step kernels."""
+    dims, n, k = (4, 4, 4, 4), 2, 64
+    ctx, _ = make_ctx(dims, 0.2)
+    b = inputs.gaussian_sources(dims, 76, n_rhs=n)
+    y0, st0, _ = ctx.sign_apply(b, k, 16)
+    shape = list(ctx.get_launch(n, NK_FP64))
+    ctx.set_launch(n, NK_FP64, *shape)
+    y1, st1, _ = ctx.sign_apply(b, k, 16)
+    assert st1["launches"] == st0["launches"]
+    np.testing.assert_array_equal(y0, y1)
+    shape[2] += 1
+    ctx.set_launch(n, NK_FP64, *shape)
+    _, st2, _ = ctx.sign_apply(b, k, 16)
+    assert st2["launches"] > st0["launches"] + k
+    ctx.close()
+
+
+def test_autotune_times_the_launch_of_all_steps(tmp_path):
+    """Tuning a small FP64 batch keeps the one launch of all steps where that is faster (here by a
+    third), in the context that tuned and in one that reads the cache file."""
+    dims, n, k = (4, 4, 4, 4), 1, 64
+    path = str(tmp_path / "tune.txt")
+    b = inputs.gaussian_sources(dims, 77, n_rhs=n)
+    ctx, _ = make_ctx(dims, 0.0)
+    unset = ctx.get_launch(n, NK_FP64)
+    _, st0, _ = ctx.sign_apply(b, k, 16)
+    shape, ms = ctx.autotune(n, NK_FP64, path)
+    assert shape == unset == ctx.get_launch(n, NK_FP64) and 0.0 < ms < 10.0
+    other, _ = make_ctx(dims, 0.0)
+    assert other.autotune(n, NK_FP64, path)[0] == unset
+    for c in (ctx, other):
+        assert c.sign_apply(b, k, 16)[1]["launches"] == st0["launches"]
+        c.close()
