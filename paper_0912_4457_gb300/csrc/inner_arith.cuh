@@ -85,6 +85,19 @@ __device__ __forceinline__ double2 pivot_inv(double2 a) {
     return mk(x * r, -y * r);
 }
 
+// The same by a division, for the LU (its one chain has no other work beside it:
+// with pivot_inv 12 two-sided RHS at k = 1024, l = 128 took the same time, Hermitian
+// ones at k = 768 5.26 against 5.21 ms).
+__device__ __forceinline__ double pivot_div(double a) { return 1.0 / a; }
+__device__ __forceinline__ double2 pivot_div(double2 a) {
+    const int hx = __double2hiint(a.x) & 0x7fffffff, hy = __double2hiint(a.y) & 0x7fffffff;
+    const int e = (max(hx, hy) >> 20) - 1023;
+    if (e < -1000 || e > 1000) return t_inv(a);
+    const double s = pow2(-e), x = a.x * s, y = a.y * s;
+    const double r = (1.0 / fma(x, x, y * y)) * s;
+    return mk(x * r, -y * r);
+}
+
 // |x| as ordered bits: compares magnitudes without an FP64 comparison
 __device__ __forceinline__ unsigned long long abs_bits(double x) {
     return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;

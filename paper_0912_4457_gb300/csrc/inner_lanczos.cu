@@ -88,17 +88,6 @@ __device__ __forceinline__ void warp_total2(double2& a, double2& b) {
     b = mk(__shfl_sync(kFull, s, 16), __shfl_sync(kFull, s, 24));
 }
 
-// 1/a for the pivots: real by division; complex as conj(a) / |a|^2 with a
-// scaled by a power of two (exact) so that |a|^2 neither over- nor underflows
-__device__ __forceinline__ double pivot_inv(double a) { return 1.0 / a; }
-__device__ __forceinline__ double2 pivot_inv(double2 a) {
-    const int hx = __double2hiint(a.x) & 0x7fffffff, hy = __double2hiint(a.y) & 0x7fffffff;
-    const int e = min(max((max(hx, hy) >> 20) - 1023, -1000), 1000);
-    const double s = pow2(-e), x = a.x * s, y = a.y * s;
-    const double r = (1.0 / fma(x, x, y * y)) * s;
-    return mk(x * r, -y * r);
-}
-
 // Tridiagonal LU with partial pivoting, LAPACK gttrf semantics (rows i and
 // i + 1 are interchanged when |d_i| < |dl_i|, |.| = |re| + |im| for complex), by
 // one warp: all lanes run the recurrence, lane t keeps row c0 + t of each chunk
@@ -120,7 +109,7 @@ __device__ int gttrf_warp(int n, const double2* al, const double2* be, const dou
         bB[lane] = b;
         bA[lane] = row < n - 1 ? t_from(al[row + 1], T()) : t_zero(T());
         bG[lane] = row < n - 2 ? t_from(ga[row + 1], T()) : t_zero(T());
-        bI[lane] = t_iszero(b) ? t_zero(T()) : pivot_inv(b);
+        bI[lane] = t_iszero(b) ? t_zero(T()) : pivot_div(b);
         __syncwarp();
         T o_dl = t_zero(T()), o_di = t_zero(T()), o_du = t_zero(T()), o_du2 = t_zero(T());
         int o_pv = 0;
@@ -131,7 +120,7 @@ __device__ int gttrf_warp(int n, const double2* al, const double2* be, const dou
             const bool keep = lastrow || t_abs1(d) >= t_abs1(Bt);
             T fact, pd, pu, pu2, inv;
             if (keep) {
-                inv = zero ? t_zero(T()) : pivot_inv(d);
+                inv = zero ? t_zero(T()) : pivot_div(d);
                 fact = zero ? Bt : t_mul(Bt, inv);   // d = 0 only with a zero subdiagonal
                 pd = d;
                 pu = u;

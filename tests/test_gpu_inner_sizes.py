@@ -74,3 +74,16 @@ def test_inner_sizes(ell, herm):
 @pytest.mark.parametrize("herm", [True, False])
 def test_largest_inner_size(herm):
     check(2, 300, 256, herm, 1.3, seed=9)
+
+
+@pytest.mark.parametrize("herm", [True, False])
+@pytest.mark.parametrize("e", [-900, -200, 300, 900])
+def test_power_of_two_scale(e, herm):
+    """c depends on p H_k alone: H_k scaled by 2^e with p scaled by 2^-e gives the same bits."""
+    al, be, ga = ritz(2, 96, herm, 11)
+    ctx = Context((2, 2, 2, 2))
+    ref, _, _ = ctx.inner_sign(al, be, ga, 24, p=1.25, hermitian=herm)
+    s = 2.0 ** e
+    got, _, _ = ctx.inner_sign(al * s, be * s, ga * s, 24, p=1.25 / s, hermitian=herm)
+    ctx.close()
+    np.testing.assert_array_equal(got, ref)
