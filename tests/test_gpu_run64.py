@@ -14,7 +14,7 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
 from paper_0912_4457_gb300.nksign import (  # noqa: E402
-    NK_ASYNC, NK_DOUBLE_PASS, NK_EBREAKDOWN, NK_EINVAL, NK_ETIMEOUT, NK_FP64, NK_NO_GRAPH, NK_OK, NK_PROFILE,
+    NK_ASYNC, NK_DOUBLE_PASS, NK_EBREAKDOWN, NK_EINVAL, NK_ETIMEOUT, NK_FP64, NK_MIXED, NK_NO_GRAPH, NK_OK, NK_PROFILE,
     Context, NkError,
 )
 
@@ -197,3 +197,43 @@ def test_autotune_times_the_launch_of_all_steps(tmp_path):
     for c in (ctx, other):
         assert c.sign_apply(b, k, 16)[1]["launches"] == st0["launches"]
         c.close()
+
+
+@pytest.mark.parametrize("dims,n,mu", [((6, 6, 6, 6), 12, 0.3),     # several rounds of both halves, 12 CTAs a source
+                                       ((8, 8, 8, 8), 8, 0.0), ((8, 8, 8, 8), 4, 0.3),   # 32768 sites x vectors: one launch
+                                       ((8, 8, 8, 8), 9, 0.0), ((8, 8, 8, 8), 5, 0.3)])  # beyond: the step kernels
+def test_loops_and_both_sides_of_the_dispatch(dims, n, mu):
+    """The first 12 steps against the oracle (1e-11, as in test_gpu_parity), first and last source."""
+    k = 12
+    ctx, U = make_ctx(dims, mu)
+    b = inputs.gaussian_sources(dims, 78, n_rhs=n)
+    _, st, _ = ctx.sign_apply(b, k, 8, p=1.0)
+    assert (st["launches"] < 2 * k) == (b.shape[1] // 12 * n * (2 if mu else 1) <= 32768)
+    al, be, ga, _ = ctx.outer_lanczos_dev(torch.from_numpy(b).cuda(), n, k)
+    A, Ad, herm = nested.operator(U, dims, mu, M_W)
+    for i in (0, n - 1):
+        ref = nested.outer_basis(A, Ad, b[i], k, herm)
+        assert rel(al[i], ref.alpha) < 1e-11
+        assert rel(be[i, : k - 1], ref.beta[: k - 1]) < 1e-11
+        assert rel(ga[i, : k - 1], ref.gamma[: k - 1]) < 1e-11
+    ctx.close()
+
+
+@pytest.mark.parametrize("mu", [0.0, 0.2])
+@pytest.mark.parametrize("shape,mixed", [(None, False), ((64, 0, 1), False), ((256, 1, 3), False), (None, True)])
+def test_second_pass_regenerates_the_same_bits(mu, shape, mixed):
+    """A double-pass solve adds c'_j q_j column by column as the lift of the stored basis does, so with
+    a bit-identical second pass the results are equal."""
+    dims, n, k = (5, 4, 3, 6), 3, 256
+    ctx, _ = make_ctx(dims, mu)
+    flags = NK_MIXED if mixed else NK_FP64
+    if shape:
+        s = list(ctx.get_launch(n, flags))
+        s[0], s[1], s[5] = shape
+        s[2] += 1
+        ctx.set_launch(n, flags, *s)
+    b = inputs.gaussian_sources(dims, 79, n_rhs=n)
+    y1, _, _ = ctx.sign_apply(b, k, 64, p=1.0, flags=flags)
+    y2, _, _ = ctx.sign_apply(b, k, 64, p=1.0, flags=flags | NK_DOUBLE_PASS)
+    np.testing.assert_array_equal(y1, y2)
+    ctx.close()
