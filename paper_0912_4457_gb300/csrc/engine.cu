@@ -57,7 +57,7 @@ struct nk_ctx {
     long N;
     int antiperiodic;
     int device;
-    int sms = 152;         // multiprocessors
+    int sms;               // multiprocessors
     bool coop = false;     // the device takes cooperative launches
     unsigned long long wait_ns = 1000000000ull;   // limit of a device-side wait (nk_set_wait_limit)
     double mu = 0.0, m_w = 0.0;
@@ -298,20 +298,13 @@ Layout carve(char* base, const Geom& g, int n_rhs, int k, int ell, bool two_side
     return L;
 }
 
-int blocks_per_rhs(long N, int n_rhs) {
-    // fixed per shape and device (deterministic reductions)
-    int dev = 0, sms = 152;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
-    return nk::step_blocks(N, n_rhs, sms);
-}
-
-// The default launch shape: 128 threads per CTA, vector-fastest grid, blocks_per_rhs.
+// The default launch shape: 128 threads per CTA, vector-fastest grid, one wave of step
+// CTAs over the RHS; fixed per shape and device (deterministic reductions).
 nk_launch default_launch(const nk_ctx* c, int n_rhs) {
     nk_launch d;
     d.stencil_threads = 128;
     d.stencil_order = 0;
-    d.step2_blocks = blocks_per_rhs(c->N, n_rhs);
+    d.step2_blocks = nk::step_blocks(c->N, n_rhs);
     d.early_threads = 128;
     d.early_order = 0;
     d.stencil_split = 1;
@@ -1055,8 +1048,8 @@ int nk_create_lattice(const int dims[4], int bc_t_antiperiodic, nk_ctx** out) {
         delete c;
         return NK_ECUDA;
     }
+    c->sms = nk::device_sms();
     int attr = 0;
-    if (cudaDeviceGetAttribute(&attr, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess && attr > 0) c->sms = attr;
     if (cudaDeviceGetAttribute(&attr, cudaDevAttrCooperativeLaunch, c->device) == cudaSuccess) c->coop = attr != 0;
     nk::init_kernel_attributes();
     cudaGetLastError();
@@ -1863,7 +1856,7 @@ int nk_autotune(nk_ctx* c, int n_rhs, unsigned flags, const char* cache_path, nk
     best.early_order = 0;
     best.stencil_split = 1;
     best.early_split = 1;
-    const int b0 = blocks_per_rhs(c->N, n_rhs);
+    const int b0 = nk::step_blocks(c->N, n_rhs);
     best.step2_blocks = b0;
     // each kernel of an outer step is tuned on its own
     auto fail_out = [&](int code) { cudaStreamDestroy(st); return code; };

@@ -553,13 +553,19 @@ void launch_outer_step1(const Outer& o, int j, bool s64, cudaStream_t st) {
 #undef NK_STEP1
 }
 
+int device_sms() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0 ? sms : 152;
+}
+
 // Default CTAs per RHS of the step kernels (and of the norm): one item per
 // thread, but no more than one wave of the chip over all RHS (a CTA's block sum
 // costs the FP64 pipe as much as an item).  The wave is filled: 63 CTAs a
 // source for 12 against 60 took a step at 10^4 from 105.1 to 102.9 us, at 8^4
 // from 27.6 to 27.0.
-int step_blocks(long N, int n_rhs, int sms) {
-    const long need = (N / 2 + kStepThreads - 1) / kStepThreads, cap = (long)sms * kStepCtasPerSm / n_rhs;
+int step_blocks(long N, int n_rhs) {
+    const long need = (N / 2 + kStepThreads - 1) / kStepThreads, cap = (long)device_sms() * kStepCtasPerSm / n_rhs;
     return (int)std::max(1L, std::min(need, cap));
 }
 

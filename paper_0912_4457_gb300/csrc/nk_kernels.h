@@ -239,7 +239,8 @@ bool split_step(int precision, const Outer& o, int j);
 void launch_stencil_step(int precision, const void* U, const Geom& g, const Outer& o, int j, double kappa,
                          double mu, cudaStream_t st);
 void launch_outer_step1(const Outer& o, int j, bool s64, cudaStream_t st);
-int step_blocks(long N, int n_rhs, int sms);   // default CTAs per RHS of the step kernels
+int step_blocks(long N, int n_rhs);   // default CTAs per RHS of the step kernels
+int device_sms();                     // multiprocessors of the current device
 void launch_stencil32_step1(const void* U32, const Geom& g, const Outer& o, int j, double kappa, double mu,
                             cudaStream_t st);
 int dslash_step1_blocks(const Geom& g, int threads);

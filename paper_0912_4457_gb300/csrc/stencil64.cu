@@ -595,7 +595,7 @@ void launch_s64_step1(const double2* U, const Geom& g, const Outer& o, int j, do
 int stencil64_blocks(const Geom& g, int threads, int nvec) {
     const int S = threads / 16;
     const int nsb = (g.V + S - 1) / S;
-    const int wave = 152 * (kS64Sites / S) / nvec;
+    const int wave = device_sms() * (kS64Sites / S) / nvec;
     return nsb < wave ? nsb : (wave > 0 ? wave : 1);
 }
 
