@@ -368,8 +368,11 @@ static cudaError_t launch_rhi_t(const Inner& in, cudaStream_t st) {
     int C = in.ell >= 64 ? 8 : (in.ell >= 16 ? 4 : 1);
     if (in.ell >= 96 && in.n_rhs <= 8) {
         // 16 CTAs (a size the device may not offer) halve the update of a large
-        // matrix: one RHS, two-sided, k = 1536, l = 256, the inner part 30.7 -> 20.1 ms,
-        // k = 1024, l = 128 7.5 -> 6.7; twelve RHS no longer fit the chip at once (7.5 -> 7.7)
+        // matrix, while the chip holds the clusters of all RHS at once.  The inner part with
+        // 8 -> 16 CTAs, ms: two-sided, k = 1024, l = 128: 1 RHS 7.62 -> 6.74, 7 7.66 -> 6.77,
+        // 8 7.66 -> 7.57, 10 7.66 -> 7.79; k = 512, l = 256: 1 27.6 -> 17.0, 8 31.6 -> 26.8 (and
+        // 12 43.2 -> 35.2); l = 96: 3.96 -> 3.97.  Hermitian: l = 256 1 12.7 -> 7.9, 8 14.5 -> 10.6;
+        // l = 128 1 3.64 -> 3.62, 8 3.70 -> 3.82; l = 96 1 2.20 -> 2.30
         shape(16);
         int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, k_rhi<T>, &cfg) == cudaSuccess && n > 0) C = 16;

@@ -10,8 +10,9 @@
 // and a third of the FP64 operations per vector element (FP64 is the scarce
 // unit on GB300).  In exact arithmetic this is the paper's recurrence; the
 // coefficients alpha, beta, gamma are the entries of H_k as App. A / B define
-// them.  One outer step j is two kernels:
-//   dslash_step1 (dslash.cu): s = A q_j / n_j (and t = A^dag p_j / m_j), then
+// them.  One outer step j is:
+//   step1 (fused with the FP64 stencil in stencil64.cu; k_step1 below after a multi-RHS
+//          stencil): s = A q_j / n_j (and t = A^dag p_j / m_j), then
 //          r = s - (c_{j-1}/n_{j-1}) q_{j-1},  l = t - (beta^*_{j-1}/m_{j-1}) p_{j-1}
 //          H(j,j) = v_j^dag r (= w_j^dag r two-sided), stored r -> q_{j+1}, l -> p_{j+1};
 //   step2: r <- r - (H(j,j)/n_j) q_j,  l <- l - (H(j,j)^*/m_j) p_j,
@@ -26,8 +27,9 @@
 // Reductions are deterministic: a fixed grid, a fixed per-thread order,
 // warp-shuffle and shared-memory block sums, per-block partials and a final
 // fixed-order sum in the last block to finish (integer ticket, no
-// floating-point atomics).  The same launch configuration therefore
-// regenerates bit-identical coefficients, which the double-pass mode relies on.
+// floating-point atomics), and the FP64 arithmetic that the kernels of the two passes
+// share is written in explicit fused multiply-adds.  The same launch configuration therefore regenerates
+// bit-identical coefficients and vectors, which the double-pass mode relies on.
 #include <algorithm>
 
 #include "nk_common.cuh"
@@ -163,7 +165,7 @@ __device__ __forceinline__ void step2_finish(const Outer& o, int rhs, int j, dou
 // full): an outer step of 12 sources at 10^4, mu = 0.2, two-float stencil,
 // 220 -> 192 us; 8^4, mu = 0, FP32 stencil, 41 -> 27; one source, FP64, at 4^4,
 // mu = 0.1, 21 -> 16, at 10^4 65 -> 58 (both with the shorter tail).  20 warps
-// per SM at 102 registers: 8, 6, 4 or 3 CTAs per SM measured 201, 200, 193
+// per SM (5 CTAs, 56 to 96 registers): 8, 6, 4 or 3 CTAs per SM measured 201, 200, 193
 // and 194 us in the first case (64 registers spill).
 constexpr int kStepThreads = 128;   // at least 3 warps: the finishing block of step 1 uses warps 0 to 2
 constexpr int kStepCtasPerSm = 5;

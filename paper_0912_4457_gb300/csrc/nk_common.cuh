@@ -17,7 +17,7 @@ namespace nk {
 // read by ordinary loads (no __ldg, no const __restrict__ pointer, which would
 // also let the compiler move a load above the wait).  A caller that applies the operator again
 // and again then has no launch gap and a filled last wave: FP32 stencil, 24 vectors at 10^4,
-// 22.5 -> 19.0 us.  Behind a kernel without pdl_trigger it is an ordinary launch.
+// 24.7 -> 21.9 us a call (one call alone, and the kernel inside a solve, take what they did).  Behind a kernel without pdl_trigger it is an ordinary launch.
 // Inside an outer recurrence the kernels are launched plainly: there the
 // waiting CTAs took slots unevenly (an outer step of 12 sources at 8^4 27.5 -> 30.7 us,
 // 33 with an early trigger; 6^4, one source, 20.9 -> 22.6).
@@ -65,10 +65,6 @@ __host__ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 __device__ __forceinline__ double2 cmul_fma(double2 a, double2 b) {
     return mk(fma(a.x, b.x, -(a.y * b.y)), fma(a.x, b.y, a.y * b.x));
 }
-// conj(a) * b
-__host__ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {
-    return mk(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
 __host__ __device__ __forceinline__ double2 cconj(double2 a) { return mk(a.x, -a.y); }
 __host__ __device__ __forceinline__ double2 cscale(double2 a, double s) { return mk(a.x * s, a.y * s); }
 __host__ __device__ __forceinline__ double cabs1(double2 a) { return fabs(a.x) + fabs(a.y); }
@@ -84,15 +80,6 @@ __host__ __device__ __forceinline__ double2 cinv(double2 a) {
     }
 }
 __host__ __device__ __forceinline__ double2 cdiv(double2 a, double2 b) { return cmul(a, cinv(b)); }
-// principal square root (cut on the negative real axis)
-__host__ __device__ __forceinline__ double2 csqrt_principal(double2 z) {
-    double r = hypot(z.x, z.y);
-    if (r == 0.0) return mk(0.0, 0.0);
-    double t = sqrt(0.5 * (r + fabs(z.x)));
-    if (z.x >= 0.0) return mk(t, z.y / (2.0 * t));
-    return mk(fabs(z.y) / (2.0 * t), z.y >= 0.0 ? t : -t);
-}
-
 // sqrt(x) and 1 / sqrt(x) of a positive finite x from one reciprocal square
 // root (410 clocks; a square root takes 650, a division 620): y = rsqrt(x),
 // then one Newton correction of x y.
@@ -133,12 +120,6 @@ __host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return mk(
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return mk(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-__host__ __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
-    return mk(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
-
-__device__ __forceinline__ double2 to_d2(double2 a) { return a; }
-__device__ __forceinline__ double2 to_d2(float2 a) { return mk((double)a.x, (double)a.y); }
 
 // Warp sum of a double2 in a fixed butterfly order (deterministic).
 __device__ __forceinline__ double2 warp_sum(double2 v) {

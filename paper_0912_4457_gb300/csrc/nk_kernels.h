@@ -109,10 +109,11 @@ int stencil32_blocks(const Geom& g, int nv);
 struct Outer {
     long N;          // vector length (12 V complex)
     int n_rhs, k, nblk, npart;
-    int st_threads;  // fused stencil: sites (threads) per CTA, 64 / 128 / 256
+    int st_threads;  // fused FP64 stencil: threads per CTA at split 1, 64 / 128 / 256; 16 per site
     int st_order;    // fused stencil grid: 0 vector-fastest (link reuse in L2), 1 site-block-fastest
-    int st_split;    // fused stencil: threads per site, 1 or 3 (one colour each)
-    int st_threads_df, st_order_df, st_split_df;   // the same for the two-float stencil steps
+    int st_split;    // fused FP64 stencil: 1, or 3 times the threads (one colour row of a hop's product each)
+    // two-float stencil of the two-float recurrence: sites per CTA, grid order, threads per site
+    int st_threads_df, st_order_df, st_split_df;
     int two_sided;
     int q_ring;      // 0: Q holds all k vectors (+1 scratch) [rhs][k+1][N]; 1: ring [rhs][3][N] (double pass)
     int qcols;       // vectors per RHS in Q: k + 1 or 3
@@ -226,14 +227,14 @@ constexpr int kCopyNone = 0, kCopy32 = 1, kCopyDF = 2;
 void launch_outer_init(const Outer& o, int copy_mode, cudaStream_t st, bool keep_status = false);
 // Stencil + first half of step j; precision 32 (FP32, the multi-RHS stencil
 // of stencil32.cu, then the FP64 step-1 kernel of lanczos.cu; fused with a
-// two-float epilogue in the two-float recurrence), 48 (two-float) or 64
-// (FP64) (dslash.cu).  Returns the number of kernels launched.
+// two-float epilogue in the two-float recurrence), 48 (two-float, dslash.cu) or 64
+// (FP64, stencil64.cu).  Returns the number of kernels launched.
 int launch_dslash_step1(int precision, const void* U, const Geom& g, const Outer& o, int j,
                         double kappa, double mu, cudaStream_t st);
 // The FP32 and two-float steps of an FP64 recurrence (precision 32 or 48
 // before o.ring_from, with o.s32 / o.s64): the multi-RHS stencil, which leaves
 // s = (A q_j)/n_j and t = (A^dag p_j)/m_j in o.s32 (FP32) or o.s64 (FP64 from
-// the two-float stencil) (dslash.cu), then the first half of outer step j in
+// the two-float stencil, stencil_df.cu), then the first half of outer step j in
 // FP64 (lanczos.cu).
 bool split_step(int precision, const Outer& o, int j);
 void launch_stencil_step(int precision, const void* U, const Geom& g, const Outer& o, int j, double kappa,

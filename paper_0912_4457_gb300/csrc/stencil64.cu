@@ -15,8 +15,8 @@
 // component each.  No FP64 operation is done twice, the sums run over the
 // hops in the order 0..7, and a CTA of S sites (S = 4, 8 or 16) is short
 // enough to fill the chip from 4^4 on.  Measured, outer step (this kernel and
-// step 2) of one source: 4^4, mu = 0 51.5 -> 16.8 us; 6^4, mu = 0.1 58 -> 28;
-// 10^4, mu = 0.2 95 -> 65; 12 sources at 10^4, mu = 0: 235.  The stencil alone
+// step 2) of one source: 4^4, mu = 0 51.5 -> 16.8 us (13.5 with the present step 2); 6^4,
+// mu = 0.1 58 -> 28 (21); 10^4, mu = 0.2 95 -> 65 (58).  The stencil alone
 // on 12 vectors at 16^3 x 32, 2.44 -> 2.34 ms (its FP64 floor is 2.25), and
 // straight from and to the ABI layout, without the two conversion passes
 // (0.2 ms).  Profile at 10^4: FP64 pipe 82% busy while an SM has work.
