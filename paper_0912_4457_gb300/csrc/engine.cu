@@ -420,8 +420,8 @@ int copy_mode_for(const Schedule& s, int j) {
 // Whether the FP64 steps of this recurrence run as one cooperative launch
 // (k_run64): a small batch -- up to kRunSiteVecs sites times vectors, beyond which
 // the FP64 pipe hides the step kernels' launches and tails and their finer grain
-// wins (measured us per step, run against step kernels: 6^4 x 2 vectors 17.4 / 21.0,
-// 10^4 x 2 52.2 / 58.1, 6^4 x 24 74.5 / 79.4, 8^4 x 8 74.8 / 79.6, 8^4 x 12 114.7 / 112.4) -- with
+// wins (measured us per step, run against step kernels: 6^4 x 2 vectors 17.1 / 21.0,
+// 10^4 x 2 52.7 / 58.3, 6^4 x 24 75.1 / 79.5, 8^4 x 8 75.2 / 79.3, 8^4 x 12 114.7 / 112.4) -- with
 // no launch shape of its own (a set or tuned shape other than the default names the
 // kernels of a step).
 // A cooperative launch keeps its SMs for the whole run, so a solve beside others

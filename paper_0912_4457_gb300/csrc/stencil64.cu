@@ -295,18 +295,19 @@ __global__ void __launch_bounds__(16 * S * SPLIT, SPLIT == 1 ? kS64Sites / S : 1
 // launch, at most one CTA per SM and RHS share, and per step two grid barriers
 // of the RHS's CTAs; after each every CTA adds the partial sums and forms the
 // scalars for itself (the same values in the same order everywhere), so nothing
-// waits for a second hop through memory.  128 threads work on eight sites as in
+// waits for a second hop through memory.  128 (64) threads work on eight (four) sites as in
 // k_stencil64_step1 (group of the CTA with its own named barrier), then all on
 // (component pair, site) items as in k_step2.  Vectors written by the launch are
 // read past L1.
 // The barriers' waits are bounded: a CTA whose wait runs out marks its RHS
 // kStatusTimeout and leaves; the others' waits then run out too.
 // Measured, us per step against the step kernels: 4^4, mu = 0 13.5 -> 9.7; 6^4, mu = 0.1
-// 21.0 -> 17.4; 10^4, mu = 0.2 58.1 -> 52.2 (all one source).  Registers capped for two
+// 21.0 -> 17.1; 10^4, mu = 0.2 58.1 -> 52.7 (all one source).  Registers capped for two
 // CTAs per SM cost 4% at 10^4 (62.7 -> 65.2 ms a solve of k = 1024); 256 threads per CTA 18.5
-// at 6^4, 55.5 at 10^4.  Groups of 64 threads on four sites leave a quarter of the lanes
-// idle in the sum over the hops: 54 at 10^4.
-constexpr int kRunSites = 8, kRunGroup = 16 * kRunSites, kRunThreads = 384, kRunGroups = kRunThreads / kRunGroup;
+// at 6^4, 55.5 at 10^4.
+constexpr int kRunThreads = 384;
+template <int S> constexpr int kRunGroup = 16 * S;                            // threads of a group on S sites
+template <int S> constexpr int kRunGroups = kRunThreads / kRunGroup<S>;   // groups of a CTA
 
 __device__ __forceinline__ unsigned long long run_ns() {
     unsigned long long t;
@@ -356,24 +357,24 @@ __device__ __forceinline__ double2 run_total(const double2* part, int ncta) {
 
 // First half of step j, stencil and step 1 on this CTA's share of the site blocks;
 // returns the thread's part of H(j,j).
-template <bool TS, bool PASS2>
+template <bool TS, bool PASS2, int S>
 __device__ __forceinline__ double2 run_half1(const double2* __restrict__ U, const Geom& g, const Outer& o, int rhs, int j,
-                                             int cta, int ncta, const double2* sc, double2 (*sx)[48 * kRunSites],
+                                             int cta, int ncta, const double2* sc, double2 (*sx)[48 * S],
                                              double kappa, double emu, double emu_inv) {
-    const int tid = threadIdx.x, grp = tid / kRunGroup, gt = tid % kRunGroup;
-    const int V = g.V, nsb = (V + kRunSites - 1) / kRunSites;
+    const int tid = threadIdx.x, grp = tid / kRunGroup<S>, gt = tid % kRunGroup<S>;
+    const int V = g.V, nsb = (V + S - 1) / S;
     const int jp = j > 0 ? j - 1 : j;
     const bool left = TS && j < o.k - 1;
     // the warp that idles in the sum differs from group to group (FP64 pipes, as in k_stencil64)
-    const int t2 = (gt + 32 * (grp & 3)) % kRunGroup;
-    const int s = t2 % kRunSites, comp = t2 / kRunSites, sp = comp / 3, a = comp % 3;
+    const int t2 = (gt + 32 * (grp & 3)) % kRunGroup<S>;
+    const int s = t2 % S, comp = t2 / S, sp = comp / 3, a = comp % 3;
     const unsigned sg = sp < 2 ? 0u : 0x80000000u;
     double2 dot = make_double2(0.0, 0.0);
-    for (int u = cta + ncta * grp; u < (left ? 2 : 1) * nsb; u += ncta * kRunGroups) {
+    for (int u = cta + ncta * grp; u < (left ? 2 : 1) * nsb; u += ncta * kRunGroups<S>) {
         const int side = u >= nsb ? 1 : 0, b = u - side * nsb;
         const double2* in = side ? outer_p(o, rhs, j) : outer_q(o, rhs, j);
-        s64_hops<kRunSites, 1, false, true>(U, in, g, b * kRunSites, sx[grp], gt);
-        const int site = b * kRunSites + s;
+        s64_hops<S, 1, false, true>(U, in, g, b * S, sx[grp], gt);
+        const int site = b * S + s;
         const bool live = comp < 12 && site < V;
         const size_t idx = (size_t)comp * V + site;
         double2 p = make_double2(0.0, 0.0), pv = p, d = p;
@@ -382,11 +383,11 @@ __device__ __forceinline__ double2 run_half1(const double2* __restrict__ U, cons
             pv = __ldcg((side ? outer_p(o, rhs, jp) : outer_q(o, rhs, jp)) + idx);
             if (side == 0) d = __ldcg((TS ? outer_p(o, rhs, j) : outer_q(o, rhs, j)) + idx);
         }
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kRunGroup) : "memory");
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kRunGroup<S>) : "memory");
         if (live) {
             double wp, wm;
             t_weights(g, site, side, emu, emu_inv, wp, wm);
-            const double2 acc = s64_sum<kRunSites>(sx[grp], s, sp, a, wp, wm);
+            const double2 acc = s64_sum<S>(sx[grp], s, sp, a, wp, wm);
             const double2 v = make_double2(flip(fma(-kappa, acc.x, p.x), sg), flip(fma(-kappa, acc.y, p.y), sg));
             const double2 scl = sc[side ? kScM : kScN], c1 = sc[side ? kScC1L : kScC1];
             double2 rr;
@@ -406,7 +407,7 @@ __device__ __forceinline__ double2 run_half1(const double2* __restrict__ U, cons
                 }
             }
         }
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kRunGroup) : "memory");   // sx is rewritten
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(kRunGroup<S>) : "memory");   // sx is rewritten
     }
     return dot;
 }
@@ -483,11 +484,11 @@ __device__ __forceinline__ void run_beta(const Outer& o, int rhs, int j, bool wr
     }
 }
 
-template <bool TS, bool PASS2>
+template <bool TS, bool PASS2, int S>
 __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict__ U, Geom g, Outer o, int j_lo, int j_hi,
                                                           double kappa, double emu, double emu_inv,
                                                           unsigned long long wait_ns) {
-    __shared__ double2 sx[kRunGroups][48 * kRunSites];
+    __shared__ double2 sx[kRunGroups<S>][48 * S];
     __shared__ double2 sh[33];
     __shared__ double2 sc[kScalars];
     __shared__ bool ok_sh;   // a barrier's outcome (written inside run_barrier only)
@@ -502,7 +503,7 @@ __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict
     if (tid < kScalars) sc[tid] = o.sc[(size_t)rhs * kScalars + tid];
     __syncthreads();
     for (int j = j_lo; j < j_hi; ++j) {
-        const double2 dot = block_sum(run_half1<TS, PASS2>(U, g, o, rhs, j, cta, ncta, sc, sx, kappa, emu, emu_inv), sh);
+        const double2 dot = block_sum(run_half1<TS, PASS2, S>(U, g, o, rhs, j, cta, ncta, sc, sx, kappa, emu, emu_inv), sh);
         if (tid == 0) part1[cta] = dot;
         target += (unsigned)ncta;
         if (!run_barrier(counter, target, wait_ns, &ok_sh)) {
@@ -531,15 +532,15 @@ __global__ void __launch_bounds__(kRunThreads) k_run64(const double2* __restrict
 // step to the last, and a second solve waits for a place; these come and go.  HALF 0
 // is the first half of step j, HALF 1 the second; the CTA that finishes last forms
 // the scalars, for all (formed by every CTA, as in k_run64, they would take an SM's
-// FP64 pipe from the other solves: 10.4 against 8.0 below).  us per step of one of 16
+// FP64 pipe from the other solves: 10.4 against 8.4 below).  us per step of one of 16
 // solves in flight, all steps in one launch -> a launch per half step: 4^4, mu = 0.1 3.4 -> 3.1;
-// 6^4, mu = 0.1 11.2 -> 8.0; 8^4 21.8 -> 18.3; 10^4, mu = 0.2 46.2 -> 40.2 (k_run64 there with
-// registers for three CTAs per SM; one per SM 14 at 6^4); of one alone 12.4 -> 17.3, 17.4 -> 22.5,
-// 27.6 -> 33.9, 52.2 -> 59.2.
-template <bool TS, bool PASS2, int HALF>
+// 6^4, mu = 0.1 11.2 -> 8.4; 8^4 21.8 -> 18.3; 10^4, mu = 0.2 46.2 -> 40.2 (k_run64 there with
+// registers for three CTAs per SM; one per SM 14 at 6^4); of one alone 12.7 -> 17.3, 17.1 -> 22.6,
+// 27.9 -> 33.7, 52.7 -> 59.4.
+template <bool TS, bool PASS2, int HALF, int S>
 __global__ void __launch_bounds__(kRunThreads, HALF == 0 ? 2 : 3) k_run64_half(const double2* __restrict__ U, Geom g, Outer o, int j,
                                                                double kappa, double emu, double emu_inv) {
-    __shared__ double2 sx[HALF == 0 ? kRunGroups : 1][48 * kRunSites];
+    __shared__ double2 sx[HALF == 0 ? kRunGroups<S> : 1][48 * S];
     __shared__ double2 sh[33];
     __shared__ double2 sc[kScalars];
     __shared__ bool go_sh;
@@ -550,7 +551,7 @@ __global__ void __launch_bounds__(kRunThreads, HALF == 0 ? 2 : 3) k_run64_half(c
     double2* home = o.sc + (size_t)rhs * kScalars;
     if (tid < kScalars) sc[tid] = home[tid];
     __syncthreads();
-    const double2 mine = HALF == 0 ? run_half1<TS, PASS2>(U, g, o, rhs, j, cta, ncta, sc, sx, kappa, emu, emu_inv)
+    const double2 mine = HALF == 0 ? run_half1<TS, PASS2, S>(U, g, o, rhs, j, cta, ncta, sc, sx, kappa, emu, emu_inv)
                                    : run_half2<TS>(o, rhs, j, cta, ncta, sc);
     if (!finish_partial(block_sum(mine, sh), part, o.counters + rhs, cta, ncta)) return;
     __threadfence();
@@ -563,11 +564,18 @@ __global__ void __launch_bounds__(kRunThreads, HALF == 0 ? 2 : 3) k_run64_half(c
     if (tid == 0) o.counters[rhs] = 0u;
 }
 
-// CTAs per RHS of a run: one per SM over the RHS, fewer where there are not so many
-// units of work.
-int run_ctas(const Geom& g, const Outer& o, int sms) {
-    const int units = (o.two_sided ? 2 : 1) * ((g.V + kRunSites - 1) / kRunSites);
-    return std::max(1, std::min(sms / o.n_rhs, units));
+// Sites of a group and CTAs per RHS of a run.  One CTA per SM over the RHS, fewer where
+// there are not so many blocks of eight sites.  Eight sites per group waste no lanes
+// in the sum over the hops; with one to three blocks of eight per CTA, groups of four
+// share them out more evenly (us per step, four / eight: 6^4 1 vector 11.5 / 12.0, 2 vectors
+// 17.1 / 17.7, 5x4x3x6 x 2 x 2 13.8 / 14.4; one block or less: 4^4 1 9.9 / 9.6, 2 13.5 / 12.7; more
+// than three: 8^4 1 17.9 / 17.3, 2 29.5 / 28.0, 10^4 2 54.4 / 52.7).
+struct RunShape {
+    int sites, ctas;
+};
+RunShape run_shape(const Geom& g, const Outer& o, int sms) {
+    const int most = std::max(1, sms / o.n_rhs), blocks = (o.two_sided ? 2 : 1) * ((g.V + 7) / 8);
+    return {blocks > most && blocks <= 3 * most ? 4 : 8, std::min(most, blocks)};
 }
 
 template <int S, int SPLIT>
@@ -618,7 +626,8 @@ bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int 
                   unsigned long long wait_ns, cudaStream_t st) {
     cudaMemsetAsync(o.run_bar, 0, sizeof(unsigned) * o.n_rhs, st);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(run_ctas(g, o, sms) * o.n_rhs));
+    const RunShape sh = run_shape(g, o, sms);
+    cfg.gridDim = dim3((unsigned)(sh.ctas * o.n_rhs));
     cfg.blockDim = dim3(kRunThreads);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -629,27 +638,33 @@ bool launch_run64(const void* U64, const Geom& g, const Outer& o, int j_lo, int 
     const double2* U = (const double2*)U64;
     const double ep = exp(mu), em = exp(-mu);
     const bool pass2 = o.y != nullptr;
-    cudaError_t e;
-    if (o.two_sided)
-        e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<true, true>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns)
-                  : cudaLaunchKernelEx(&cfg, k_run64<true, false>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns);
-    else
-        e = pass2 ? cudaLaunchKernelEx(&cfg, k_run64<false, true>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns)
-                  : cudaLaunchKernelEx(&cfg, k_run64<false, false>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns);
+#define NK_RUN(TS_, P2_)                                                                                            \
+    (sh.sites == 4 ? cudaLaunchKernelEx(&cfg, k_run64<TS_, P2_, 4>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns) \
+                   : cudaLaunchKernelEx(&cfg, k_run64<TS_, P2_, 8>, U, g, o, j_lo, j_hi, kappa, ep, em, wait_ns))
+    const cudaError_t e = o.two_sided ? (pass2 ? NK_RUN(true, true) : NK_RUN(true, false))
+                                      : (pass2 ? NK_RUN(false, true) : NK_RUN(false, false));
+#undef NK_RUN
     return e == cudaSuccess;
 }
 
 void launch_run64_half(const void* U64, const Geom& g, const Outer& o, int half, int j, double kappa, double mu, int sms,
                        cudaStream_t st) {
-    const unsigned grid = (unsigned)(run_ctas(g, o, sms) * o.n_rhs);
+    const RunShape sh = run_shape(g, o, sms);
+    const unsigned grid = (unsigned)(sh.ctas * o.n_rhs);
     const double ep = exp(mu), em = exp(-mu);
-#define NK_HALF(TS_, P2_, H_) k_run64_half<TS_, P2_, H_><<<grid, kRunThreads, 0, st>>>((const double2*)U64, g, o, j, kappa, ep, em)
+#define NK_HALF(TS_, P2_, H_, S_) k_run64_half<TS_, P2_, H_, S_><<<grid, kRunThreads, 0, st>>>((const double2*)U64, g, o, j, kappa, ep, em)
+#define NK_HALF0(TS_, P2_)                           \
+    do {                                              \
+        if (sh.sites == 4) NK_HALF(TS_, P2_, 0, 4);   \
+        else NK_HALF(TS_, P2_, 0, 8);                 \
+    } while (0)
     if (half == 0) {
-        if (o.two_sided) { if (o.y) NK_HALF(true, true, 0); else NK_HALF(true, false, 0); }
-        else { if (o.y) NK_HALF(false, true, 0); else NK_HALF(false, false, 0); }
-    } else {
-        if (o.two_sided) NK_HALF(true, false, 1); else NK_HALF(false, false, 1);
+        if (o.two_sided) { if (o.y) NK_HALF0(true, true); else NK_HALF0(true, false); }
+        else { if (o.y) NK_HALF0(false, true); else NK_HALF0(false, false); }
+    } else {   // (does not see the sites)
+        if (o.two_sided) NK_HALF(true, false, 1, 8); else NK_HALF(false, false, 1, 8);
     }
+#undef NK_HALF0
 #undef NK_HALF
 }
 
